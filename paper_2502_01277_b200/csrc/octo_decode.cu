@@ -3,7 +3,7 @@
 // HBM-bound scan.  For logit heads sigma <= 1 makes sigma(obj) > conf a necessary condition
 // for score = fl(sigma(obj) * sigma(cls)) > conf, so the scan reads only the obj value of
 // each 340-byte row (one DRAM sector) and fetches the whole row, 32 bytes at a time by a group
-// of eight lanes (four passing rows per warp in flight together), for the few anchors that pass.  Probability heads are read densely.  A passing row is
+// of eight lanes (four passing rows per warp in flight together), for the few anchors that pass.  Probability heads are read densely (decode_dense_kernel, where a 16-byte boundary allows it).  A passing row is
 // reduced by eight lanes (finite check, first-maximum class), scored in the fixed binary32
 // sequence and appended to the image's key list with one atomic; the key carries class,
 // inverted score bits and anchor, so later steps need nothing else from this kernel and the
@@ -292,6 +292,86 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
     }
 }
 
+// Rows layout, probabilities: nothing bounds a row's score before its class values are known, so the
+// head is read whole and the scan is bound by HBM.  A CTA takes kDenseRows consecutive rows, which are
+// one contiguous piece of memory: one bulk copy stages them (five CTAs of 85-value rows keep 218 KB per
+// SM in flight), then a thread reduces a row out of shared memory.  A row of an odd number of values is
+// read without bank conflicts as it stands (lane stride = row length); for the others the lanes start
+// at rotated positions.  us per launch on [n, 25200, 5 + C] against the row groups of decode_kernel:
+// C = 80, n = 1 10.8 (18.7), n = 4 18.8 (23.0), n = 32 70.1 (95.7: 274 MB at 3.9 instead of 2.9 TB/s);
+// C = 7, n = 8 10.7 (31.3); C = 20, n = 64 44.1 (108.0).  64 rows per CTA measure the same, 256 worse
+// (n = 32 82.7).
+constexpr int kDenseRows = 128;
+
+__global__ void __launch_bounds__(kDenseRows)
+decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, int key_stride,
+                    unsigned long long* __restrict__ keys, int* __restrict__ cand_count,
+                    unsigned int* __restrict__ status, int pdl) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ __align__(8) uint64_t bar;
+    pdl_enter(pdl);
+    const bool agnostic = (mode & 2) != 0;
+    const bool multi = (mode & 4) != 0;
+    const int img = blockIdx.y, t = threadIdx.x;
+    const int row_len = 5 + C;
+    const int a0 = blockIdx.x * kDenseRows;
+    const int rows = min(kDenseRows, A - a0);
+    const float* __restrict__ src = head + ((size_t)img * (size_t)A + (size_t)a0) * (size_t)row_len;
+    float* const s = reinterpret_cast<float*>(smem);
+    const int values = rows * row_len, bulk = values & ~3;  // the copy moves multiples of 16 bytes
+    if (t == 0) {
+        mbar_init(&bar, 1);
+        mbar_fence_init();
+        fence_proxy_async();
+        mbar_expect_tx(&bar, (uint32_t)bulk * 4u);
+        if (bulk) bulk_g2s(s, src, (uint32_t)bulk * 4u, &bar);
+    }
+    if (t < values - bulk) s[bulk + t] = __ldg(src + bulk + t);
+    __syncthreads();
+    if (!mbar_wait_bounded(&bar, 0) && !mbar_wait_bounded(&bar, 0)) {
+        if (t == 0) atomicOr(status, 0x4u);
+        return;
+    }
+    if (t >= rows) return;
+    // lanes whose rows start in the same bank (32 / gcd(row_len, 32) lanes apart) start at different values
+    const int banks = row_len & -row_len;  // gcd with a power of two
+    int e = banks >= 32 ? (t & 31) : (t & 31) / (32 / banks);
+    const float* const row = s + t * row_len;
+    bool fin = true;
+    float best = -INFINITY;
+    int best_k = 0x7fffffff;
+#pragma unroll 4
+    for (int i = 0; i < row_len; ++i) {
+        const float v = row[e];
+        fin &= finite_f(v);
+        const int k = e - 5;
+        if (k >= 0 && (v > best || (v == best && k < best_k))) { best = v; best_k = k; }  // first maximum
+        e = e + 1 == row_len ? 0 : e + 1;
+    }
+    if (!fin) atomicOr(status, 0x1u);
+    const float ob = row[4];
+    if (!fin || !(row[2] > 0.0f) || !(row[3] > 0.0f)) return;
+    auto emit = [&](int cls, float score) {
+        const int slot = atomicAdd(cand_count + img, 1);
+        if (slot < key_stride) keys[(size_t)img * key_stride + slot] = make_key(cls, score, a0 + t);
+        else atomicOr(status, 0x10u);
+    };
+    if (!multi) {
+        const float score = __fmul_rn(ob, best);
+        if (score > conf) emit(agnostic ? 0 : best_k, score);
+    } else {
+        for (int k = 0; k < C; ++k) {
+            const float score = __fmul_rn(ob, row[5 + k]);
+            if (score > conf) emit(k, score);
+        }
+    }
+}
+
+cudaError_t prepare_decode() {
+    return cudaFuncSetAttribute(decode_dense_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kDenseRows * (5 + OCTO_MAX_CLASSES) * (int)sizeof(float));
+}
+
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
     // d_cand_count is zero on entry: zeroed at stage creation and re-zeroed by the NMS kernel.
     const int mode = (a.logits ? 1 : 0) | (a.class_agnostic ? 2 : 0) | (a.multi_label ? 4 : 0);
@@ -317,6 +397,14 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
             return launch_kernel(decode_planes_kernel<1>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C,
                                  mode, a.conf, pre, a.key_stride, a.d_keys, a.d_cand_count, a.d_status, pdl);
         }
+    }
+    if (!a.logits && ((long long)a.A * (5 + a.C)) % 4 == 0 && (reinterpret_cast<uintptr_t>(a.d_head) & 15) == 0) {
+        // (every image starts on a 16-byte boundary, as the bulk copies need; any other head is read
+        // by the row groups of decode_kernel)
+        dim3 grid((a.A + kDenseRows - 1) / kDenseRows, a.n);
+        return launch_kernel(decode_dense_kernel, grid, dim3(kDenseRows), sizeof(float) * kDenseRows * (5 + (size_t)a.C),
+                             stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, a.key_stride, a.d_keys, a.d_cand_count,
+                             a.d_status, pdl);
     }
     const int per_cta4 = kDecThreads * 4;
     if ((long long)a.n * ((a.A + per_cta4 - 1) / per_cta4) >= 296) {

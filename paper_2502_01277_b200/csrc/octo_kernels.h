@@ -97,6 +97,7 @@ int report_cuda_error(cudaError_t e, const char* what);
 
 // Opt the kernels of every table capacity into the shared memory they need (current device).
 cudaError_t prepare_letterbox();
+cudaError_t prepare_decode();
 // max_cluster (optional): the largest cluster of the NMS kernel (8, 4, 2 or 1) that the current
 // device can co-schedule.
 cudaError_t prepare_nms(int* max_cluster = nullptr);

@@ -44,8 +44,8 @@ std::mutex g_mu;
 unsigned char* g_dev_ptr[kMaxDevices];  // device address of g_static_scratch, per device
 bool g_ready[kMaxDevices];
 
-// First use on a device: resolve the device address of the array and opt the NMS kernel
-// into its shared memory.  Neither call allocates.
+// First use on a device: resolve the device address of the array and opt the kernels
+// into their shared memory.  Neither call allocates.
 cudaError_t setup_device(int device, unsigned char** out) {
     std::lock_guard<std::mutex> lock(g_mu);
     if (!g_ready[device]) {
@@ -54,6 +54,7 @@ cudaError_t setup_device(int device, unsigned char** out) {
         if (e != cudaSuccess) return e;
         if (p == nullptr) return cudaErrorInvalidSymbol;
         e = prepare_nms(nullptr);
+        if (e == cudaSuccess) e = prepare_decode();
         if (e != cudaSuccess) return e;
         g_dev_ptr[device] = p;
         g_ready[device] = true;

@@ -168,6 +168,7 @@ extern "C" int octo_stage_create(const octo_stage_config_t* cfg, octo_stage_t** 
     if (e == cudaSuccess) e = dev_alloc(&st->d_ctr, 1, &st->workspace_bytes);
     if (e == cudaSuccess) e = dev_alloc(&st->d_tab, mb, &st->workspace_bytes);
     if (e == cudaSuccess) e = prepare_letterbox();
+    if (e == cudaSuccess) e = prepare_decode();
     if (e == cudaSuccess) e = prepare_nms(&st->nms_max_cluster);
     if (e == cudaSuccess) {
         // an integer the NMS kernel writes and the host reads without a copy

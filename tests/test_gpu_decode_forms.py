@@ -1,0 +1,54 @@
+"""The dense forms of the decode step at the sizes where they can go wrong: rows-layout probabilities
+staged in tiles of 128 rows (partial tiles, rows whose length shares factors with the 32 banks, heads
+that do not start every image on a 16-byte boundary).  Oracle: the CPU decode + NMS; every decision is
+made in the same individually rounded binary32 operations, so kept detections are bit-equal."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2502_01277_b200 as octo
+from gpu_harness import run_stage_gpu
+from test_gpu_parity import _check_dets
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(head, planes, num_anchors, num_classes, **kw):
+    n, s = head.shape[0], 128
+    frames = [np.zeros((96, 384), dtype=np.uint8) for _ in range(n)]
+    sizes = [(128, 96)] * n
+    st = octo.Stage(net_size=s, max_batch=n, num_anchors=num_anchors, num_classes=num_classes, max_det=300,
+                    head_layout="planes" if planes else "rows", branches=((8, 8),), **kw)
+    try:
+        res = run_stage_gpu(st, frames, sizes, head, max_items=[4])
+        ref = oracle.run_stage(frames, sizes, head, s, ((8, 8),), logits=kw.get("head_is_logits", True), max_det=300,
+                               agnostic=kw.get("class_agnostic", False), layout="planes" if planes else "rows",
+                               multi_label=kw.get("multi_label", False), do_letterbox=False, do_crops=False)
+        _check_dets(res, ref)
+        assert res.stats["candidates"] == int(ref.n_cand.sum())
+        return res, ref
+    finally:
+        st.close()
+
+
+def _boxes(rng, shape):
+    return np.concatenate([rng.uniform(0, 128, shape + (2,)), rng.uniform(4, 60, shape + (2,))], -1).astype(np.float32)
+
+
+@pytest.mark.parametrize("anchors", [1, 127, 128, 129, 401])
+@pytest.mark.parametrize("classes", [1, 3, 11, 27, 80, 128])
+@pytest.mark.parametrize("variant", ["single", "multi", "agnostic"])
+def test_probability_rows(anchors, classes, variant):
+    rng = np.random.default_rng(anchors * 131 + classes)
+    head = np.zeros((2, anchors, 5 + classes), dtype=np.float32)
+    head[..., :4] = _boxes(rng, (2, anchors))
+    head[..., 4] = rng.uniform(0.2, 1.0, (2, anchors))
+    few = rng.random((2, anchors, classes)) < 1.2 / classes  # about one label an anchor: the workspace holds two
+    head[..., 5:] = np.where(few, np.round(rng.uniform(0, 1, few.shape) * 16) / 16, 0.01)  # ties among the classes
+    if anchors > 4:
+        head[0, 1, 4 + classes] = np.nan
+        head[1, 2, 2] = 0.0
+        head[1, anchors - 1, 3] = np.inf
+    res, _ = _run(head, False, anchors, classes, head_is_logits=False, multi_label=variant == "multi",
+                  class_agnostic=variant == "agnostic")
+    assert res.status & ~0x2 == (0x1 if anchors > 4 else 0)
