@@ -174,35 +174,42 @@ decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf
 }
 
 // Planes layout [n, 4 + C, A].  A thread owns VEC consecutive anchors (VEC = 4 with 16-byte
-// loads when A is a multiple of 4, else 1); the lanes of a warp and kPlaneAnchorWarps warps side
-// by side read consecutive addresses of one plane, so a CTA fetches long contiguous runs (DRAM
-// pages are used better the longer the run).  kPlaneClassWarps groups of warps split the C class
-// planes between them (group g takes classes g, g + groups, ...) and leave their running first
-// maxima in shared memory, where one thread per anchor merges them.  For multi-label heads in logit form a value is only run
-// through the fixed logistic sequence when it lies above `pre`, a bound placed safely below
-// the threshold's logit, so that the common case costs one comparison per value.
-// Measured on [256, 84, 8400]: 8 x 1 warps (4 KB contiguous per plane and CTA) 0.141 ms, 4 x 2
-// 0.142, 2 x 4 0.156, 1 x 8 0.167; the unroll depth makes no difference from 2 to 16.
-constexpr int kPlaneUnroll = 8;
-constexpr int kPlaneAnchorWarps = 8;                          // warps side by side along the anchors
-constexpr int kPlaneClassWarps = kDecThreads / 32 / kPlaneAnchorWarps;  // warps splitting the classes
+// loads when A is a multiple of 4, else 1); the lanes of a warp and AW warps side by side read
+// consecutive addresses of one plane, so a CTA fetches long contiguous runs (DRAM pages are used
+// better the longer the run).  CW = 8 / AW groups of warps split the C class planes between them
+// (group g takes classes g, g + CW, ...) and leave their running first maxima in shared memory, where
+// one thread per anchor merges them.  Every thread keeps kPlaneBatch planes in flight.
+// Bound by HBM for large batches and by the number of planes a warp walks one after another for small
+// ones, so the split follows the size of the grid: 4 x 2 warps where that still gives every SM six CTAs,
+// else 1 x 8 (measured us per launch, heads of [n, 84, 8400], 1 x 8 / 4 x 2 / 8 x 1: n = 1 8.7 / 12.3 /
+// 17.1, n = 8 14.8 / 20.9 / 33.3, n = 32 31.2 / 31.2 / 41.4, n = 64 47.7 / 45.4 / 50.0, n = 200 110.7 /
+// 105.9 / 121.7; 25.2, 53.8, 61.4, - and 129.4 with 8 x 1 warps and no explicit batch of loads, which
+// the compiler had not kept in flight together).
+// For multi-label heads in logit form a value is only run through the fixed logistic sequence when it
+// lies above `pre`, a bound placed safely below the threshold's logit, so that the common case costs
+// one comparison per value.
+constexpr int kPlaneBatch = 5;
+constexpr int kPlaneWideCtas = 888;  // six CTAs for each of 148 SMs
+constexpr int kPlaneRepeat = 5;      // class planes a lane reads at a time the second time (multi-label)
 
-template <int VEC>
+template <int VEC, int AW, bool MULTI>
 __global__ void __launch_bounds__(kDecThreads)
 decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, float pre, int key_stride,
                      unsigned long long* __restrict__ keys, int* __restrict__ cand_count,
                      unsigned int* __restrict__ status, int pdl) {
     pdl_enter(pdl);
-    constexpr int kCtaAnchors = kPlaneAnchorWarps * 32 * VEC;
-    __shared__ float s_best[kPlaneClassWarps][kCtaAnchors];
-    __shared__ int s_k[kPlaneClassWarps][kCtaAnchors];
-    __shared__ unsigned s_flags[kPlaneClassWarps][kPlaneAnchorWarps * 32];  // bits 0..3: non-finite, 4..7: above `pre`
+    constexpr int CW = kDecThreads / 32 / AW;
+    constexpr int kCtaAnchors = AW * 32 * VEC;
+    __shared__ float s_best[CW][kCtaAnchors];
+    __shared__ unsigned char s_k[CW][kCtaAnchors];
+    __shared__ unsigned char s_flags[CW][AW * 32];  // bits 0..3: non-finite, 4..7: above `pre`
+    __shared__ unsigned short s_list[MULTI ? kCtaAnchors : 1];  // multi-label: anchors with a value above `pre`
+    __shared__ int s_nlist;
     const int logits = mode & 1;
     const bool agnostic = (mode & 2) != 0;
-    const bool multi = (mode & 4) != 0;
     const int img = blockIdx.y;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int aw = warp % kPlaneAnchorWarps, cw = warp / kPlaneAnchorWarps;
+    const int aw = warp % AW, cw = warp / AW;
     const float* __restrict__ hbase = head + (size_t)img * (size_t)(4 + C) * (size_t)A;
     const int col = aw * 32 + lane;  // this thread's group of VEC anchors inside the CTA
     const int a0 = blockIdx.x * kCtaAnchors + col * VEC;
@@ -211,82 +218,108 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
     int best_k[VEC];
     unsigned flags = 0u;
 #pragma unroll
-    for (int u = 0; u < VEC; ++u) { best[u] = -INFINITY; best_k[u] = 0x7fffffff; }
+    for (int u = 0; u < VEC; ++u) { best[u] = -INFINITY; best_k[u] = 255; }
     if (a0 < A) {
         const float* __restrict__ cls0 = hbase + (size_t)4 * A + a0;
-#pragma unroll kPlaneUnroll
-        for (int k = cw; k < C; k += kPlaneClassWarps) {
-            float v[VEC];
-            if (VEC == 4) {
-                const float4 q = __ldg(reinterpret_cast<const float4*>(cls0 + (size_t)k * A));
-                v[0] = q.x; v[1 % VEC] = q.y; v[2 % VEC] = q.z; v[3 % VEC] = q.w;
-            } else {
-                v[0] = __ldg(cls0 + (size_t)k * A);
+        for (int k0 = cw; k0 < C; k0 += CW * kPlaneBatch) {
+            float v[kPlaneBatch][VEC];
+#pragma unroll
+            for (int j = 0; j < kPlaneBatch; ++j) {
+                const int k = min(k0 + j * CW, C - 1);  // past the end: the last plane again (no new maximum)
+                if (VEC == 4) {
+                    const float4 q = __ldg(reinterpret_cast<const float4*>(cls0 + (size_t)k * A));
+                    v[j][0] = q.x; v[j][1 % VEC] = q.y; v[j][2 % VEC] = q.z; v[j][3 % VEC] = q.w;
+                } else {
+                    v[j][0] = __ldg(cls0 + (size_t)k * A);
+                }
             }
 #pragma unroll
-            for (int u = 0; u < VEC; ++u) {
-                if (!finite_f(v[u])) flags |= 1u << u;
-                if (v[u] > best[u]) { best[u] = v[u]; best_k[u] = k; }
-                if (multi && v[u] > pre) flags |= 16u << u;
+            for (int j = 0; j < kPlaneBatch; ++j) {
+                const int k = k0 + j * CW;
+#pragma unroll
+                for (int u = 0; u < VEC; ++u) {
+                    const float x = v[j][u];
+                    if (!finite_f(x)) flags |= 1u << u;
+                    if (x > best[u] && k < C) { best[u] = x; best_k[u] = k; }
+                    if (MULTI && x > pre) flags |= 16u << u;
+                }
             }
         }
     }
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
         s_best[cw][col * VEC + u] = best[u];
-        s_k[cw][col * VEC + u] = best_k[u];
+        s_k[cw][col * VEC + u] = (unsigned char)best_k[u];
     }
-    s_flags[cw][col] = flags;
+    s_flags[cw][col] = (unsigned char)flags;
+    if (threadIdx.x == 0) s_nlist = 0;
     __syncthreads();
 
+    auto emit = [&](int cls, float score, int anchor) {
+        const int slot = atomicAdd(cand_count + img, 1);
+        if (slot < key_stride) keys[(size_t)img * key_stride + slot] = make_key(cls, score, anchor);
+        else atomicOr(status, 0x10u);
+    };
     // one thread per anchor of the CTA
     for (int t = threadIdx.x; t < kCtaAnchors; t += kDecThreads) {
         const int u = t % VEC;
         const int anchor = blockIdx.x * kCtaAnchors + t;
         if (anchor >= A) break;
         float bv = -INFINITY;
-        int bk = 0x7fffffff;
+        int bk = 255;
         unsigned fl = 0u;
 #pragma unroll
-        for (int w = 0; w < kPlaneClassWarps; ++w) {
+        for (int w = 0; w < CW; ++w) {
             const float v = s_best[w][t];
             const int k = s_k[w][t];
             if (v > bv || (v == bv && k < bk)) { bv = v; bk = k; }  // first maximum over all classes
             fl |= s_flags[w][t / VEC];
         }
         const bool bad = (fl >> u) & 1u;
-        if (bad) atomicOr(status, 0x1u);
-        const float* __restrict__ bx = hbase + anchor;
-        auto box_ok = [&]() {  // finite box with w, h > 0
-            const float cx = __ldg(bx), cy = __ldg(bx + A), bw = __ldg(bx + 2 * (size_t)A),
-                        bh = __ldg(bx + 3 * (size_t)A);
-            if (!(finite_f(cx) && finite_f(cy) && finite_f(bw) && finite_f(bh))) {
-                atomicOr(status, 0x1u);
-                return false;
-            }
-            return bw > 0.0f && bh > 0.0f;
-        };
-        auto emit = [&](int cls, float score) {
-            const int slot = atomicAdd(cand_count + img, 1);
-            if (slot < key_stride) keys[(size_t)img * key_stride + slot] = make_key(cls, score, anchor);
-            else atomicOr(status, 0x10u);
-        };
-        if (!multi) {
-            if (bad || bk == 0x7fffffff) continue;
-            const float score = logits ? sigmoid_fixed(bv) : bv;
+        if (bad) {
+            atomicOr(status, 0x1u);
+            continue;
+        }
+        float score = 0.0f;
+        if (!MULTI) {
+            score = logits ? sigmoid_fixed(bv) : bv;
             if (!(score > conf)) continue;
-            if (!box_ok()) continue;
-            emit(agnostic ? 0 : bk, score);
-        } else {
-            // rare: walk the anchor's classes again (the values are in L1 / L2 by now)
-            if (bad || !((fl >> (4 + u)) & 1u)) continue;
-            if (!box_ok()) continue;
+        } else if (!((fl >> (4 + u)) & 1u)) {
+            continue;
+        }
+        // finite box with w, h > 0
+        const float* __restrict__ bx = hbase + anchor;
+        const float cx = __ldg(bx), cy = __ldg(bx + A), bw = __ldg(bx + 2 * (size_t)A), bh = __ldg(bx + 3 * (size_t)A);
+        if (!(finite_f(cx) && finite_f(cy) && finite_f(bw) && finite_f(bh))) {
+            atomicOr(status, 0x1u);
+            continue;
+        }
+        if (!(bw > 0.0f && bh > 0.0f)) continue;
+        if (!MULTI) emit(agnostic ? 0 : bk, score, anchor);
+        else s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)t;
+    }
+    if (!MULTI) return;
+    // Multi-label: every (listed anchor, class) pair is tested by its own lane, a warp taking a class
+    // plane at a time and kPlaneRepeat planes in flight.  Bound by the latency of these second reads
+    // (L2 hits, 4 bytes each): with one thread walking the C classes of its anchor in turn the launch
+    // took 115 us on [32, 84, 8400] with 300 candidates an image, 32-34 us this way (31 without labels).
+    __syncthreads();
+    const int nlist = s_nlist;
+    for (int k0 = warp; k0 < C; k0 += (kDecThreads / 32) * kPlaneRepeat) {
+        for (int q = lane; q < nlist; q += 32) {
+            const int anchor = blockIdx.x * kCtaAnchors + (int)s_list[q];
             const float* __restrict__ cv = hbase + (size_t)4 * A + anchor;
-            for (int k = 0; k < C; ++k) {
-                const float v = __ldg(cv + (size_t)k * A);
-                if (!(v > pre)) continue;
-                const float score = logits ? sigmoid_fixed(v) : v;
-                if (score > conf) emit(k, score);
+            float v[kPlaneRepeat];
+#pragma unroll
+            for (int j = 0; j < kPlaneRepeat; ++j) {
+                const int k = k0 + j * (kDecThreads / 32);
+                v[j] = k < C ? __ldg(cv + (size_t)k * A) : -INFINITY;
+            }
+#pragma unroll
+            for (int j = 0; j < kPlaneRepeat; ++j) {
+                if (!(v[j] > pre)) continue;
+                const float score = logits ? sigmoid_fixed(v[j]) : v[j];
+                if (score > conf) emit(k0 + j * (kDecThreads / 32), score, anchor);
             }
         }
     }
@@ -372,6 +405,22 @@ cudaError_t prepare_decode() {
                                 kDenseRows * (5 + OCTO_MAX_CLASSES) * (int)sizeof(float));
 }
 
+template <int VEC, int AW>
+static cudaError_t launch_planes_split(const DecodeArgs& a, int mode, float pre, cudaStream_t stream) {
+    dim3 grid((a.A + 32 * VEC * AW - 1) / (32 * VEC * AW), a.n);
+    auto kernel = a.multi_label ? decode_planes_kernel<VEC, AW, true> : decode_planes_kernel<VEC, AW, false>;
+    return launch_kernel(kernel, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, pre,
+                         a.key_stride, a.d_keys, a.d_cand_count, a.d_status, a.pdl ? 1 : 0);
+}
+
+// Warps side by side along the anchors, by the number of CTAs that gives (see decode_planes_kernel).
+template <int VEC>
+static cudaError_t launch_planes(const DecodeArgs& a, int mode, float pre, cudaStream_t stream) {
+    const long long ctas = (long long)a.n * ((a.A + 128 * VEC - 1) / (128 * VEC));
+    return ctas >= kPlaneWideCtas ? launch_planes_split<VEC, 4>(a, mode, pre, stream)
+                                  : launch_planes_split<VEC, 1>(a, mode, pre, stream);
+}
+
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
     // d_cand_count is zero on entry: zeroed at stage creation and re-zeroed by the NMS kernel.
     const int mode = (a.logits ? 1 : 0) | (a.class_agnostic ? 2 : 0) | (a.multi_label ? 4 : 0);
@@ -388,15 +437,8 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
                 pre = (float)(t - 1e-3 * (1.0 + fabs(t)));
             }
         }
-        if ((a.A & 3) == 0 && (reinterpret_cast<uintptr_t>(a.d_head) & 15) == 0) {
-            dim3 grid((a.A + 128 * kPlaneAnchorWarps - 1) / (128 * kPlaneAnchorWarps), a.n);
-            return launch_kernel(decode_planes_kernel<4>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C,
-                                 mode, a.conf, pre, a.key_stride, a.d_keys, a.d_cand_count, a.d_status, pdl);
-        } else {
-            dim3 grid((a.A + 32 * kPlaneAnchorWarps - 1) / (32 * kPlaneAnchorWarps), a.n);
-            return launch_kernel(decode_planes_kernel<1>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C,
-                                 mode, a.conf, pre, a.key_stride, a.d_keys, a.d_cand_count, a.d_status, pdl);
-        }
+        const bool vec = (a.A & 3) == 0 && (reinterpret_cast<uintptr_t>(a.d_head) & 15) == 0;
+        return vec ? launch_planes<4>(a, mode, pre, stream) : launch_planes<1>(a, mode, pre, stream);
     }
     if (!a.logits && ((long long)a.A * (5 + a.C)) % 4 == 0 && (reinterpret_cast<uintptr_t>(a.d_head) & 15) == 0) {
         // (every image starts on a 16-byte boundary, as the bulk copies need; any other head is read

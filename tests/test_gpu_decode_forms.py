@@ -1,7 +1,9 @@
 """The dense forms of the decode step at the sizes where they can go wrong: rows-layout probabilities
 staged in tiles of 128 rows (partial tiles, rows whose length shares factors with the 32 banks, heads
-that do not start every image on a 16-byte boundary).  Oracle: the CPU decode + NMS; every decision is
-made in the same individually rounded binary32 operations, so kept detections are bit-equal."""
+that do not start every image on a 16-byte boundary), and planes heads in both warp splits with the
+second look of multi-label heads at the anchors with a value above the threshold.  Oracle: the CPU
+decode + NMS; every decision is made in the same individually rounded binary32 operations, so kept
+detections are bit-equal."""
 import numpy as np
 import pytest
 
@@ -52,3 +54,31 @@ def test_probability_rows(anchors, classes, variant):
     res, _ = _run(head, False, anchors, classes, head_is_logits=False, multi_label=variant == "multi",
                   class_agnostic=variant == "agnostic")
     assert res.status & ~0x2 == (0x1 if anchors > 4 else 0)
+
+
+@pytest.mark.parametrize("anchors", [3, 4, 127, 128, 516, 1028])
+@pytest.mark.parametrize("classes,logits", [(1, False), (39, True), (41, False), (128, True)])
+@pytest.mark.parametrize("multi", [False, True])
+def test_planes(anchors, classes, logits, multi):
+    """Class counts around the planes a warp looks at together (8 warps x 5 planes), anchor counts around
+    a CTA's share (128 or 32), in the vector and the scalar form (anchors not a multiple of four)."""
+    _planes(2, anchors, classes, logits, multi)
+
+
+@pytest.mark.parametrize("anchors,n", [(128 * 5, 512), (128 * 2 - 1, 512)])
+def test_planes_wide_split(anchors, n):
+    """Enough CTAs (888) for four warps side by side along the anchors: vector and scalar form."""
+    _planes(n, anchors, 9, True, True)
+
+
+def _planes(n, anchors, classes, logits, multi):
+    rng = np.random.default_rng(anchors * 17 + classes)
+    head = np.full((n, 4 + classes, anchors), -6.0, dtype=np.float32)
+    head[:, :4] = np.moveaxis(_boxes(rng, (n, anchors)), -1, 1)
+    some = rng.random((n, 1, anchors)) < max(0.05, 3.0 / anchors)
+    strong = some & (rng.random((n, classes, anchors)) < 1.2 / classes)  # about one label: the workspace holds two
+    head[:, 4:] = np.where(strong, rng.normal(0.0, 1.5, strong.shape), -6.0)
+    head[1, 4 + classes - 1, anchors - 1] = 3.0  # the last value of the head
+    if not logits:
+        head[:, 4:] = 1.0 / (1.0 + np.exp(-head[:, 4:]))
+    _run(head.astype(np.float32), True, anchors, classes, head_is_logits=logits, multi_label=multi and classes > 1)
