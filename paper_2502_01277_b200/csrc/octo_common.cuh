@@ -400,16 +400,53 @@ __device__ __forceinline__ void iou_terms(const float4 a, const float4 b, float&
 // next float up (or on it, when that next float has an even mantissa and so wins the tie).
 // inter, uni and mid have 24, 24 and 25 significant bits, so mid * uni is exact in binary64
 // and the comparison is exact.  Non-finite operands compare false, like the quotient would.
+//
+// Almost every pair is decided in binary32 already: t = fl(midf * uni), midf = fl(mid), is within
+// 2^-22.9 of mid * uni (two roundings, t a normal number), so |inter - t| > 2^-20 t settles the sign.
+// The binary64 form needs two conversions per pair, which issue at a fraction of the binary32 rate.
 struct IouTest {
     double mid;
+    float midf;
+    float share;  // mid / (1 + mid), see iou_by_share
     int tie_up;
 };
-__device__ __forceinline__ bool iou_above(const float4 a, const float4 b, const IouTest t) {
-    float inter, uni;
-    iou_terms(a, b, inter, uni);
+__device__ __forceinline__ bool iou_exact(float inter, float uni, const IouTest& t) {
     if (!(uni > 0.0f)) return false;
     const double lhs = (double)inter, rhs = __dmul_rn(t.mid, (double)uni);
     return t.tie_up ? lhs >= rhs : lhs > rhs;
+}
+// The binary32 decision; `close` is set when it does not settle the pair.
+__device__ __forceinline__ bool iou_quick(const float4 a, const float4 b, const IouTest& t, bool& close) {
+    float inter, uni;
+    iou_terms(a, b, inter, uni);
+    const float prod = __fmul_rn(t.midf, uni);
+    const float d = __fsub_rn(inter, prod);
+    close |= !(fabsf(d) > __fmul_rn(prod, 0x1p-20f) && prod > 0x1p-100f);
+    return d > 0.0f;
+}
+// The same decision for a box that meets many others: inter > mid * (area_a + area_b - inter) is inter >
+// share * area_a + share * area_b, with the two products made once per box (iou_share).  All roundings
+// together (those of the formula's own union among them) stay below 2^-21 of the sum, so a distance of
+// more than 2^-19 of it settles the pair.  One side of the overlap may stay negative: with the other
+// clamped to zero the product is then at most zero, as it should be.
+__device__ __forceinline__ float iou_share(const float4 a, const IouTest& t) {
+    return __fmul_rn(t.share, __fmul_rn(__fsub_rn(a.z, a.x), __fsub_rn(a.w, a.y)));
+}
+__device__ __forceinline__ bool iou_by_share(const float4 a, float share_a, const float4 b, float share_b, bool& close) {
+    const float iw = fmaxf(__fsub_rn(fminf(a.z, b.z), fmaxf(a.x, b.x)), 0.0f);
+    const float ih = __fsub_rn(fminf(a.w, b.w), fmaxf(a.y, b.y));
+    const float s = __fadd_rn(share_a, share_b);
+    const float d = __fsub_rn(__fmul_rn(iw, ih), s);
+    close |= !(fabsf(d) > __fmaf_rn(s, 0x1p-19f, 0x1p-100f));
+    return d > 0.0f;
+}
+__device__ __forceinline__ bool iou_above(const float4 a, const float4 b, const IouTest& t) {
+    bool close = false;
+    const bool quick = iou_quick(a, b, t, close);
+    if (!close) return quick;
+    float inter, uni;
+    iou_terms(a, b, inter, uni);
+    return iou_exact(inter, uni, t);
 }
 
 }  // namespace octo

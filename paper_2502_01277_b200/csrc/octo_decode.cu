@@ -43,9 +43,9 @@ __device__ __forceinline__ unsigned long long make_key(int cls, float score, int
 // kDecPerThread anchors per thread: 4 for large batches, 1 when the grid would otherwise be
 // too small to cover the SMs.
 template <int kDecPerThread>
-__global__ void __launch_bounds__(kDecThreads)
+__global__ void __launch_bounds__(kDecThreads, kDecPerThread == 1 ? 5 : 1)
 decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, int key_stride,
-              unsigned long long* __restrict__ keys, int* __restrict__ cand_count,
+              unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
               unsigned int* __restrict__ status, int pdl) {
     pdl_enter(pdl);
     // mode bit 0: obj / class values are logits; bit 1: class-agnostic NMS (key class field 0);
@@ -124,6 +124,7 @@ decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf
             const float bw = __shfl_sync(0xffffffffu, e0, gbase + 2);
             const float bh = __shfl_sync(0xffffffffu, e0, gbase + 3);
             const float ob = __shfl_sync(0xffffffffu, e0, gbase + 4);
+            const float cy = __shfl_sync(0xffffffffu, e0, gbase + 1);  // (the group's first lane holds cx)
             if (bad) nonfinite_seen = true;
             const bool ok = have && !bad && bw > 0.0f && bh > 0.0f;
             if (!multi) {
@@ -138,16 +139,19 @@ decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf
                                                : __fmul_rn(ob, best);
                     if (score > conf) {
                         const int slot = atomicAdd(cand_count + img, 1);
-                        if (slot < key_stride)
+                        if (slot < key_stride) {
                             keys[(size_t)img * key_stride + slot] = make_key(agnostic ? 0 : best_k, score, ra);
-                        else
+                            boxes[(size_t)img * key_stride + slot] = box_corners(e0, cy, bw, bh);
+                        } else {
                             atomicOr(status, 0x10u);
+                        }
                     }
                 }
             } else {
                 // one candidate per class whose own score passes; the keys of a row go out in
                 // groups of up to eight with one counter update per group
                 const float so = logits ? sigmoid_fixed(ob) : ob;
+                const float4 box = box_corners(__shfl_sync(0xffffffffu, e0, gbase), cy, bw, bh);
                 for (int e0i = 0; e0i < row_len; e0i += 8) {  // the same trip count in every group
                     const int e = e0i + gl;
                     float score = 0.0f;
@@ -163,8 +167,12 @@ decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf
                     base = __shfl_sync(0xffffffffu, base, gbase);
                     if (hit) {
                         const int slot = base + __popc(hits & ((1u << lane) - 1u));
-                        if (slot < key_stride) keys[(size_t)img * key_stride + slot] = make_key(e - 5, score, ra);
-                        else atomicOr(status, 0x10u);
+                        if (slot < key_stride) {
+                            keys[(size_t)img * key_stride + slot] = make_key(e - 5, score, ra);
+                            boxes[(size_t)img * key_stride + slot] = box;
+                        } else {
+                            atomicOr(status, 0x10u);
+                        }
                     }
                 }
             }
@@ -195,7 +203,7 @@ constexpr int kPlaneRepeat = 5;      // class planes a lane reads at a time the 
 template <int VEC, int AW, bool MULTI>
 __global__ void __launch_bounds__(kDecThreads)
 decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, float pre, int key_stride,
-                     unsigned long long* __restrict__ keys, int* __restrict__ cand_count,
+                     unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
                      unsigned int* __restrict__ status, int pdl) {
     pdl_enter(pdl);
     constexpr int CW = kDecThreads / 32 / AW;
@@ -204,6 +212,7 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
     __shared__ unsigned char s_k[CW][kCtaAnchors];
     __shared__ unsigned char s_flags[CW][AW * 32];  // bits 0..3: non-finite, 4..7: above `pre`
     __shared__ unsigned short s_list[MULTI ? kCtaAnchors : 1];  // multi-label: anchors with a value above `pre`
+    __shared__ float4 s_box[MULTI ? kCtaAnchors : 1];           // ... and their boxes
     __shared__ int s_nlist;
     const int logits = mode & 1;
     const bool agnostic = (mode & 2) != 0;
@@ -255,10 +264,14 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
     if (threadIdx.x == 0) s_nlist = 0;
     __syncthreads();
 
-    auto emit = [&](int cls, float score, int anchor) {
+    auto emit = [&](int cls, float score, int anchor, const float4 box) {
         const int slot = atomicAdd(cand_count + img, 1);
-        if (slot < key_stride) keys[(size_t)img * key_stride + slot] = make_key(cls, score, anchor);
-        else atomicOr(status, 0x10u);
+        if (slot < key_stride) {
+            keys[(size_t)img * key_stride + slot] = make_key(cls, score, anchor);
+            boxes[(size_t)img * key_stride + slot] = box;
+        } else {
+            atomicOr(status, 0x10u);
+        }
     };
     // one thread per anchor of the CTA
     for (int t = threadIdx.x; t < kCtaAnchors; t += kDecThreads) {
@@ -295,8 +308,14 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
             continue;
         }
         if (!(bw > 0.0f && bh > 0.0f)) continue;
-        if (!MULTI) emit(agnostic ? 0 : bk, score, anchor);
-        else s_list[atomicAdd(&s_nlist, 1)] = (unsigned short)t;
+        const float4 box = box_corners(cx, cy, bw, bh);
+        if (!MULTI) {
+            emit(agnostic ? 0 : bk, score, anchor, box);
+        } else {
+            const int q = atomicAdd(&s_nlist, 1);
+            s_list[q] = (unsigned short)t;
+            s_box[q] = box;
+        }
     }
     if (!MULTI) return;
     // Multi-label: every (listed anchor, class) pair is tested by its own lane, a warp taking a class
@@ -319,7 +338,7 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
             for (int j = 0; j < kPlaneRepeat; ++j) {
                 if (!(v[j] > pre)) continue;
                 const float score = logits ? sigmoid_fixed(v[j]) : v[j];
-                if (score > conf) emit(k0 + j * (kDecThreads / 32), score, anchor);
+                if (score > conf) emit(k0 + j * (kDecThreads / 32), score, anchor, s_box[q]);
             }
         }
     }
@@ -338,7 +357,7 @@ constexpr int kDenseRows = 128;
 
 __global__ void __launch_bounds__(kDenseRows)
 decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, int key_stride,
-                    unsigned long long* __restrict__ keys, int* __restrict__ cand_count,
+                    unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
                     unsigned int* __restrict__ status, int pdl) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
@@ -386,8 +405,12 @@ decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, floa
     if (!fin || !(row[2] > 0.0f) || !(row[3] > 0.0f)) return;
     auto emit = [&](int cls, float score) {
         const int slot = atomicAdd(cand_count + img, 1);
-        if (slot < key_stride) keys[(size_t)img * key_stride + slot] = make_key(cls, score, a0 + t);
-        else atomicOr(status, 0x10u);
+        if (slot < key_stride) {
+            keys[(size_t)img * key_stride + slot] = make_key(cls, score, a0 + t);
+            boxes[(size_t)img * key_stride + slot] = box_corners(row[0], row[1], row[2], row[3]);
+        } else {
+            atomicOr(status, 0x10u);
+        }
     };
     if (!multi) {
         const float score = __fmul_rn(ob, best);
@@ -410,7 +433,7 @@ static cudaError_t launch_planes_split(const DecodeArgs& a, int mode, float pre,
     dim3 grid((a.A + 32 * VEC * AW - 1) / (32 * VEC * AW), a.n);
     auto kernel = a.multi_label ? decode_planes_kernel<VEC, AW, true> : decode_planes_kernel<VEC, AW, false>;
     return launch_kernel(kernel, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, pre,
-                         a.key_stride, a.d_keys, a.d_cand_count, a.d_status, a.pdl ? 1 : 0);
+                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, a.pdl ? 1 : 0);
 }
 
 // Warps side by side along the anchors, by the number of CTAs that gives (see decode_planes_kernel).
@@ -445,18 +468,18 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
         // by the row groups of decode_kernel)
         dim3 grid((a.A + kDenseRows - 1) / kDenseRows, a.n);
         return launch_kernel(decode_dense_kernel, grid, dim3(kDenseRows), sizeof(float) * kDenseRows * (5 + (size_t)a.C),
-                             stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, a.key_stride, a.d_keys, a.d_cand_count,
+                             stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count,
                              a.d_status, pdl);
     }
     const int per_cta4 = kDecThreads * 4;
     if ((long long)a.n * ((a.A + per_cta4 - 1) / per_cta4) >= 296) {
         dim3 grid((a.A + per_cta4 - 1) / per_cta4, a.n);
         return launch_kernel(decode_kernel<4>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode,
-                             a.conf, a.key_stride, a.d_keys, a.d_cand_count, a.d_status, pdl);
+                             a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, pdl);
     }
     dim3 grid((a.A + kDecThreads - 1) / kDecThreads, a.n);
     return launch_kernel(decode_kernel<1>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf,
-                         a.key_stride, a.d_keys, a.d_cand_count, a.d_status, pdl);
+                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, pdl);
 }
 
 }  // namespace octo

@@ -23,6 +23,7 @@ struct DecodeArgs {
     float conf;
     int key_stride;
     unsigned long long* d_keys;
+    float4* d_boxes;  // box of every candidate, at its key's slot
     int* d_cand_count;
     unsigned int* d_status;
     bool pdl;  // launch with programmatic stream serialisation (small batches)

@@ -144,7 +144,7 @@ extern "C" int octo_postprocess_frame_static(int32_t device, const float* d_head
     da.logits = head_is_logits; da.class_agnostic = 0; da.multi_label = 0;
     da.conf = conf_thresh;
     da.key_stride = key_stride;
-    da.d_keys = d_keys; da.d_cand_count = d_cand; da.d_status = &d_ctr->status;
+    da.d_keys = d_keys; da.d_boxes = d_boxes; da.d_cand_count = d_cand; da.d_status = &d_ctr->status;
     da.pdl = false;
     e = launch_decode(da, stream);
     if (e != cudaSuccess) return report_cuda_error(e, "decode_kernel");

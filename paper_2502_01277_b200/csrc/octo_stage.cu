@@ -418,7 +418,7 @@ extern "C" int octo_postprocess_batch(octo_stage_t* st, const float* d_head, int
         da.logits = c.head_is_logits; da.class_agnostic = c.class_agnostic; da.multi_label = c.multi_label;
         da.conf = c.conf_thresh;
         da.key_stride = st->key_stride;
-        da.d_keys = st->d_keys; da.d_cand_count = st->d_cand_count; da.d_status = &st->d_ctr->status;
+        da.d_keys = st->d_keys; da.d_boxes = st->d_boxes; da.d_cand_count = st->d_cand_count; da.d_status = &st->d_ctr->status;
         da.pdl = n <= kPdlMaxBatch;
         OCTO_CUDA(launch_decode(da, stream));
     }

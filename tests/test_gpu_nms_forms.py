@@ -1,0 +1,85 @@
+"""NMS where its forms meet: candidate counts around a warp, the short path (512, with 4, 2 and 1 threads
+per candidate), a class that the whole CTA takes (128 .. 512 and above, in blocks of 128), the network
+sort (512), the half-sized and the full on-chip capacity; chains of overlapping boxes (as many rounds as
+links), identical boxes, IoU values that lie exactly on the threshold, a small cap, clusters.  The oracle
+makes the same binary32 decisions, so kept detections are bit-equal."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2502_01277_b200 as octo
+from gpu_harness import run_stage_gpu
+from paper_2502_01277_b200 import binding as B
+from test_gpu_parity import _check_dets
+
+pytestmark = pytest.mark.gpu
+CLASSES, SIDE = 5, 256
+
+
+def _boxes(rng, m, kind):
+    """(cx, cy, w, h) of m boxes."""
+    if kind == "chain":  # neighbours overlap above the threshold, the next but one does not
+        i = np.arange(m)
+        per = 60
+        return np.stack([8 + 4.0 * (i % per), 6 + 12.0 * ((i // per) % 20), np.full(m, 10.0), np.full(m, 10.0)], 1)
+    if kind == "same":
+        return np.tile(np.array([[100.0, 90.0, 30.0, 20.0]]), (m, 1))
+    # a coarse grid of sizes and places: many IoU values are simple fractions, 1/2 among them
+    return np.stack([rng.integers(4, 60, m) * 4.0, rng.integers(4, 40, m) * 4.0, rng.integers(1, 9, m) * 4.0,
+                     rng.integers(1, 9, m) * 4.0], 1)
+
+
+def _check(m, kind, share, cluster=0, agnostic=False, max_det=300, batch=1, iou=0.5):
+    rng = np.random.default_rng(m * 7 + len(kind))
+    anchors = max(m, 4) + 3
+    head = np.zeros((batch, anchors, 5 + CLASSES), dtype=np.float32)
+    for b in range(batch):
+        at = rng.permutation(anchors)[:m]
+        head[b, at, :4] = _boxes(rng, m, kind)
+        head[b, at, 4] = 1.0
+        cls = np.where(rng.random(m) < share, 2, rng.integers(0, CLASSES, m))
+        head[b, at, 5 + cls] = np.round(rng.uniform(0.3, 0.99, m) * 512) / 512  # ties in the score
+        if kind == "chain":  # strongest first: every second link survives, one link settled per round
+            head[b, at, 5:] = 0.0
+            head[b, at, 7] = np.linspace(0.99, 0.3, m)
+    frames, sizes = [np.zeros((192, 768), dtype=np.uint8)] * batch, [(256, 192)] * batch
+    st = octo.Stage(net_size=SIDE, max_batch=batch, num_anchors=anchors, num_classes=CLASSES, head_is_logits=False,
+                    iou_thresh=iou, max_det=max_det, branches=((8, 8),), class_agnostic=agnostic)
+    try:
+        st.set_nms_cluster(cluster)
+        ref = oracle.run_stage(frames, sizes, head, SIDE, ((8, 8),), logits=False, iou_thr=iou, max_det=max_det,
+                               agnostic=agnostic, do_letterbox=False, do_crops=False)
+        assert int(ref.n_cand[0]) == m
+        for _ in range(2):  # the counters are left clean
+            res = run_stage_gpu(st, frames, sizes, head, max_items=[4])
+            _check_dets(res, ref)
+        assert res.status & ~0x2 == (B.OCTO_STATUS_BIG_NMS if m > 8192 else 0)
+        assert np.array_equal(res.offsets[0][:2], ref.offsets[0][:2])
+    finally:
+        st.close()
+
+
+@pytest.mark.parametrize("m", [0, 1, 2, 31, 32, 33, 127, 130, 255, 256, 257, 400, 511, 512, 513])
+@pytest.mark.parametrize("kind", ["grid", "chain", "same"])
+@pytest.mark.parametrize("agnostic", [False, True])
+def test_short_path(m, kind, agnostic):
+    _check(m, kind, 0.5, agnostic=agnostic)
+
+
+@pytest.mark.parametrize("m,share", [(513, 0.0), (520, 0.4), (640, 1.0), (1024, 0.9), (1030, 1.0), (2100, 0.2),
+                                     (4097, 1.0), (8192, 0.3), (8200, 1.0)])
+@pytest.mark.parametrize("cluster", [1, 4])
+def test_large_classes(m, share, cluster):
+    _check(m, "grid", share, cluster=cluster, max_det=1000)
+
+
+@pytest.mark.parametrize("m,max_det", [(120, 5), (256, 300), (600, 5), (600, 1), (1100, 70)])
+@pytest.mark.parametrize("kind", ["grid", "chain"])
+def test_cap_and_chains(m, max_det, kind):
+    _check(m, kind, 1.0, max_det=max_det, batch=2)
+
+
+def test_thresholds_at_the_ends():
+    for iou in (0.0, 1.0):
+        _check(150, "grid", 0.7, iou=iou)
+        _check(600, "grid", 0.7, iou=iou)
