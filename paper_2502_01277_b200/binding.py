@@ -10,6 +10,8 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
+from collections import deque
 from dataclasses import dataclass
 from typing import List, Optional, Sequence, Tuple
 
@@ -324,6 +326,16 @@ def octo_stage_get_stats(handle, stream: int = 0) -> dict:
 
 # ---- convenience object for torch callers ----------------------------------------------------
 
+def _stream_getter(torch, device):
+    """Raw handle of torch's current stream on `device`.  The stream object torch.cuda.current_stream
+    builds costs a microsecond per call, which a pass of 25 us over one small frame makes three times."""
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return lambda: int(torch.cuda.current_stream(device).cuda_stream)
+    index = device.index
+    return lambda: raw(index)
+
+
 class Stage:
     """Owns one octo_stage_t and the torch tensors a caller usually wants around it."""
 
@@ -335,6 +347,9 @@ class Stage:
         self.device = torch.device("cuda", self.cfg.device)
         self.n = 0
         self._frames_keepalive: List = []
+        self._lib = load_library()
+        self._current_stream = _stream_getter(torch, self.device)
+        self._frame_array = (Frame * self.cfg.max_batch)()  # refilled by every preprocess call
 
     def close(self) -> None:
         if getattr(self, "handle", None):
@@ -348,9 +363,7 @@ class Stage:
             pass
 
     def _stream(self, stream) -> int:
-        if stream is None:
-            stream = self._torch.cuda.current_stream(self.device)
-        return int(stream.cuda_stream)
+        return self._current_stream() if stream is None else int(stream.cuda_stream)
 
     def preprocess(self, frames, sizes, out=None, stream=None):
         """frames: list of uint8 CUDA tensors [h, pitch]; sizes: (w, h) per frame.
@@ -359,8 +372,14 @@ class Stage:
         n, s = len(frames), self.cfg.net_size
         if out is None:
             out = t.empty((n, 3, s, s), dtype=t.float16, device=self.device)
-        desc = [(f.data_ptr(), w, h, f.stride(0)) for f, (w, h) in zip(frames, sizes)]
-        octo_preprocess_batch(self.handle, desc, out.data_ptr(), self._stream(stream))
+        arr = self._frame_array if n <= self.cfg.max_batch else (Frame * n)()  # (the library refuses the latter)
+        flat = []
+        for f, (w, h) in zip(frames, sizes):
+            flat += (f.data_ptr(), w, h, f.stride()[0], 0)
+        struct.pack_into("@" + "Piiii" * n, arr, 0, *flat)
+        rc = self._lib.octo_preprocess_batch(self.handle, arr, n, out.data_ptr(), self._stream(stream))
+        if rc != OCTO_OK:
+            raise OctoError(rc, "octo_preprocess_batch")
         self._frames_keepalive = list(frames)
         self.n = n
         return out
@@ -374,7 +393,7 @@ class Stage:
         return arr
 
     def preprocess_array(self, arr, n, out, stream=None, keepalive=None):
-        rc = load_library().octo_preprocess_batch(self.handle, arr, n, out.data_ptr(), self._stream(stream))
+        rc = self._lib.octo_preprocess_batch(self.handle, arr, n, out.data_ptr(), self._stream(stream))
         if rc != OCTO_OK:
             raise OctoError(rc, "octo_preprocess_batch")
         if keepalive is not None:
@@ -427,23 +446,27 @@ class Stage:
             dets = t.empty((n, self.cfg.max_det, 32), dtype=t.uint8, device=self.device)
         if counts is None:
             counts = t.empty((n,), dtype=t.int32, device=self.device)
-        octo_postprocess_batch(self.handle, head.data_ptr(), n, dets.data_ptr(), counts.data_ptr(),
-                               self._stream(stream))
+        rc = self._lib.octo_postprocess_batch(self.handle, head.data_ptr(), n, dets.data_ptr(), counts.data_ptr(),
+                                              self._stream(stream))
+        if rc != OCTO_OK:
+            raise OctoError(rc, "octo_postprocess_batch")
         self._dets_keepalive = dets
         return dets, counts
 
     def crop(self, branch, max_items, first_item=0, out=None, offsets=None, n_items=None, stream=None):
         """Returns (crops fp16 [max_items, 3, oh, ow], offsets int32 [n+1], n_items int32 [2])."""
         t = self._torch
-        ow, oh = self.cfg.branch[branch].out_w, self.cfg.branch[branch].out_h
         if out is None:
+            ow, oh = self.cfg.branch[branch].out_w, self.cfg.branch[branch].out_h
             out = t.empty((max(max_items, 1), 3, oh, ow), dtype=t.float16, device=self.device)
         if offsets is None:
             offsets = t.empty((self.n + 1,), dtype=t.int32, device=self.device)
         if n_items is None:
             n_items = t.empty((2,), dtype=t.int32, device=self.device)
-        octo_crop_batch(self.handle, branch, first_item, max_items, out.data_ptr(), offsets.data_ptr(),
-                        n_items.data_ptr(), self._stream(stream))
+        rc = self._lib.octo_crop_batch(self.handle, branch, first_item, max_items, out.data_ptr(), offsets.data_ptr(),
+                                       n_items.data_ptr(), self._stream(stream))
+        if rc != OCTO_OK:
+            raise OctoError(rc, "octo_crop_batch")
         return out, offsets, n_items
 
     def item_table(self, branch: int, count: int) -> np.ndarray:
@@ -513,7 +536,9 @@ class Queue:
         if rc != OCTO_OK:
             raise OctoError(rc, "octo_queue_create")
         self.handle = h
-        self._keepalive = []
+        self._lib = load_library()
+        self._current_stream = _stream_getter(torch, self.device)
+        self._keepalive = deque(maxlen=64)  # frames of the latest pushes
 
     def close(self) -> None:
         if getattr(self, "handle", None):
@@ -521,9 +546,7 @@ class Queue:
             self.handle = None
 
     def _stream(self, stream) -> int:
-        if stream is None:
-            stream = self._torch.cuda.current_stream(self.device)
-        return int(stream.cuda_stream)
+        return self._current_stream() if stream is None else int(stream.cuda_stream)
 
     def set_options(self, keep_aspect: bool = False, mean=None, std=None, pad_value: int = 114) -> None:
         """Crop options of the downstream model (see octo_branch_cfg_t)."""
@@ -539,11 +562,10 @@ class Queue:
             raise OctoError(rc, "octo_queue_set_options")
 
     def push(self, stage: "Stage", branch: int = 0, stream=None) -> None:
-        rc = load_library().octo_queue_push(self.handle, stage.handle, branch, self._stream(stream))
+        rc = self._lib.octo_queue_push(self.handle, stage.handle, branch, self._stream(stream))
         if rc != OCTO_OK:
             raise OctoError(rc, "octo_queue_push")
         self._keepalive.append(list(stage._frames_keepalive))  # frames stay alive while queued
-        self._keepalive = self._keepalive[-64:]
 
     def pop(self, bz: int, out=None, items=None, info=None, stream=None, max_wait: int = -1):
         """Returns (crops fp16 [bz, 3, oh, ow], items uint8 [bz, 48], info int32 [4]).  With
@@ -556,8 +578,8 @@ class Queue:
             items = t.zeros((bz, QITEM_DTYPE.itemsize), dtype=t.uint8, device=self.device)
         if info is None:
             info = t.zeros((4,), dtype=t.int32, device=self.device)
-        rc = load_library().octo_queue_pop_due(self.handle, bz, max_wait, out.data_ptr(), items.data_ptr(),
-                                               info.data_ptr(), self._stream(stream))
+        rc = self._lib.octo_queue_pop_due(self.handle, bz, max_wait, out.data_ptr(), items.data_ptr(),
+                                          info.data_ptr(), self._stream(stream))
         if rc != OCTO_OK:
             raise OctoError(rc, "octo_queue_pop_due")
         return out, items, info
