@@ -709,11 +709,11 @@ cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int
     memset(&opts, 0, sizeof(opts));
     if (general) opts = *general;
     auto kernel = general ? crop_kernel<1, true, true> : crop_kernel<1, true, false>;
-    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, false, tab,
+    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, true, tab,
                          (const FrameDesc*)nullptr, 0, 0, 0, bz, (const int*)nullptr, (const int*)nullptr,
                          (const octo_det_t*)nullptr, (int*)nullptr, (int*)nullptr, (octo_item_t*)nullptr,
                          reinterpret_cast<__half*>(d_out), out_w, out_h, swap_rb, (StageCounters*)nullptr, d_staged,
-                         d_qpacked, d_status, d_sched, opts, 0);
+                         d_qpacked, d_status, d_sched, opts, 1);
 }
 
 }  // namespace octo
