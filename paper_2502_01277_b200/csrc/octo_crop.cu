@@ -275,7 +275,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                 }
                 t.f = lo;
                 if (OCTO_IN_RANGE(item - s_off[t.f] >= 0 && item - s_off[t.f] < max_det, status))
-                    t.det = bidx[(size_t)t.f * max_det + (item - s_off[t.f])];
+                    t.det = bidx ? bidx[(size_t)t.f * max_det + (item - s_off[t.f])] : item - s_off[t.f];
                 if (!OCTO_IN_RANGE(t.det >= 0 && t.det < max_det, status)) t.det = 0;
                 const octo_det_t d = dets[(size_t)t.f * max_det + t.det];
                 const FrameDesc fd = gtab ? gtab[t.f] : tab.f[t.f];

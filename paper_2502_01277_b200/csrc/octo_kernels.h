@@ -47,8 +47,9 @@ struct NmsArgs {
     int num_branches;
     int class_agnostic;  // NMS across classes; the class of a survivor is recomputed for the output
     BranchMasks masks;
+    int full_branches;  // bit b: the mask of branch b holds every class
     int* d_bcount;
-    int* d_bidx;
+    int* d_bidx;        // not written for those branches
     int max_batch;
     StageCounters* d_ctr;
     // CTAs per image (a thread-block cluster; 1, 2, 4 or 8).  More than one pays off when few
@@ -77,7 +78,7 @@ struct CropArgs {
     int n;
     int max_det, first_item, max_items;
     const int* d_bcount;  // this branch's [max_batch]
-    const int* d_bidx;    // this branch's [max_batch][max_det]
+    const int* d_bidx;    // this branch's [max_batch][max_det], or null: item j of a frame is its detection j
     const octo_det_t* d_dets;
     int* d_offsets;
     int* d_n_items;

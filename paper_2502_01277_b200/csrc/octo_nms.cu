@@ -42,12 +42,7 @@ static NmsParams nms_params(const NmsArgs& a) {
     p.counts = a.d_counts;
     p.num_branches = a.num_branches; p.class_agnostic = a.class_agnostic;
     p.masks = a.masks;
-    p.full_branches = 0;
-    for (int b = 0; b < a.num_branches; ++b) {
-        bool full = true;
-        for (int k = 0; k < a.C; ++k) full = full && ((a.masks.m[b][k >> 5] >> (k & 31)) & 1u);
-        if (full) p.full_branches |= 1 << b;
-    }
+    p.full_branches = a.full_branches;
     p.bcount = a.d_bcount; p.bidx = a.d_bidx;
     p.max_batch = a.max_batch;
     p.ctr = a.d_ctr;

@@ -306,15 +306,6 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
     const RegionMap map(fd);
     unsigned long long* ordered;  // survivors in output order (inverted score | anchor | class)
     int nout;
-    // index list of a branch that takes every class: all detections, known before their order is
-    auto write_full_lists = [&]() {
-        for (int b = 0; b < P.num_branches; ++b) {
-            if (!((P.full_branches >> b) & 1)) continue;
-            int* const list = P.bidx + ((size_t)b * P.max_batch + img) * max_det;
-            for (int r = tid; r < nout; r += NT) list[r] = r;
-            if (tid == NT - 1) P.bcount[b * P.max_batch + img] = nout;
-        }
-    };
     if (cnt <= kSmallMax) {
         if (crank != 0) return;  // the first CTA alone; no cluster barrier follows on this path
         // Thread (candidate c = word * 32 + lane, part): the 4, 2 or 1 parts of a candidate's work are warps, and
@@ -451,7 +442,6 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
         if (tid == 0) surv[m] = kKeySentinel;
         __syncthreads();
         nout = min(m, max_det);
-        write_full_lists();
         // the survivors' order by counting among themselves
         const int mwords = max((m + 31) >> 5, 1);
         const int q = (warp % mwords) * 32 + lane, mpart = warp / mwords, mparts = min((NT / 32) / mwords, 4);
@@ -771,7 +761,6 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
         // (a box slot is twice a key, and total <= cnt: the padded list, its ranks and the ordered list fit)
         if (tid == 0) packed[total] = kKeySentinel;
         nout = min(total, max_det);
-        write_full_lists();
         const int mwords = max((total + 31) >> 5, 1);
         if (2 * mwords <= NT / 32) {
             int* const rank = reinterpret_cast<int*>(keys);  // (dead as well once packed)
@@ -838,6 +827,9 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
     }
     if (tid == NT - 1) {
         P.counts[img] = nout;
+        // a branch that takes every class has no index list: item j of an image is its detection j
+        for (int b = 0; b < P.num_branches; ++b)
+            if ((P.full_branches >> b) & 1) P.bcount[b * P.max_batch + img] = nout;
         atomicAdd(&P.ctr->kept, (unsigned long long)nout);
     }
     // ---- index lists of the other branches, filtered by class (stable), one warp per branch ----

@@ -64,7 +64,7 @@ queue_push_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* 
             if (s_off[mid] <= item) lo = mid; else hi = mid;
         }
         const int f = lo;
-        const int det = bidx[(size_t)f * max_det + (item - s_off[f])];
+        const int det = bidx ? bidx[(size_t)f * max_det + (item - s_off[f])] : item - s_off[f];
         const octo_det_t d = dets[(size_t)f * max_det + det];
         const FrameDesc fd = gtab ? gtab[f] : tab.f[f];
         // outward-rounded rectangle, clamped so that it is never empty
@@ -130,7 +130,9 @@ static cudaError_t push_cap(const octo_stage* st, int branch, QRecord* ring, int
     return launch_kernel(queue_push_kernel<CAP>, dim3(1), dim3(kQueueThreads), 0, stream, pdl, tab,
                          st->tab_on_device ? st->d_tab : (const FrameDesc*)nullptr, st->n_frames, c.max_det,
                          st->d_bcount + (size_t)branch * c.max_batch,
-                         st->d_bidx + (size_t)branch * c.max_batch * c.max_det, st->d_dets, ring, cap, state, pdl ? 1 : 0);
+                         (st->full_branches >> branch) & 1 ? (const int*)nullptr
+                                                           : st->d_bidx + (size_t)branch * c.max_batch * c.max_det,
+                         st->d_dets, ring, cap, state, pdl ? 1 : 0);
 }
 
 }  // namespace octo

@@ -155,6 +155,11 @@ extern "C" int octo_stage_create(const octo_stage_config_t* cfg, octo_stage_t** 
     while (ks < cfg->num_anchors) ks <<= 1;
     if (cfg->multi_label) ks <<= 1;  // an anchor can yield several candidates
     st->key_stride = ks;
+    for (int b = 0; b < cfg->num_branches; ++b) {
+        bool full = true;
+        for (int k = 0; k < cfg->num_classes; ++k) full = full && ((cfg->branch[b].class_mask[k >> 5] >> (k & 31)) & 1u);
+        if (full) st->full_branches |= 1 << b;
+    }
 
     const size_t mb = (size_t)cfg->max_batch;
     if (e == cudaSuccess) e = dev_alloc(&st->d_keys, mb * ks, &st->workspace_bytes);
@@ -444,6 +449,7 @@ extern "C" int octo_postprocess_batch(octo_stage_t* st, const float* d_head, int
     a.class_agnostic = c.class_agnostic;
     memset(&a.masks, 0, sizeof(a.masks));
     for (int b = 0; b < c.num_branches; ++b) memcpy(a.masks.m[b], c.branch[b].class_mask, sizeof(uint32_t) * 4);
+    a.full_branches = st->full_branches;
     a.d_bcount = st->d_bcount;
     a.d_bidx = st->d_bidx;
     a.max_batch = c.max_batch;
@@ -508,7 +514,7 @@ extern "C" int octo_crop_batch(octo_stage_t* st, int32_t branch, int32_t first_i
     a.first_item = first_item;
     a.max_items = max_items;
     a.d_bcount = st->d_bcount + (size_t)branch * c.max_batch;
-    a.d_bidx = st->d_bidx + (size_t)branch * c.max_batch * c.max_det;
+    a.d_bidx = (st->full_branches >> branch) & 1 ? nullptr : st->d_bidx + (size_t)branch * c.max_batch * c.max_det;
     a.d_dets = st->d_dets;
     a.d_offsets = d_offsets;
     a.d_n_items = d_n_items;

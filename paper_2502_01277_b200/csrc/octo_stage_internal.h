@@ -11,6 +11,7 @@ struct octo_stage {
     octo_stage_config_t cfg;
     int sm_count;
     int key_stride;  // candidate slots per image: next power of two >= A
+    int full_branches;  // bit b: branch b takes every class (it needs no index list)
     // device workspace
     unsigned long long* d_keys;
     float4* d_boxes;
