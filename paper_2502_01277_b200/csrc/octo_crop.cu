@@ -684,7 +684,7 @@ static cudaError_t launch_crop_cap(const CropArgs& a, cudaStream_t stream) {
                          a.max_det, a.first_item, a.max_items, a.d_bcount, a.d_bidx, a.d_dets, a.d_offsets, a.d_n_items,
                          a.d_items, reinterpret_cast<__half*>(a.d_out), a.out_w, a.out_h, a.swap_rb, a.d_ctr,
                          (const QRecord*)nullptr, (const int*)nullptr, (unsigned int*)nullptr, a.d_ctr->sched, a.opts,
-                         a.pdl ? 1 : 0);
+                         a.early ? 1 : 0);
 }
 
 cudaError_t prepare_crop() {

@@ -435,7 +435,7 @@ static cudaError_t launch_planes_split(const DecodeArgs& a, int mode, float pre,
     dim3 grid((a.A + 32 * VEC * AW - 1) / (32 * VEC * AW), a.n);
     auto kernel = a.multi_label ? decode_planes_kernel<VEC, AW, true> : decode_planes_kernel<VEC, AW, false>;
     return launch_kernel(kernel, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, pre,
-                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, a.pdl ? 1 : 0);
+                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, a.early ? 1 : 0);
 }
 
 // Warps side by side along the anchors, by the number of CTAs that gives (see decode_planes_kernel).
@@ -449,7 +449,7 @@ static cudaError_t launch_planes(const DecodeArgs& a, int mode, float pre, cudaS
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
     // d_cand_count is zero on entry: zeroed at stage creation and re-zeroed by the NMS kernel.
     const int mode = (a.logits ? 1 : 0) | (a.class_agnostic ? 2 : 0) | (a.multi_label ? 4 : 0);
-    const int pdl = a.pdl ? 1 : 0;
+    const int pdl = a.early ? 1 : 0;
     if (a.layout == OCTO_HEAD_PLANES) {
         // Multi-label prefilter in the head's own units: for probabilities the threshold itself;
         // for logits the threshold's logit lowered by a margin that dwarfs the few-ulp error of

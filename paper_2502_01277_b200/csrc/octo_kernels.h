@@ -26,13 +26,15 @@ struct DecodeArgs {
     float4* d_boxes;  // box of every candidate, at its key's slot
     int* d_cand_count;
     unsigned int* d_status;
-    bool pdl;  // launch with programmatic stream serialisation (small batches)
+    bool pdl;    // launch with programmatic stream serialisation
+    bool early;  // ... and let the next kernel be scheduled right away (small batches)
 };
 
 struct NmsArgs {
     const FrameDesc* frames;  // host
     const FrameDesc* d_tab;   // device-resident frame table of a chained stage, or null
-    bool pdl;                 // launch with programmatic stream serialisation (small batches)
+    bool pdl;                 // launch with programmatic stream serialisation
+    bool early;               // ... and let the next kernel be scheduled right away (small batches)
     int n;
     const float* d_head;
     int A, C;
@@ -74,7 +76,8 @@ struct CropOpts {
 struct CropArgs {
     const FrameDesc* frames;  // host
     const FrameDesc* d_tab;   // device-resident frame table of a chained stage, or null
-    bool pdl;                 // launch with programmatic stream serialisation (small batches)
+    bool pdl;                 // launch with programmatic stream serialisation
+    bool early;               // ... and let the next kernel be scheduled right away (small batches)
     int n;
     int max_det, first_item, max_items;
     const int* d_bcount;  // this branch's [max_batch]
@@ -106,7 +109,7 @@ cudaError_t prepare_nms(int* max_cluster = nullptr);
 cudaError_t prepare_crop();
 
 cudaError_t launch_letterbox(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                             int swap_rb, unsigned int* d_status, bool pdl, cudaStream_t stream);
+                             int swap_rb, unsigned int* d_status, bool early, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream);
 cudaError_t launch_nms(const NmsArgs& a, cudaStream_t stream);
 cudaError_t launch_crop(const CropArgs& a, cudaStream_t stream);  // batch assembler + crop-resize
@@ -116,8 +119,8 @@ cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int
 
 constexpr int kLetterboxMaxWidth = 8192;  // widest frame the row staging supports
 
-// Batches up to this size are launched with programmatic dependent launch (see pdl_enter).
-constexpr int kPdlMaxBatch = 16;
+// The kernels of batches up to this size let their successor be scheduled right away (see pdl_enter).
+constexpr int kEarlyMaxBatch = 16;
 
 // One kernel launch; with `pdl` the launch carries the programmatic stream serialisation
 // attribute, so the kernel may be scheduled while its predecessor in the stream still runs (it

@@ -102,7 +102,7 @@ static cudaError_t launch_cap(const NmsArgs& a, cudaStream_t stream) {
     }
     return launch_kernel_cluster(kernel, dim3((unsigned)(a.n * cluster)), dim3(half ? kNmsThreadsHalf : kNmsThreadsFull),
                                  half ? kNmsSmemBytesHalf : kNmsSmemBytes, stream, a.pdl,
-                                 cluster, tab, a.d_tab, nms_params(a), a.pdl ? 1 : 0);
+                                 cluster, tab, a.d_tab, nms_params(a), a.early ? 1 : 0);
 }
 
 cudaError_t launch_nms(const NmsArgs& a, cudaStream_t stream) {

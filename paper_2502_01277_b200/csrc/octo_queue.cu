@@ -126,13 +126,12 @@ static cudaError_t push_cap(const octo_stage* st, int branch, QRecord* ring, int
     if (!st->tab_on_device)
         for (int i = 0; i < st->n_frames; ++i) tab.f[i] = st->frames[i];
     const octo_stage_config_t& c = st->cfg;
-    const bool pdl = st->n_frames <= kPdlMaxBatch;
-    return launch_kernel(queue_push_kernel<CAP>, dim3(1), dim3(kQueueThreads), 0, stream, pdl, tab,
+    return launch_kernel(queue_push_kernel<CAP>, dim3(1), dim3(kQueueThreads), 0, stream, true, tab,
                          st->tab_on_device ? st->d_tab : (const FrameDesc*)nullptr, st->n_frames, c.max_det,
                          st->d_bcount + (size_t)branch * c.max_batch,
                          (st->full_branches >> branch) & 1 ? (const int*)nullptr
                                                            : st->d_bidx + (size_t)branch * c.max_batch * c.max_det,
-                         st->d_dets, ring, cap, state, pdl ? 1 : 0);
+                         st->d_dets, ring, cap, state, st->n_frames <= kEarlyMaxBatch ? 1 : 0);
 }
 
 }  // namespace octo

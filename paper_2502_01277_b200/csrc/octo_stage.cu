@@ -259,7 +259,7 @@ extern "C" int octo_preprocess_batch(octo_stage_t* st, const octo_frame_t* frame
     {
         ScopedKernelTimer t(st, OCTO_K_LETTERBOX, static_cast<cudaStream_t>(cuda_stream));
         OCTO_CUDA(launch_letterbox(st->frames, n, d_out_f16_nchw, st->cfg.net_size, max_w, st->cfg.pad_value,
-                                   st->cfg.swap_rb, &st->d_ctr->status, n <= kPdlMaxBatch,
+                                   st->cfg.swap_rb, &st->d_ctr->status, n <= kEarlyMaxBatch,
                                    static_cast<cudaStream_t>(cuda_stream)));
     }
     st->launches += 1;
@@ -344,7 +344,7 @@ static cudaError_t launch_adopt(const octo_stage* up, const octo_item_t* d_items
     FrameTable<CAP> tab;
     if (!up->tab_on_device)
         for (int i = 0; i < up->n_frames; ++i) tab.f[i] = up->frames[i];
-    return launch_kernel(adopt_items_kernel<CAP>, dim3((n + 255) / 256), dim3(256), 0, stream, false, tab,
+    return launch_kernel(adopt_items_kernel<CAP>, dim3((n + 255) / 256), dim3(256), 0, stream, true, tab,
                          up->tab_on_device ? up->d_tab : (const FrameDesc*)nullptr, d_items, d_n_items, first, n, S,
                          d_out);
 }
@@ -424,14 +424,16 @@ extern "C" int octo_postprocess_batch(octo_stage_t* st, const float* d_head, int
         da.conf = c.conf_thresh;
         da.key_stride = st->key_stride;
         da.d_keys = st->d_keys; da.d_boxes = st->d_boxes; da.d_cand_count = st->d_cand_count; da.d_status = &st->d_ctr->status;
-        da.pdl = n <= kPdlMaxBatch;
+        da.pdl = true;
+        da.early = n <= kEarlyMaxBatch;
         OCTO_CUDA(launch_decode(da, stream));
     }
     st->launches += 1;
     NmsArgs a;
     a.frames = st->frames;
     a.d_tab = st->tab_on_device ? st->d_tab : nullptr;
-    a.pdl = n <= kPdlMaxBatch;
+    a.pdl = true;
+    a.early = n <= kEarlyMaxBatch;
     a.n = n;
     a.d_head = d_head;
     a.A = c.num_anchors;
@@ -508,7 +510,8 @@ extern "C" int octo_crop_batch(octo_stage_t* st, int32_t branch, int32_t first_i
     CropArgs a;
     a.frames = st->frames;
     a.d_tab = st->tab_on_device ? st->d_tab : nullptr;
-    a.pdl = st->n_frames <= kPdlMaxBatch;
+    a.pdl = true;
+    a.early = st->n_frames <= kEarlyMaxBatch;
     a.n = st->n_frames;
     a.max_det = c.max_det;
     a.first_item = first_item;
