@@ -59,19 +59,15 @@ struct StageCounters {
 #define OCTO_IN_RANGE(cond, status_ptr) (true)
 #endif
 
-// Programmatic dependent launch.  Every kernel of the library starts with pdl_enter: it waits
-// until the kernel before it in the stream has completed and its writes are visible (a no-op
-// for a launch without the programmatic attribute).  The stage launches all its kernels with that
-// attribute: even when nothing is signalled early, the successor's launch then overlaps the end of
-// its predecessor (32 planes-layout frames 230 -> 222 us per pass, a two-level cascade 180 -> 174.5, 64
-// frames with two branches 446 -> 440).  With `early` set a kernel lets the next one be scheduled as
-// soon as all its CTAs run; the host sets it for small batches only: there the launch latency between
-// the kernels of a pass is most of the pass, while a large grid loses more to the waiting CTAs of its
-// successor than it gains (256 frames 1180 -> 1230 us).
-__device__ __forceinline__ void pdl_enter(int early) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// Programmatic dependent launch.  Every kernel of the library is launched with the programmatic
+// attribute and starts with pdl_wait: until then the kernel before it in the stream may still be
+// running, after it that kernel has completed and its writes are visible.  What this hides is the launch
+// latency at the end of the predecessor (32 planes-layout frames 230 -> 222 us per pass, 64 frames with
+// two branches 446 -> 440).  No kernel signals its successor before its own end: CTAs that wait at
+// pdl_wait take room and time from the ones that work (with a signal at the start of each kernel of a small
+// batch: one 320x240 frame 19.4 against 18.5 us per pass, one camera 28.4 / 27.1, eight 62.1 / 58.3,
+// twelve 100 / 86.5, a two-level cascade 174 / 162).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 constexpr int kKeyAnchorBits = 25;  // anchor index field of a candidate key
 constexpr unsigned long long kKeySentinel = ~0ull;

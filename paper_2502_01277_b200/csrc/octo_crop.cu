@@ -127,9 +127,9 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             int* __restrict__ offsets, int* __restrict__ n_items, octo_item_t* __restrict__ items,
             __half* __restrict__ out, int ow, int oh, int swap_rb, StageCounters* __restrict__ ctr,
             const QRecord* __restrict__ qrec, const int* __restrict__ qpacked, unsigned int* __restrict__ qstatus,
-            int* __restrict__ sched, const CropOpts opts, int pdl) {
+            int* __restrict__ sched, const CropOpts opts) {
     extern __shared__ __align__(128) unsigned char smem[];
-    pdl_enter(pdl);
+    pdl_wait();
     __shared__ __align__(8) uint64_t full[kCropStages], empty[kCropStages];
     __shared__ CropPass s_pass[kCropStages];
     __shared__ __align__(16) RowInfo s_row[kCropStages][kCropMaxPassRows];  // per-row data of the staged passes
@@ -680,11 +680,10 @@ static cudaError_t launch_crop_cap(const CropArgs& a, cudaStream_t stream) {
     const int grid = crop_grid(a.sm_count, a.max_items, a.out_h);
     const size_t smem = crop_smem_bytes(a.out_w);
     auto kernel = a.general ? crop_kernel<CAP, false, true> : crop_kernel<CAP, false, false>;
-    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, a.pdl, tab, a.d_tab, a.n,
+    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, tab, a.d_tab, a.n,
                          a.max_det, a.first_item, a.max_items, a.d_bcount, a.d_bidx, a.d_dets, a.d_offsets, a.d_n_items,
                          a.d_items, reinterpret_cast<__half*>(a.d_out), a.out_w, a.out_h, a.swap_rb, a.d_ctr,
-                         (const QRecord*)nullptr, (const int*)nullptr, (unsigned int*)nullptr, a.d_ctr->sched, a.opts,
-                         a.early ? 1 : 0);
+                         (const QRecord*)nullptr, (const int*)nullptr, (unsigned int*)nullptr, a.d_ctr->sched, a.opts);
 }
 
 cudaError_t prepare_crop() {
@@ -724,11 +723,11 @@ cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int
     memset(&opts, 0, sizeof(opts));
     if (general) opts = *general;
     auto kernel = general ? crop_kernel<1, true, true> : crop_kernel<1, true, false>;
-    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, true, tab,
+    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, tab,
                          (const FrameDesc*)nullptr, 0, 0, 0, bz, (const int*)nullptr, (const int*)nullptr,
                          (const octo_det_t*)nullptr, (int*)nullptr, (int*)nullptr, (octo_item_t*)nullptr,
                          reinterpret_cast<__half*>(d_out), out_w, out_h, swap_rb, (StageCounters*)nullptr, d_staged,
-                         d_qpacked, d_status, d_sched, opts, 1);
+                         d_qpacked, d_status, d_sched, opts);
 }
 
 }  // namespace octo

@@ -48,8 +48,8 @@ template <int kDecPerThread>
 __global__ void __launch_bounds__(kDecThreads, kDecPerThread == 1 ? 5 : 6)
 decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, int key_stride,
               unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
-              unsigned int* __restrict__ status, int pdl) {
-    pdl_enter(pdl);
+              unsigned int* __restrict__ status) {
+    pdl_wait();
     // mode bit 0: obj / class values are logits; bit 1: class-agnostic NMS (key class field 0);
     // bit 2: multi-label candidates
     const int logits = mode & 1;
@@ -206,8 +206,8 @@ template <int VEC, int AW, bool MULTI>
 __global__ void __launch_bounds__(kDecThreads)
 decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, float pre, int key_stride,
                      unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
-                     unsigned int* __restrict__ status, int pdl) {
-    pdl_enter(pdl);
+                     unsigned int* __restrict__ status) {
+    pdl_wait();
     constexpr int CW = kDecThreads / 32 / AW;
     constexpr int kCtaAnchors = AW * 32 * VEC;
     __shared__ float s_best[CW][kCtaAnchors];
@@ -360,10 +360,10 @@ constexpr int kDenseRows = 128;
 __global__ void __launch_bounds__(kDenseRows)
 decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, int key_stride,
                     unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
-                    unsigned int* __restrict__ status, int pdl) {
+                    unsigned int* __restrict__ status) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(8) uint64_t bar;
-    pdl_enter(pdl);
+    pdl_wait();
     const bool agnostic = (mode & 2) != 0;
     const bool multi = (mode & 4) != 0;
     const int img = blockIdx.y, t = threadIdx.x;
@@ -434,8 +434,8 @@ template <int VEC, int AW>
 static cudaError_t launch_planes_split(const DecodeArgs& a, int mode, float pre, cudaStream_t stream) {
     dim3 grid((a.A + 32 * VEC * AW - 1) / (32 * VEC * AW), a.n);
     auto kernel = a.multi_label ? decode_planes_kernel<VEC, AW, true> : decode_planes_kernel<VEC, AW, false>;
-    return launch_kernel(kernel, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, pre,
-                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, a.early ? 1 : 0);
+    return launch_kernel(kernel, grid, dim3(kDecThreads), 0, stream, a.d_head, a.A, a.C, mode, a.conf, pre,
+                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status);
 }
 
 // Warps side by side along the anchors, by the number of CTAs that gives (see decode_planes_kernel).
@@ -449,7 +449,6 @@ static cudaError_t launch_planes(const DecodeArgs& a, int mode, float pre, cudaS
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
     // d_cand_count is zero on entry: zeroed at stage creation and re-zeroed by the NMS kernel.
     const int mode = (a.logits ? 1 : 0) | (a.class_agnostic ? 2 : 0) | (a.multi_label ? 4 : 0);
-    const int pdl = a.early ? 1 : 0;
     if (a.layout == OCTO_HEAD_PLANES) {
         // Multi-label prefilter in the head's own units: for probabilities the threshold itself;
         // for logits the threshold's logit lowered by a margin that dwarfs the few-ulp error of
@@ -470,18 +469,18 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
         // by the row groups of decode_kernel)
         dim3 grid((a.A + kDenseRows - 1) / kDenseRows, a.n);
         return launch_kernel(decode_dense_kernel, grid, dim3(kDenseRows), sizeof(float) * kDenseRows * (5 + (size_t)a.C),
-                             stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count,
-                             a.d_status, pdl);
+                             stream, a.d_head, a.A, a.C, mode, a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count,
+                             a.d_status);
     }
     const int per_cta4 = kDecThreads * 4;
     if ((long long)a.n * ((a.A + per_cta4 - 1) / per_cta4) >= 296) {
         dim3 grid((a.A + per_cta4 - 1) / per_cta4, a.n);
-        return launch_kernel(decode_kernel<4>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode,
-                             a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, pdl);
+        return launch_kernel(decode_kernel<4>, grid, dim3(kDecThreads), 0, stream, a.d_head, a.A, a.C, mode,
+                             a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status);
     }
     dim3 grid((a.A + kDecThreads - 1) / kDecThreads, a.n);
-    return launch_kernel(decode_kernel<1>, grid, dim3(kDecThreads), 0, stream, a.pdl, a.d_head, a.A, a.C, mode, a.conf,
-                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status, pdl);
+    return launch_kernel(decode_kernel<1>, grid, dim3(kDecThreads), 0, stream, a.d_head, a.A, a.C, mode, a.conf,
+                         a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status);
 }
 
 }  // namespace octo

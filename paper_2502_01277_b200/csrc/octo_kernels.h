@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "octo.h"
 #include "octo_common.cuh"
 
@@ -26,15 +28,11 @@ struct DecodeArgs {
     float4* d_boxes;  // box of every candidate, at its key's slot
     int* d_cand_count;
     unsigned int* d_status;
-    bool pdl;    // launch with programmatic stream serialisation
-    bool early;  // ... and let the next kernel be scheduled right away (small batches)
 };
 
 struct NmsArgs {
     const FrameDesc* frames;  // host
     const FrameDesc* d_tab;   // device-resident frame table of a chained stage, or null
-    bool pdl;                 // launch with programmatic stream serialisation
-    bool early;               // ... and let the next kernel be scheduled right away (small batches)
     int n;
     const float* d_head;
     int A, C;
@@ -76,8 +74,6 @@ struct CropOpts {
 struct CropArgs {
     const FrameDesc* frames;  // host
     const FrameDesc* d_tab;   // device-resident frame table of a chained stage, or null
-    bool pdl;                 // launch with programmatic stream serialisation
-    bool early;               // ... and let the next kernel be scheduled right away (small batches)
     int n;
     int max_det, first_item, max_items;
     const int* d_bcount;  // this branch's [max_batch]
@@ -109,7 +105,7 @@ cudaError_t prepare_nms(int* max_cluster = nullptr);
 cudaError_t prepare_crop();
 
 cudaError_t launch_letterbox(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                             int swap_rb, unsigned int* d_status, bool early, cudaStream_t stream);
+                             int swap_rb, unsigned int* d_status, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream);
 cudaError_t launch_nms(const NmsArgs& a, cudaStream_t stream);
 cudaError_t launch_crop(const CropArgs& a, cudaStream_t stream);  // batch assembler + crop-resize
@@ -119,32 +115,12 @@ cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int
 
 constexpr int kLetterboxMaxWidth = 8192;  // widest frame the row staging supports
 
-// The kernels of batches up to this size let their successor be scheduled right away (see pdl_enter).
-constexpr int kEarlyMaxBatch = 16;
-
-// One kernel launch; with `pdl` the launch carries the programmatic stream serialisation
-// attribute, so the kernel may be scheduled while its predecessor in the stream still runs (it
-// waits for that predecessor in pdl_enter before it touches memory).
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                 bool pdl, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1u : 0u;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
-// The same with a thread-block cluster of `cluster` CTAs along x (grid.x is a multiple of it).
+// One kernel launch with the programmatic stream serialisation attribute: the kernel may be scheduled
+// while its predecessor in the stream ends (it waits for it in pdl_wait before it touches memory).  With
+// `cluster` > 1, thread-block clusters of that many CTAs along x (grid.x is a multiple of it).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
-                                         cudaStream_t stream, bool pdl, int cluster, Args&&... args) {
+                                         cudaStream_t stream, int cluster, Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -152,6 +128,9 @@ inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, di
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     unsigned na = 0;
+    attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
     if (cluster > 1) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
         attr[na].val.clusterDim.x = (unsigned)cluster;
@@ -159,14 +138,15 @@ inline cudaError_t launch_kernel_cluster(void (*kernel)(KArgs...), dim3 grid, di
         attr[na].val.clusterDim.z = 1;
         ++na;
     }
-    if (pdl) {
-        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[na].val.programmaticStreamSerializationAllowed = 1;
-        ++na;
-    }
     cfg.attrs = attr;
     cfg.numAttrs = na;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                 Args&&... args) {
+    return launch_kernel_cluster(kernel, grid, block, smem, stream, 1, std::forward<Args>(args)...);
 }
 
 }  // namespace octo

@@ -20,10 +20,9 @@ constexpr int kLbRows = 8;  // most output rows a CTA produces; fewer for very w
 template <int CAP>
 __global__ void __launch_bounds__(kLbThreads)
 letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict__ out, int S, int band_rows,
-                 int slot_bytes, int nslots, uint32_t fill_h2, int swap_rb, unsigned int* __restrict__ status,
-                 int pdl) {
+                 int slot_bytes, int nslots, uint32_t fill_h2, int swap_rb, unsigned int* __restrict__ status) {
     extern __shared__ __align__(128) unsigned char smem[];
-    pdl_enter(pdl);
+    pdl_wait();
     __shared__ __align__(8) uint64_t bar;
     __shared__ __align__(16) RowInfo s_row[kLbRows];  // per-row data; step < 0 marks a canvas (pad) row
 
@@ -159,7 +158,7 @@ static size_t lb_smem_bytes(int S, int slots, int slot_bytes) {
 
 template <int CAP>
 static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                              int swap_rb, unsigned int* d_status, bool early, cudaStream_t stream) {
+                              int swap_rb, unsigned int* d_status, cudaStream_t stream) {
     FrameTable<CAP> tab;  // built per call (copied into kernel parameter space by the launch)
     for (int i = 0; i < n; ++i) tab.f[i] = frames[i];
     const int slot_bytes = ((3 * max_w + 15) & ~15) + 16;  // 16 bytes of slack: a tap reads 12 bytes from its word
@@ -176,9 +175,9 @@ static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S
     const uint32_t fb = *reinterpret_cast<const unsigned short*>(&hf);
     const uint32_t fill_h2 = fb | (fb << 16);
     dim3 grid((S + band_rows - 1) / band_rows, n);
-    return launch_kernel(letterbox_kernel<CAP>, grid, dim3(kLbThreads), smem, stream, true, tab,
+    return launch_kernel(letterbox_kernel<CAP>, grid, dim3(kLbThreads), smem, stream, tab,
                          reinterpret_cast<__half*>(d_out), S, band_rows, slot_bytes,
-                         band_rows * slots_per_row(frames, n), fill_h2, swap_rb, d_status, early ? 1 : 0);
+                         band_rows * slots_per_row(frames, n), fill_h2, swap_rb, d_status);
 }
 
 // largest dynamic shared memory a launch may ask for (see kLetterboxMaxWidth)
@@ -194,10 +193,10 @@ cudaError_t prepare_letterbox() {
 }
 
 cudaError_t launch_letterbox(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                             int swap_rb, unsigned int* d_status, bool early, cudaStream_t stream) {
-    if (n <= 8) return launch_cap<8>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, early, stream);
-    if (n <= 64) return launch_cap<64>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, early, stream);
-    return launch_cap<512>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, early, stream);
+                             int swap_rb, unsigned int* d_status, cudaStream_t stream) {
+    if (n <= 8) return launch_cap<8>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, stream);
+    if (n <= 64) return launch_cap<64>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, stream);
+    return launch_cap<512>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, stream);
 }
 
 }  // namespace octo

@@ -9,13 +9,13 @@ namespace octo {
 template <int CAP, int NT>
 __global__ void __launch_bounds__(NT, kNmsThreadsFull / NT)
 nms_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __restrict__ gtab,
-           const __grid_constant__ NmsParams params, int pdl) {
+           const __grid_constant__ NmsParams params) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // fetch the parameters' constant-cache lines while the launch waits for its predecessor
     asm volatile("" ::"l"(params.bidx), "l"(params.bcount), "l"(params.counts), "l"(params.dets), "l"(params.gkeys),
                  "l"(params.ctr), "r"(params.masks.m[0][0]), "r"(params.launch_seq), "r"(params.num_branches),
                  "f"(tab.f[0].gx), "r"(tab.f[0].w));
-    pdl_enter(pdl);
+    pdl_wait();
     constexpr bool kCluster = NT == kNmsThreadsFull;  // half-sized CTAs never form clusters
     const int img = (int)(blockIdx.x / (kCluster ? cg::this_cluster().num_blocks() : 1u));
     // The frame table comes by value (first-level stages) or from device memory (chained stages,
@@ -101,8 +101,8 @@ static cudaError_t launch_cap(const NmsArgs& a, cudaStream_t stream) {
         if (half) kernel = nms_kernel<512, kNmsThreadsHalf>;
     }
     return launch_kernel_cluster(kernel, dim3((unsigned)(a.n * cluster)), dim3(half ? kNmsThreadsHalf : kNmsThreadsFull),
-                                 half ? kNmsSmemBytesHalf : kNmsSmemBytes, stream, a.pdl,
-                                 cluster, tab, a.d_tab, nms_params(a), a.early ? 1 : 0);
+                                 half ? kNmsSmemBytesHalf : kNmsSmemBytes, stream,
+                                 cluster, tab, a.d_tab, nms_params(a));
 }
 
 cudaError_t launch_nms(const NmsArgs& a, cudaStream_t stream) {

@@ -145,8 +145,6 @@ extern "C" int octo_postprocess_frame_static(int32_t device, const float* d_head
     da.conf = conf_thresh;
     da.key_stride = key_stride;
     da.d_keys = d_keys; da.d_boxes = d_boxes; da.d_cand_count = d_cand; da.d_status = &d_ctr->status;
-    da.pdl = false;
-    da.early = false;
     e = launch_decode(da, stream);
     if (e != cudaSuccess) return report_cuda_error(e, "decode_kernel");
 
@@ -155,8 +153,6 @@ extern "C" int octo_postprocess_frame_static(int32_t device, const float* d_head
     NmsArgs a;
     a.frames = &fd;
     a.d_tab = nullptr;
-    a.pdl = false;
-    a.early = false;
     a.n = 1;
     a.d_head = d_head;
     a.A = num_anchors;

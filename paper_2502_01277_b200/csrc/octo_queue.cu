@@ -31,9 +31,9 @@ __global__ void __launch_bounds__(kQueueThreads)
 queue_push_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __restrict__ gtab, int n, int max_det,
                   const int* __restrict__ bcount,
                   const int* __restrict__ bidx, const octo_det_t* __restrict__ dets, QRecord* __restrict__ ring,
-                  int cap, QueueState* __restrict__ state, int pdl) {
+                  int cap, QueueState* __restrict__ state) {
     __shared__ int s_off[CAP + 1];
-    pdl_enter(pdl);
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (warp == 0) {
         int run = 0;
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(256)
 queue_pop_kernel(const QRecord* __restrict__ ring, int cap, QueueState* __restrict__ state, int bz, int max_wait,
                  QRecord* __restrict__ staged, QRecord* __restrict__ items_out, int* __restrict__ info,
                  int* __restrict__ qpacked) {
-    pdl_enter(1);
+    pdl_wait();
     const long long head = state->head, tail = state->tail;
     const long long pending = tail - head;
     // max_wait < 0: release whatever is pending.  Otherwise a batch is released when it is full, or
@@ -126,12 +126,12 @@ static cudaError_t push_cap(const octo_stage* st, int branch, QRecord* ring, int
     if (!st->tab_on_device)
         for (int i = 0; i < st->n_frames; ++i) tab.f[i] = st->frames[i];
     const octo_stage_config_t& c = st->cfg;
-    return launch_kernel(queue_push_kernel<CAP>, dim3(1), dim3(kQueueThreads), 0, stream, true, tab,
+    return launch_kernel(queue_push_kernel<CAP>, dim3(1), dim3(kQueueThreads), 0, stream, tab,
                          st->tab_on_device ? st->d_tab : (const FrameDesc*)nullptr, st->n_frames, c.max_det,
                          st->d_bcount + (size_t)branch * c.max_batch,
                          (st->full_branches >> branch) & 1 ? (const int*)nullptr
                                                            : st->d_bidx + (size_t)branch * c.max_batch * c.max_det,
-                         st->d_dets, ring, cap, state, st->n_frames <= kEarlyMaxBatch ? 1 : 0);
+                         st->d_dets, ring, cap, state);
 }
 
 }  // namespace octo
@@ -230,9 +230,7 @@ extern "C" int octo_queue_pop_due(octo_queue_t* q, int32_t bz, int32_t max_wait,
     if (cudaSetDevice(q->device) != cudaSuccess) return OCTO_E_CUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     static_assert(sizeof(octo_qitem_t) == sizeof(QRecord), "public and internal queue records match");
-    // One CTA, then the crops: both are launched ahead of their predecessor's end (pdl_enter), which hides
-    // two launch latencies per pop (two cameras, bz = 64: 43.3 -> 39.0 us per pass).
-    cudaError_t e = launch_kernel(queue_pop_kernel, dim3(1), dim3(256), 0, stream, true, q->d_ring, q->capacity, q->d_state,
+    cudaError_t e = launch_kernel(queue_pop_kernel, dim3(1), dim3(256), 0, stream, q->d_ring, q->capacity, q->d_state,
                                   bz, max_wait, q->d_staged, reinterpret_cast<QRecord*>(d_items_out), d_info, q->d_qpacked);
     if (e != cudaSuccess) return OCTO_E_CUDA;
     e = launch_crop_queue(q->d_staged, q->d_qpacked, bz, d_out_f16, q->out_w, q->out_h, q->swap_rb,

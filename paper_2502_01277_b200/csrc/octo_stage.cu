@@ -259,7 +259,7 @@ extern "C" int octo_preprocess_batch(octo_stage_t* st, const octo_frame_t* frame
     {
         ScopedKernelTimer t(st, OCTO_K_LETTERBOX, static_cast<cudaStream_t>(cuda_stream));
         OCTO_CUDA(launch_letterbox(st->frames, n, d_out_f16_nchw, st->cfg.net_size, max_w, st->cfg.pad_value,
-                                   st->cfg.swap_rb, &st->d_ctr->status, n <= kEarlyMaxBatch,
+                                   st->cfg.swap_rb, &st->d_ctr->status,
                                    static_cast<cudaStream_t>(cuda_stream)));
     }
     st->launches += 1;
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(256)
 adopt_items_kernel(const __grid_constant__ FrameTable<CAP> up_tab, const FrameDesc* __restrict__ up_gtab,
                    const octo_item_t* __restrict__ items, const int* __restrict__ up_n_items, int first, int n, int S,
                    FrameDesc* __restrict__ out) {
-    pdl_enter(0);
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     FrameDesc fd;
@@ -344,7 +344,7 @@ static cudaError_t launch_adopt(const octo_stage* up, const octo_item_t* d_items
     FrameTable<CAP> tab;
     if (!up->tab_on_device)
         for (int i = 0; i < up->n_frames; ++i) tab.f[i] = up->frames[i];
-    return launch_kernel(adopt_items_kernel<CAP>, dim3((n + 255) / 256), dim3(256), 0, stream, true, tab,
+    return launch_kernel(adopt_items_kernel<CAP>, dim3((n + 255) / 256), dim3(256), 0, stream, tab,
                          up->tab_on_device ? up->d_tab : (const FrameDesc*)nullptr, d_items, d_n_items, first, n, S,
                          d_out);
 }
@@ -354,7 +354,7 @@ static cudaError_t launch_adopt(const octo_stage* up, const octo_item_t* d_items
 // returns.  No copy is in flight at any point and the shared memory dies with the CTA.
 __global__ void wait_selftest_kernel(unsigned int* __restrict__ status, int polls) {
     __shared__ __align__(8) uint64_t bar;
-    pdl_enter(0);
+    pdl_wait();
     if (threadIdx.x == 0) {
         mbar_init(&bar, 1);
         mbar_fence_init();
@@ -396,7 +396,7 @@ extern "C" int octo_adopt_items_device(octo_stage_t* st, const octo_stage_t* ups
 extern "C" int octo_stage_selftest_wait(octo_stage_t* st, int32_t polls, void* cuda_stream) {
     if (!st || polls < 1 || polls > (1 << 20)) return OCTO_E_INVALID_ARG;
     OCTO_CUDA(cudaSetDevice(st->cfg.device));
-    OCTO_CUDA(launch_kernel(wait_selftest_kernel, dim3(1), dim3(32), 0, static_cast<cudaStream_t>(cuda_stream), false,
+    OCTO_CUDA(launch_kernel(wait_selftest_kernel, dim3(1), dim3(32), 0, static_cast<cudaStream_t>(cuda_stream),
                             &st->d_ctr->status, (int)polls));
     st->launches += 1;
     return OCTO_OK;
@@ -424,16 +424,12 @@ extern "C" int octo_postprocess_batch(octo_stage_t* st, const float* d_head, int
         da.conf = c.conf_thresh;
         da.key_stride = st->key_stride;
         da.d_keys = st->d_keys; da.d_boxes = st->d_boxes; da.d_cand_count = st->d_cand_count; da.d_status = &st->d_ctr->status;
-        da.pdl = true;
-        da.early = n <= kEarlyMaxBatch;
         OCTO_CUDA(launch_decode(da, stream));
     }
     st->launches += 1;
     NmsArgs a;
     a.frames = st->frames;
     a.d_tab = st->tab_on_device ? st->d_tab : nullptr;
-    a.pdl = true;
-    a.early = n <= kEarlyMaxBatch;
     a.n = n;
     a.d_head = d_head;
     a.A = c.num_anchors;
@@ -510,8 +506,6 @@ extern "C" int octo_crop_batch(octo_stage_t* st, int32_t branch, int32_t first_i
     CropArgs a;
     a.frames = st->frames;
     a.d_tab = st->tab_on_device ? st->d_tab : nullptr;
-    a.pdl = true;
-    a.early = st->n_frames <= kEarlyMaxBatch;
     a.n = st->n_frames;
     a.max_det = c.max_det;
     a.first_item = first_item;
