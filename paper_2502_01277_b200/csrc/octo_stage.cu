@@ -176,10 +176,10 @@ extern "C" int octo_stage_create(const octo_stage_config_t* cfg, octo_stage_t** 
     if (e == cudaSuccess) e = prepare_decode();
     if (e == cudaSuccess) e = prepare_nms(&st->nms_max_cluster);
     if (e == cudaSuccess) {
-        // an integer the NMS kernel writes and the host reads without a copy
-        e = cudaHostAlloc(reinterpret_cast<void**>(&st->h_dense_seen), sizeof(int), cudaHostAllocMapped);
+        // two integers the NMS kernel writes and the host reads without a copy
+        e = cudaHostAlloc(reinterpret_cast<void**>(&st->h_dense_seen), 2 * sizeof(int), cudaHostAllocMapped);
         if (e == cudaSuccess) {
-            st->h_dense_seen[0] = -(1 << 30);  // no image with many candidates seen yet
+            st->h_dense_seen[0] = st->h_dense_seen[1] = 0;  // none seen yet (launches count from 1)
             e = cudaHostGetDevicePointer(reinterpret_cast<void**>(&st->d_dense_seen), st->h_dense_seen, 0);
         }
     }
@@ -455,23 +455,30 @@ extern "C" int octo_postprocess_batch(octo_stage_t* st, const float* d_head, int
     // A cluster of CTAs per image while images with many candidates were seen in the kernel's latest
     // launches and the batch is too small to fill the GPU with one CTA per image.
     st->nms_seq += 1;
+    // (the window counts from the launch that finds a new report, not from the one that made it: a host that
+    // runs a hundred launches ahead of the GPU would otherwise see every report too late)
+    bool crowded[2];
+    for (int k = 0; k < 2; ++k) {
+        const int reported = static_cast<const volatile int*>(st->h_dense_seen)[k];
+        if (reported != st->nms_dense_reported[k]) {
+            st->nms_dense_reported[k] = reported;
+            st->nms_dense_until[k] = st->nms_seq + kNmsClusterWindow - 1;
+        }
+        crowded[k] = st->nms_seq <= st->nms_dense_until[k];
+    }
     a.cluster = 1;
     a.d_dense_seen = st->d_dense_seen;
     a.launch_seq = st->nms_seq;
     if (st->nms_cluster_mode > 0) {
         a.cluster = st->nms_cluster_mode < st->nms_max_cluster ? st->nms_cluster_mode : st->nms_max_cluster;
-    } else if (st->h_dense_seen) {
-        const int last_dense = *static_cast<const volatile int*>(st->h_dense_seen);
-        if (st->nms_seq - last_dense <= kNmsClusterWindow) {
-            const int want = n * 8 <= st->sm_count ? 8 : n * 4 <= st->sm_count ? 4 : n * 2 <= st->sm_count ? 2 : 1;
-            a.cluster = want < st->nms_max_cluster ? want : st->nms_max_cluster;
-        }
+    } else if (crowded[1]) {
+        const int want = n * 8 <= st->sm_count ? 8 : n * 4 <= st->sm_count ? 4 : n * 2 <= st->sm_count ? 2 : 1;
+        a.cluster = want < st->nms_max_cluster ? want : st->nms_max_cluster;
     }
     st->nms_cluster_last = a.cluster;
     // More images than SMs and no crowded image lately: two half-sized CTAs per SM, one wave.
     // (the half-sized kernel exists for the largest frame-table size only, i.e. for more than 64 images)
-    a.half_ctas = a.cluster == 1 && n > st->sm_count && n > 64 && st->nms_cluster_mode == 0 && st->h_dense_seen &&
-                  st->nms_seq - *static_cast<const volatile int*>(st->h_dense_seen) > kNmsClusterWindow;
+    a.half_ctas = a.cluster == 1 && n > st->sm_count && n > 64 && st->nms_cluster_mode == 0 && !crowded[0];
     st->nms_half_last = a.half_ctas;
     cudaError_t e;
     {

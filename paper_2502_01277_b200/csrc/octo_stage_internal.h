@@ -31,17 +31,19 @@ struct octo_stage {
     const octo_det_t* d_dets;
     const int32_t* d_last_n_items[OCTO_MAX_BRANCHES];  // {packed, total} of the last crop call per branch (caller's buffer)
     int64_t launches;
-    // Cluster size of the NMS launches.  The kernel reports through an integer in mapped host memory
-    // (no copy, no synchronisation) the number of the latest launch that saw an image with many
-    // candidates; for kNmsClusterWindow launches after it (the host may have enqueued many launches
-    // that the GPU has not run yet), launches with few images give every image a cluster of CTAs.
+    // Form of the NMS launches.  The kernel reports through two integers in mapped host memory (no copy, no
+    // synchronisation) the number of the latest launch that saw an image with more than 1024 candidates
+    // ([0]) and with more than the short path takes, 512 ([1]).  For kNmsClusterWindow launches from the one
+    // that finds a report, launches with few images give every image a cluster of CTAs ([1]) and launches
+    // with many keep to full-sized CTAs ([0]).
     int nms_max_cluster;
     int nms_cluster_mode;  // 0 automatic, else the caller's size
     int nms_cluster_last;  // size of the latest launch
     bool nms_half_last;    // the latest launch ran two half-sized CTAs per SM
     int nms_seq;
+    int nms_dense_reported[2], nms_dense_until[2];  // latest report taken note of; last launch it counts for
     int* h_dense_seen;  // host view (volatile reads)
-    int* d_dense_seen;  // device view of the same integer
+    int* d_dense_seen;  // device view of the same integers
     // optional per-kernel timing
     bool timing;
     cudaEvent_t ev[2 * kEventPairs];

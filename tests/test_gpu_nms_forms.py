@@ -1,6 +1,6 @@
 """NMS where its forms meet: candidate counts around a warp, the short path (512, with 4, 2 and 1 threads
-per candidate), a class that the whole CTA takes (128 .. 512 and above, in blocks of 128), the network
-sort (512), the half-sized and the full on-chip capacity; chains of overlapping boxes (as many rounds as
+per candidate), batches of classes, a class that the whole CTA takes (above 512, in blocks of 128), survivors
+ordered by counting (96), in registers and by a network (above 1024), the half-sized and the full on-chip capacity; chains of overlapping boxes (as many rounds as
 links), identical boxes, IoU values that lie exactly on the threshold, a small cap, clusters.  The oracle
 makes the same binary32 decisions, so kept detections are bit-equal."""
 import numpy as np
@@ -22,6 +22,9 @@ def _boxes(rng, m, kind):
         i = np.arange(m)
         per = 60
         return np.stack([8 + 4.0 * (i % per), 6 + 12.0 * ((i // per) % 20), np.full(m, 10.0), np.full(m, 10.0)], 1)
+    if kind == "apart":
+        i = np.arange(m)
+        return np.stack([2 + 5.0 * (i % 48), 2 + 5.0 * (i // 48), np.full(m, 4.0), np.full(m, 4.0)], 1)
     if kind == "same":
         return np.tile(np.array([[100.0, 90.0, 30.0, 20.0]]), (m, 1))
     # a coarse grid of sizes and places: many IoU values are simple fractions, 1/2 among them
@@ -66,8 +69,9 @@ def test_short_path(m, kind, agnostic):
     _check(m, kind, 0.5, agnostic=agnostic)
 
 
-@pytest.mark.parametrize("m,share", [(513, 0.0), (520, 0.4), (640, 1.0), (1024, 0.9), (1030, 1.0), (2100, 0.2),
-                                     (4097, 1.0), (8192, 0.3), (8200, 1.0)])
+@pytest.mark.parametrize("m,share", [(513, 0.0), (520, 0.4), (640, 1.0), (640, 0.8), (1024, 0.5), (1024, 0.9),
+                                     (1030, 1.0), (2100, 0.0), (2100, 0.2), (4097, 1.0), (8192, 0.3), (8200, 1.0),
+                                     (8300, 0.0)])
 @pytest.mark.parametrize("cluster", [1, 4])
 def test_large_classes(m, share, cluster):
     _check(m, "grid", share, cluster=cluster, max_det=1000)
@@ -77,6 +81,12 @@ def test_large_classes(m, share, cluster):
 @pytest.mark.parametrize("kind", ["grid", "chain"])
 def test_cap_and_chains(m, max_det, kind):
     _check(m, kind, 1.0, max_det=max_det, batch=2)
+
+
+@pytest.mark.parametrize("m", [96, 97, 700, 1500])
+def test_many_survivors(m):
+    """Boxes that do not overlap: every candidate survives (counting, register sort, network)."""
+    _check(m, "apart", 0.3, max_det=2000)
 
 
 def test_thresholds_at_the_ends():
