@@ -81,14 +81,16 @@ constexpr unsigned long long kKeySentinel = ~0ull;
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void src_coord(int d, int src, int dst, float inv_den, int& i0, int& rem) {
     const int den = 2 * dst;
-    int num = (2 * d + 1) * src - dst;
-    if (num <= 0) { i0 = 0; rem = 0; return; }
+    // selections instead of branches: several coordinates of a thread are computed side by side
+    const int num = max((2 * d + 1) * src - dst, 0);
     int q = __float2int_rz(__int2float_rn(num) * inv_den);
     int r = num - q * den;
-    if (r < 0) { q -= 1; r += den; }
-    else if (r >= den) { q += 1; r -= den; }
-    if (q >= src - 1) { i0 = src - 1; rem = 0; return; }
-    i0 = q; rem = r;
+    const int fix = r < 0 ? -1 : (r >= den ? 1 : 0);
+    q += fix;
+    r -= fix * den;
+    const bool edge = q >= src - 1;
+    i0 = edge ? src - 1 : q;
+    rem = edge ? 0 : r;
 }
 
 // ---------------------------------------------------------------------------------------

@@ -99,12 +99,35 @@ __device__ __forceinline__ void unpack_f32x2(unsigned long long v, float& lo, fl
 template <bool GENERAL>
 __device__ __forceinline__ void build_table(XEntry* xt, int ow, int rx0, int cw, int nw, int pl, int t, int threads) {
     const float inv_dx = 1.0f / (float)(2 * nw);
-    for (int dx = t; dx < ow; dx += threads) {
-        const int ix = dx - pl, ixc = GENERAL ? min(max(ix, 0), nw - 1) : dx;
-        XEntry e = make_xentry(ixc, cw, nw, inv_dx, 3 * rx0);
-        if (GENERAL && ix != ixc) e.wts = 0u;
-        xt[dx] = e;
+    for (int d0 = t; d0 < ow; d0 += 4 * threads) {
+        XEntry e[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int dx = min(d0 + j * threads, ow - 1);
+            const int ix = dx - pl, ixc = GENERAL ? min(max(ix, 0), nw - 1) : dx;
+            e[j] = make_xentry(ixc, cw, nw, inv_dx, 3 * rx0);
+            if (GENERAL && ix != ixc) e[j].wts = 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (d0 + j * threads < ow) xt[d0 + j * threads] = e[j];
     }
+}
+
+// floor(a / b) for 0 <= a < 2^22 and 1 <= b < 2^22: the quotient of the binary32 values is within two
+// units in its last place, so its integer part is off by at most one, which the remainder shows.  About
+// a third of the latency of the compiler's integer division.
+// The producer's way to a tile's first copy is a serial chain of such steps that nothing hides while a CTA
+// has few tiles.  With them, 32-bit tile numbers, four tap-table entries of a lane side by side and all that
+// needs no counts moved before the wait for the previous kernel, a pass went from 18.9 to 18.1 us (one
+// small frame), 26.9 to 25.6 (one camera), 58.3 to 56.5 (eight), 1286 to 1257 (32 crowds, 770 crops each:
+// the producer is what their small crops wait for).  The consumers building every tile's table instead, with
+// a barrier among them per tile, helped one camera as much and cost larger batches 1 %; 16-byte copies by
+// the producer's lanes instead of one bulk copy per row cost 1 to 4 % (rows up to 512 bytes) and 13 % (1 KB).
+__device__ __forceinline__ int div_small(int a, int b) {
+    const int q = __float2int_rz(__fdividef((float)a, (float)b));
+    const int r = a - q * b;
+    return q + (r < 0 ? -1 : (r >= b ? 1 : 0));
 }
 
 // QUEUE = false: items come from the stage's current batch through the assembler above.
@@ -129,7 +152,6 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             const QRecord* __restrict__ qrec, const int* __restrict__ qpacked, unsigned int* __restrict__ qstatus,
             int* __restrict__ sched, const CropOpts opts) {
     extern __shared__ __align__(128) unsigned char smem[];
-    pdl_wait();
     __shared__ __align__(8) uint64_t full[kCropStages], empty[kCropStages];
     __shared__ CropPass s_pass[kCropStages];
     __shared__ __align__(16) RowInfo s_row[kCropStages][kCropMaxPassRows];  // per-row data of the staged passes
@@ -141,6 +163,27 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
     unsigned int* const status = QUEUE ? qstatus : &ctr->status;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+
+    if (threadIdx.x == 32) {
+        for (int b = 0; b < kCropStages; ++b) {
+            mbar_init(&full[b], 1);
+            mbar_init(&empty[b], kCropConsumerWarps);
+        }
+        mbar_fence_init();
+    }
+    // Producer: row runs that fit the consumer threads side by side, and the divisions by their number and
+    // by the units of a run as multiplications (of a crop that is not split into column tiles).
+    uint32_t w_quads = 0u, w_run_magic = 0u, w_unit_magic = 0u;
+    int w_runs = 1;
+    auto cut_runs = [&](uint32_t quads) {
+        if (quads == w_quads) return;
+        w_quads = quads;
+        w_runs = max(1, min(kCropConsumers / (int)quads, kCropMaxPassRows));
+        w_run_magic = w_runs > 1 ? 0xffffffffu / (uint32_t)w_runs + 1u : 0u;
+        w_unit_magic = quads > 1u ? 0xffffffffu / quads + 1u : 0u;
+    };
+    if (warp == kCropConsumerWarps) cut_runs((uint32_t)max(ow >> 2, 1));
+    pdl_wait();
 
     // ---- assembler: offsets of the branch's items per frame ------------------------------------
     if (!QUEUE && warp == 0) {
@@ -158,13 +201,6 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             run += __shfl_sync(0xffffffffu, inc, 31);
         }
         if (lane == 0) s_off[n] = run;
-    }
-    if (threadIdx.x == 0) {
-        for (int b = 0; b < kCropStages; ++b) {
-            mbar_init(&full[b], 1);
-            mbar_init(&empty[b], kCropConsumerWarps);
-        }
-        mbar_fence_init();
     }
     __syncthreads();
     const int total = QUEUE ? 0 : s_off[n];
@@ -184,19 +220,23 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
     // Tiles are (slot, row band).  One band per crop amortises the per-tile work (item lookup, tap
     // table) best; crops are cut into bands (multiples of 8 rows) only as far as needed to give
     // every CTA about kCropTilesPerCta tiles, which keeps the end of the grid short.
-    const int bands_want = packed > 0 ? (kCropTilesPerCta * (int)gridDim.x + packed - 1) / packed : 1;
-    const int bands_req = min(max(bands_want, 1), (oh + 7) >> 3);
-    const int band_rows = min(((oh + bands_req - 1) / bands_req + 7) & ~7, oh);
-    const int bands = (oh + band_rows - 1) / band_rows;
+    // (Divisions of small numbers throughout: crops are cut only where there are fewer than tiles wanted.)
+    const int tiles_want = kCropTilesPerCta * (int)gridDim.x;
+    const int groups = (oh + 7) >> 3;  // of 8 rows
+    const int bands_want = packed > 0 && packed < tiles_want ? div_small(tiles_want + packed - 1, packed) : 1;
+    const int bands_req = min(bands_want, groups);
+    const int band_rows = bands_req > 1 ? min((div_small(oh + bands_req - 1, bands_req) + 7) & ~7, oh) : oh;
+    const int bands = bands_req > 1 ? div_small(oh + band_rows - 1, band_rows) : 1;
     // The CTAs would end up to one tile apart, so the last crops (about one tile of the coarse cut
     // per CTA) are cut finer and even the end out: into kCropTailBands bands where a whole crop is a
     // tile, into twice as many bands as the others where crops are cut already.
-    const int tail_req = min(bands == 1 ? kCropTailBands : 2 * bands, (oh + 7) >> 3);
-    const int tail_rows = min(((oh + tail_req - 1) / tail_req + 7) & ~7, oh);
-    const int tail_bands = (oh + tail_rows - 1) / tail_rows;
-    const int tail_crops = tail_bands > bands ? min(packed, max((int)gridDim.x / bands, 1)) : 0;
-    const long long coarse_tiles = (long long)(packed - tail_crops) * bands;
-    const long long all_tiles = coarse_tiles + (long long)tail_crops * tail_bands;
+    const int tail_req = min(bands == 1 ? kCropTailBands : 2 * bands, groups);
+    const bool tail_same = band_rows == 8 || tail_req == 1;  // nothing finer than the coarse cut
+    const int tail_rows = tail_same ? band_rows : min((div_small(oh + tail_req - 1, tail_req) + 7) & ~7, oh);
+    const int tail_bands = tail_same ? bands : div_small(oh + tail_rows - 1, tail_rows);
+    const int tail_crops = tail_bands > bands ? min(packed, max(div_small((int)gridDim.x, bands), 1)) : 0;
+    const int coarse_tiles = (packed - tail_crops) * bands;
+    const int all_tiles = coarse_tiles + tail_crops * tail_bands;
     const size_t plane = (size_t)ow * (size_t)oh;
 
     if (warp == kCropConsumerWarps) {
@@ -216,8 +256,6 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
         int w_row_lo = 0, w_row_hi = 0, w_tile_cols = ow;
         int w_c0 = 0, w_ncols = 0, w_r0 = 0;
         int w_seg_lo = 0, w_seg = 0, w_stride = 16, w_cap_slots = 2;
-        int w_runs = 1;           // row runs that fit the consumer threads side by side
-        uint32_t w_run_magic = 0, w_unit_magic = 0;  // divisions by w_runs / by the units of a run, as multiplications
         bool w_valid = false, w_new = false;
         // size and offset of the resized rectangle inside the slot: the whole slot unless the
         // branch keeps the aspect ratio
@@ -246,14 +284,11 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             w_seg_lo = lo;
             w_seg = hi - lo;
             w_stride = w_seg + 16;
-            w_cap_slots = kCropRowBudget / w_stride;  // >= 2
+            w_cap_slots = div_small(kCropRowBudget, w_stride);  // >= 2
             // Work units of a pass: (run of consecutive rows, two column pairs half a tile apart).
             // A pass is cut into as many runs as fit the consumer threads side by side (224
             // columns: 4 runs x 56 units = the 224 consumer threads).
-            const uint32_t quads = (uint32_t)max(w_ncols >> 2, 1);
-            w_runs = max(1, min(kCropConsumers / (int)quads, kCropMaxPassRows));
-            w_run_magic = w_runs > 1 ? 0xffffffffu / (uint32_t)w_runs + 1u : 0u;
-            w_unit_magic = quads > 1u ? 0xffffffffu / quads + 1u : 0u;
+            cut_runs((uint32_t)max(w_ncols >> 2, 1));
         };
         // A tile resolved: (slot, band) -> item -> detection -> outward-rounded rectangle in its frame.
         // Three dependent global round trips when the tile number comes from the counter; no warp
@@ -262,19 +297,19 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             int ok, slot, band, band_rows, f, det, rx0, ry0, rx1, ry1, pitch, fh;
             const uint8_t* data;
         };
-        auto resolve = [&](long long tile) {
+        auto resolve = [&](int tile) {
             Tile t;
             t.ok = tile < all_tiles ? 1 : 0;
             t.slot = 0; t.band = 0; t.band_rows = band_rows; t.f = 0; t.det = 0;
             t.rx0 = 0; t.ry0 = 0; t.rx1 = 1; t.ry1 = 1; t.pitch = 0; t.fh = 1; t.data = nullptr;
             if (!t.ok) return t;
             if (tile < coarse_tiles) {
-                t.slot = (int)(tile / bands);
-                t.band = (int)(tile - (long long)t.slot * bands);
+                t.slot = bands > 1 ? div_small(tile, bands) : tile;
+                t.band = tile - t.slot * bands;
             } else {
-                const long long u = tile - coarse_tiles;
-                t.slot = (packed - tail_crops) + (int)(u / tail_bands);
-                t.band = (int)(u % tail_bands);
+                const int u = tile - coarse_tiles, c = div_small(u, tail_bands);
+                t.slot = (packed - tail_crops) + c;
+                t.band = u - c * tail_bands;
                 t.band_rows = tail_rows;
             }
             if (QUEUE) {
@@ -308,8 +343,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
         // The first kCropTilesAhead tiles of a CTA are fixed (block index + j * grid size) and
         // resolved up front, lane j resolving tile j, so that their round trips overlap: with few
         // tiles per CTA (small batches) the chain is paid once, not once per tile.
-        const Tile ahead = resolve(lane < kCropTilesAhead ? (long long)blockIdx.x + (long long)lane * (long long)gridDim.x
-                                                          : all_tiles);
+        const Tile ahead = resolve(lane < kCropTilesAhead ? (int)blockIdx.x + lane * (int)gridDim.x : all_tiles);
         // first pass of the next tile, if there is one
         auto open_tile = [&]() {
             Tile t;
@@ -332,8 +366,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             } else {
                 int c = 0;
                 if (lane == 0) c = atomicAdd(sched, 1);
-                t = resolve((long long)kCropTilesAhead * (long long)gridDim.x +
-                            (long long)__shfl_sync(0xffffffffu, c, 0));
+                t = resolve(kCropTilesAhead * (int)gridDim.x + __shfl_sync(0xffffffffu, c, 0));
             }
             w_tiles += 1;
             w_valid = t.ok != 0;
