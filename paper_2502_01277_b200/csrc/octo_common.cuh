@@ -341,13 +341,18 @@ __device__ __forceinline__ bool mbar_wait_sleeping(uint64_t* bar, uint32_t parit
     return false;
 }
 // Global -> shared bulk copy; both addresses 16-byte aligned, bytes a multiple of 16.
-__device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {
+__device__ __forceinline__ void bulk_g2s(uint32_t dst_smem, const void* src_gmem, uint32_t bytes, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst_smem)),
-        "l"(src_gmem), "r"(bytes), "r"(smem_u32(bar))
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_smem),
+        "l"(src_gmem), "r"(bytes), "r"(bar)
         : "memory");
 }
+__device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {
+    bulk_g2s(smem_u32(dst_smem), src_gmem, bytes, smem_u32(bar));
+}
+// A value that is the same in every lane of a converged warp (or zero in the others), in a register that
+// the warp shares.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
 
 // ---------------------------------------------------------------------------------------
 // Fixed binary32 arithmetic shared by decode and NMS.  Every operation is an explicitly

@@ -454,10 +454,9 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             // tap already?  Source rows never decrease from one output row to the next, so the
             // row before is the only one that can share them.
             const int maxrow = y0 + need2;
-            int p_has = __shfl_up_sync(0xffffffffu, has_row ? 1 : 0, 1);
-            const int p_max = __shfl_up_sync(0xffffffffu, maxrow, 1);
-            const int p_need2 = __shfl_up_sync(0xffffffffu, need2, 1);
-            if (lane == 0) p_has = 0;
+            const int prev = __shfl_up_sync(0xffffffffu, has_row ? 2 * maxrow + need2 : -1, 1);
+            const bool p_has = lane != 0 && prev >= 0;
+            const int p_max = prev >> 1, p_need2 = prev & 1;
             int newrows = 0, back = 0;
             uint32_t code = 2u;
             if (has_row) {
@@ -475,9 +474,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             const int slot_top = incl - newrows - back;
             RowInfo ri;
             ri.row0 = 0; ri.step = 0; ri.wx = 0.0f; ri.wy = 0.0f;
-            uint32_t bytes = 0;
             if (in_pass && has_row) {
-                bytes = (uint32_t)(newrows * w_seg);
                 ri.row0 = slot_top * w_stride - w_seg_lo;  // table offsets are relative to the frame row
                 ri.step = (int32_t)((need2 ? (uint32_t)w_stride : 0u) | (code << 16));
                 ri.wx = (float)(2 * w_nh - ry) * w_inv_all;
@@ -485,7 +482,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             } else if (GENERAL) {
                 ri.step = -1;  // canvas row: nothing is staged for it
             }
-            const uint32_t total_tx = __reduce_add_sync(0xffffffffu, bytes);
+            const uint32_t total_tx = (uint32_t)(__shfl_sync(0xffffffffu, incl, max(nr - 1, 0)) * w_seg);
             CropPass p;
             p.valid = w_valid ? 1 : 0;
             p.table = tb;
@@ -515,6 +512,11 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             __syncwarp();  // table, pass record and row data are written before the barrier is armed
             if (lane == 0) mbar_expect_tx(&full[b], total_tx);
             __syncwarp();
+            // One bulk copy per row, and the lanes' copies go out one after the other: with the operands they
+            // have in common in registers that the warp shares, each is cheaper (90 -> 80 cycles a copy beside
+            // the consumers; 32 crowds, whose small crops wait for the producer: 1257 -> 1228 us a pass).  One
+            // lane that walks the rows is no faster, a loop of all lanes with one issuing 30 % slower.
+            const uint32_t seg = warp_uniform((uint32_t)w_seg), bar = warp_uniform(smem_u32(&full[b]));
             if (in_pass && newrows > 0) {
                 // the new rows are the last `newrows` of {y0, y0 + 1}
                 const int first_new = need2 + 1 - newrows;  // 0: y0 is new, 1: only y0 + 1
@@ -533,8 +535,8 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                 }
 #endif
                 if (ok) {
-                    bulk_g2s(dst, src, (uint32_t)w_seg, &full[b]);
-                    if (newrows == 2) bulk_g2s(dst + w_stride, src + w_pitch, (uint32_t)w_seg, &full[b]);
+                    bulk_g2s(smem_u32(dst), src, seg, bar);
+                    if (newrows == 2) bulk_g2s(smem_u32(dst) + (uint32_t)w_stride, src + w_pitch, seg, bar);
                 }
             }
             advance(nr);
