@@ -398,7 +398,7 @@ OCTO_API int32_t octo_stage_last_nms_cluster(const octo_stage_t* st);
 
 /* 1 when the stage's latest NMS launch ran two half-sized CTAs per SM, else 0.  In automatic mode a
  * batch of more images than the GPU has SMs is launched that way (one wave of CTAs instead of
- * two) unless one of the stage's latest 64 NMS launches is known to have seen an image with more
+ * two), except for 64 launches from the call that finds the report of an image with more
  * than 1024 candidates; a half-sized CTA holds 4096 candidates on chip instead of 8192 and sends
  * a larger image through the global-memory path.  Results do not depend on the form. */
 OCTO_API int32_t octo_stage_last_nms_half_ctas(const octo_stage_t* st);

@@ -5,13 +5,13 @@
 // so the ascending order of the keys of a class is its NMS order.
 //
 // Candidates are worked on in batches of whole classes, one thread (or up to four) per candidate
-// (nms_batch): put in order (words of 32 by counting, then every candidate's place in every word by binary
-// search); each tested against the earlier candidates of its class (one bit each); which survive is settled
+// (nms_batch): put in order (by counting inside a class, or inside its score bucket; where one is large, words
+// of 32 by counting, then every candidate's place in every word by binary search); each tested against the earlier candidates of its class (one bit each); which survive is settled
 // word by word of those bits (resolve_words), in a time that follows the length of the chains of overlapping
 // boxes, not the number of candidates of a class.  Up to kSmallMax candidates (the usual case in serving) are
 // one batch; more are bucketed by class first (histogram, scan, scatter) and cut into about as many
 // batches as the image has CTAs.  Survivors are re-keyed to (inverted score | anchor | class) and put in order
-// by counting or by a sort in registers.
+// by counting or by score buckets.
 // us per launch (CUDA events), against one thread per class that walked its candidates (and one warp per
 // class above 256): 200 candidates of one class, 8 images, 16.8 (67.4), of 7 classes 13.9 (28.3), of 80 classes
 // 12.7 (12.6); 90 candidates under class-agnostic NMS 12.7 (35.7); 5000 candidates of 80 classes, one image
