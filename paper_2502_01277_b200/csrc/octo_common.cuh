@@ -81,7 +81,20 @@ constexpr unsigned long long kKeySentinel = ~0ull;
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ void src_coord(int d, int src, int dst, float inv_den, int& i0, int& rem) {
     const int den = 2 * dst;
-    // selections instead of branches: several coordinates of a thread are computed side by side
+    int num = (2 * d + 1) * src - dst;
+    if (num <= 0) { i0 = 0; rem = 0; return; }
+    int q = __float2int_rz(__int2float_rn(num) * inv_den);
+    int r = num - q * den;
+    if (r < 0) { q -= 1; r += den; }
+    else if (r >= den) { q += 1; r -= den; }
+    if (q >= src - 1) { i0 = src - 1; rem = 0; return; }
+    i0 = q; rem = r;
+}
+// The same with selections instead of branches, for a thread that computes several coordinates side by side
+// (the crop kernel's producer: one camera 26.9 -> 26.4 us a pass).  The letterbox kernel, whose threads compute
+// one at a time, keeps the branches: 200 frames of 320x240 take 152 us with them and 162 us without.
+__device__ __forceinline__ void src_coord_flat(int d, int src, int dst, float inv_den, int& i0, int& rem) {
+    const int den = 2 * dst;
     const int num = max((2 * d + 1) * src - dst, 0);
     int q = __float2int_rz(__int2float_rn(num) * inv_den);
     int r = num - q * den;
@@ -105,9 +118,11 @@ struct XEntry {
     uint32_t wts;  // (den - rem) | rem << 16
 };
 
+template <bool FLAT>
 __device__ __forceinline__ XEntry make_xentry(int d, int src, int dst, float inv_den, int byte_base) {
     int x0, rem;
-    src_coord(d, src, dst, inv_den, x0, rem);
+    if (FLAT) src_coord_flat(d, src, dst, inv_den, x0, rem);
+    else src_coord(d, src, dst, inv_den, x0, rem);
     XEntry e;
     e.off = (uint32_t)(byte_base + 3 * x0);
     e.wts = (uint32_t)(2 * dst - rem) | ((uint32_t)rem << 16);

@@ -105,7 +105,7 @@ __device__ __forceinline__ void build_table(XEntry* xt, int ow, int rx0, int cw,
         for (int j = 0; j < 4; ++j) {
             const int dx = min(d0 + j * threads, ow - 1);
             const int ix = dx - pl, ixc = GENERAL ? min(max(ix, 0), nw - 1) : dx;
-            e[j] = make_xentry(ixc, cw, nw, inv_dx, 3 * rx0);
+            e[j] = make_xentry<true>(ixc, cw, nw, inv_dx, 3 * rx0);
             if (GENERAL && ix != ixc) e[j].wts = 0u;
         }
 #pragma unroll
@@ -276,8 +276,8 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                 // canvas columns count as the nearest image column
                 const int ia = min(max(w_c0 - w_pl, 0), w_nw - 1);
                 const int ib = min(max(w_c0 + w_ncols - 1 - w_pl, 0), w_nw - 1);
-                src_coord(ia, w_cw, w_nw, w_inv_dx, xa, rem);
-                src_coord(ib, w_cw, w_nw, w_inv_dx, xb, rem);
+                src_coord_flat(ia, w_cw, w_nw, w_inv_dx, xa, rem);
+                src_coord_flat(ib, w_cw, w_nw, w_inv_dx, xb, rem);
                 lo = (3 * (w_rx0 + xa)) & ~15;
                 hi = min((3 * (w_rx0 + xb) + 6 + 15) & ~15, full_hi);
             }
@@ -448,7 +448,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             const int iy = w_r0 + lane - w_pt;  // row inside the resized rectangle
             const bool has_row = cand && (!GENERAL || (iy >= 0 && iy < w_nh));
             int y0 = 0, ry = 0;
-            if (has_row) src_coord(iy, w_ch, w_nh, w_inv_dy, y0, ry);
+            if (has_row) src_coord_flat(iy, w_ch, w_nh, w_inv_dy, y0, ry);
             const int need2 = ry != 0 ? 1 : 0;
             // Which of this row's tap rows (y0, and y0 + 1 if need2) did the row before it not
             // tap already?  Source rows never decrease from one output row to the next, so the

@@ -104,7 +104,7 @@ letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict
         const int ix = dx - pad_l;
         XEntry e;
         if (ix < 0 || ix >= nw) { e.off = 0; e.wts = 0; }  // zero weights mark a canvas column
-        else e = make_xentry(ix, w, nw, inv_dx, 0);
+        else e = make_xentry<false>(ix, w, nw, inv_dx, 0);
         s_xtab[dx] = e;
     }
     __syncthreads();  // barrier armed, table and row weights visible
