@@ -32,21 +32,21 @@ def _boxes(rng, m, kind):
                      rng.integers(1, 9, m) * 4.0], 1)
 
 
-def _check(m, kind, share, cluster=0, agnostic=False, max_det=300, batch=1, iou=0.5):
+def _check(m, kind, share, cluster=0, agnostic=False, max_det=300, batch=1, iou=0.5, classes=CLASSES):
     rng = np.random.default_rng(m * 7 + len(kind))
     anchors = max(m, 4) + 3
-    head = np.zeros((batch, anchors, 5 + CLASSES), dtype=np.float32)
+    head = np.zeros((batch, anchors, 5 + classes), dtype=np.float32)
     for b in range(batch):
         at = rng.permutation(anchors)[:m]
         head[b, at, :4] = _boxes(rng, m, kind)
         head[b, at, 4] = 1.0
-        cls = np.where(rng.random(m) < share, 2, rng.integers(0, CLASSES, m))
+        cls = np.where(rng.random(m) < share, 2, rng.integers(0, classes, m))
         head[b, at, 5 + cls] = np.round(rng.uniform(0.3, 0.99, m) * 512) / 512  # ties in the score
         if kind == "chain":  # strongest first: every second link survives, one link settled per round
             head[b, at, 5:] = 0.0
             head[b, at, 7] = np.linspace(0.99, 0.3, m)
     frames, sizes = [np.zeros((192, 768), dtype=np.uint8)] * batch, [(256, 192)] * batch
-    st = octo.Stage(net_size=SIDE, max_batch=batch, num_anchors=anchors, num_classes=CLASSES, head_is_logits=False,
+    st = octo.Stage(net_size=SIDE, max_batch=batch, num_anchors=anchors, num_classes=classes, head_is_logits=False,
                     iou_thresh=iou, max_det=max_det, branches=((8, 8),), class_agnostic=agnostic)
     try:
         st.set_nms_cluster(cluster)
@@ -75,6 +75,17 @@ def test_short_path(m, kind, agnostic):
 @pytest.mark.parametrize("cluster", [1, 4])
 def test_large_classes(m, share, cluster):
     _check(m, "grid", share, cluster=cluster, max_det=1000)
+
+
+@pytest.mark.parametrize("m,share,kind,max_det", [(513, 0.0, "grid", 300), (513, 0.19, "grid", 1000), (2000, 0.21, "grid", 1000),
+                                                  (1500, 0.0, "chain", 2), (1900, 0.0, "apart", 2000),
+                                                  (900, 0.0, "same", 300), (8192, 0.1, "grid", 1000),
+                                                  (8300, 0.0, "grid", 1000)])
+def test_many_classes_on_one_cta(m, share, kind, max_det):
+    """Classes of at most a fifth of the image: one warp per class (one of more: batches); full-sized CTAs and,
+    with more images than SMs, half-sized ones."""
+    for batch in (1, 160) if m <= 2000 else (1,):
+        _check(m, kind, share, cluster=1, max_det=max_det, classes=40, batch=batch)
 
 
 @pytest.mark.parametrize("m,max_det", [(120, 5), (256, 300), (600, 5), (600, 1), (1100, 70)])
