@@ -424,6 +424,8 @@ __device__ __forceinline__ void iou_terms(const float4 a, const float4 b, float&
 // Almost every pair is decided in binary32 already: t = fl(midf * uni), midf = fl(mid), is within
 // 2^-22.9 of mid * uni (two roundings, t a normal number), so |inter - t| > 2^-20 t settles the sign.
 // The binary64 form needs two conversions per pair, which issue at a fraction of the binary32 rate.
+// Thresholds below 2^-60 have no binary32 decision (midf and share are NaN, every pair goes to the exact
+// form): the products with such a threshold may underflow where inter does not.
 struct IouTest {
     double mid;
     float midf;
@@ -448,9 +450,11 @@ __device__ __forceinline__ bool iou_quick(const float4 a, const float4 b, const 
 // share * area_a + share * area_b, with the two products made once per box (iou_share).  All roundings
 // together (those of the formula's own union among them) stay below 2^-21 of the sum, so a distance of
 // more than 2^-19 of it settles the pair.  One side of the overlap may stay negative: with the other
-// clamped to zero the product is then at most zero, as it should be.
+// clamped to zero the product is then at most zero, as it should be.  A box so large that the formula's
+// sum of two areas could overflow has no share (NaN: its pairs go to the exact form).
 __device__ __forceinline__ float iou_share(const float4 a, const IouTest& t) {
-    return __fmul_rn(t.share, __fmul_rn(__fsub_rn(a.z, a.x), __fsub_rn(a.w, a.y)));
+    const float area = __fmul_rn(__fsub_rn(a.z, a.x), __fsub_rn(a.w, a.y));
+    return area < 0x1p126f ? __fmul_rn(t.share, area) : __int_as_float(0x7fffffff);
 }
 __device__ __forceinline__ bool iou_by_share(const float4 a, float share_a, const float4 b, float share_b, bool& close) {
     const float iw = fmaxf(__fsub_rn(fminf(a.z, b.z), fmaxf(a.x, b.x)), 0.0f);

@@ -31,8 +31,9 @@ static NmsParams nms_params(const NmsArgs& a) {
     // rounding boundary of the IoU test (see iou_exact)
     const float up = nextafterf(a.iou_thr, INFINITY);
     p.iou_test.mid = 0.5 * ((double)a.iou_thr + (double)up);
-    p.iou_test.midf = (float)p.iou_test.mid;
-    p.iou_test.share = (float)(p.iou_test.mid / (1.0 + p.iou_test.mid));
+    const bool quick = p.iou_test.mid >= 0x1p-60;
+    p.iou_test.midf = quick ? (float)p.iou_test.mid : NAN;
+    p.iou_test.share = quick ? (float)(p.iou_test.mid / (1.0 + p.iou_test.mid)) : NAN;
     unsigned int up_bits;
     memcpy(&up_bits, &up, sizeof(up_bits));
     p.iou_test.tie_up = (up_bits & 1u) == 0u ? 1 : 0;

@@ -25,6 +25,10 @@ def _boxes(rng, m, kind):
     if kind == "apart":
         i = np.arange(m)
         return np.stack([2 + 5.0 * (i % 48), 2 + 5.0 * (i // 48), np.full(m, 4.0), np.full(m, 4.0)], 1)
+    if kind == "powers":
+        return np.concatenate([np.zeros((m, 2)), 2.0 ** rng.integers(-50, 67, (m, 1)) * 2.0 ** rng.integers(-2, 3, (m, 2))], 1)
+    if kind == "huge":  # areas from 2^125 on: the sum of two may overflow
+        return np.concatenate([np.zeros((m, 2)), 2.0 ** 63 * (1 + 0.25 * rng.integers(-2, 4, (m, 2)))], 1)
     if kind == "same":
         return np.tile(np.array([[100.0, 90.0, 30.0, 20.0]]), (m, 1))
     # a coarse grid of sizes and places: many IoU values are simple fractions, 1/2 among them
@@ -104,3 +108,13 @@ def test_thresholds_at_the_ends():
     for iou in (0.0, 1.0):
         _check(150, "grid", 0.7, iou=iou)
         _check(600, "grid", 0.7, iou=iou)
+
+
+@pytest.mark.parametrize("iou", [0.0, 1e-45, 1e-38, 1e-30, 0.45])
+@pytest.mark.parametrize("m", [150, 700, 1100])
+def test_areas_and_thresholds_at_the_ends_of_binary32(m, iou):
+    """Boxes around one point with sides from 2^-50 to 2^66: areas from underflow to overflow, quotients that
+    round to zero, products with the threshold that underflow, sums of areas that overflow."""
+    for kind in ("powers", "huge"):
+        _check(m, kind, 0.3, iou=iou, max_det=1000)
+        _check(m, kind, 0.0, iou=iou, max_det=1000, classes=40, cluster=1)
