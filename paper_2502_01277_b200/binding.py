@@ -372,12 +372,16 @@ class Stage:
         n, s = len(frames), self.cfg.net_size
         if out is None:
             out = t.empty((n, 3, s, s), dtype=t.float16, device=self.device)
-        arr = self._frame_array if n <= self.cfg.max_batch else (Frame * n)()  # (the library refuses the latter)
         flat = []
         for f, (w, h) in zip(frames, sizes):
             flat += (f.data_ptr(), w, h, f.stride()[0], 0)
-        struct.pack_into("@" + "Piiii" * n, arr, 0, *flat)
-        rc = self._lib.octo_preprocess_batch(self.handle, arr, n, out.data_ptr(), self._stream(stream))
+        k = len(flat) // 5  # (a list longer than the other is cut, as zip does)
+        arr = self._frame_array if k <= self.cfg.max_batch else (Frame * k)()  # (the library refuses the latter)
+        try:
+            struct.pack_into("@" + "Piiii" * k, arr, 0, *flat)
+        except struct.error:  # a number that does not fit its field: as an assignment to the field takes it
+            arr = self.frame_array(frames, sizes)
+        rc = self._lib.octo_preprocess_batch(self.handle, arr, k, out.data_ptr(), self._stream(stream))
         if rc != OCTO_OK:
             raise OctoError(rc, "octo_preprocess_batch")
         self._frames_keepalive = list(frames)

@@ -88,6 +88,32 @@ def test_null_arguments_are_rejected():
     assert lib.octo_strerror(binding.OCTO_E_NO_MEMORY) == b"out of host or device memory"
 
 
+class _Recorder:
+    """Stands in for the library: notes the descriptors of octo_preprocess_batch."""
+
+    def octo_preprocess_batch(self, handle, arr, n, d_out, stream):
+        self.calls = [(arr[i].d_data, arr[i].width, arr[i].height, arr[i].pitch_bytes) for i in range(n)]
+        return binding.OCTO_OK
+
+
+@pytest.mark.parametrize("sizes", [[(40, 30), (16, 8)], [(40, 30)], [(40, 30), (16, 8), (7, 7)], [],
+                                   [(1 << 31, 30), (-(1 << 40) + 3, 8)]])
+def test_preprocess_marshals_what_it_is_given(sizes):
+    """Frames and sizes of different numbers are paired as far as they go; a number beyond 32 bits reaches the
+    library as an assignment to the field makes it, and the library decides."""
+    import torch
+    st = object.__new__(octo.Stage)
+    st._torch, st.cfg, st._lib, st.handle = torch, octo.make_config(max_batch=2), _Recorder(), None
+    st._current_stream, st._frame_array = (lambda: 0), (binding.Frame * 2)()
+    frames = [torch.zeros((h, pitch), dtype=torch.uint8) for h, pitch in ((30, 128), (8, 48))]
+    out = torch.empty((2, 3, 8, 8), dtype=torch.float16)
+    assert st.preprocess(frames, sizes, out=out) is out
+    want = [(f.data_ptr(), *(((v + (1 << 31)) % (1 << 32)) - (1 << 31) for v in wh), f.stride(0))
+            for f, wh in zip(frames, sizes)]
+    assert st._lib.calls == want and st.n == 2
+    assert [id(f) for f in st._frames_keepalive] == [id(f) for f in frames]
+
+
 def test_missing_library_fails_loudly(tmp_path):
     with pytest.raises(ImportError):
         octo.load_library(str(tmp_path / "nope.so"))
