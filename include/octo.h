@@ -340,10 +340,10 @@ OCTO_API int octo_queue_pop_due(octo_queue_t* q, int32_t bz, int32_t max_wait, v
 /* Synchronise `cuda_stream`, then read (and keep) the device status word. */
 OCTO_API int octo_stage_status(octo_stage_t* st, uint32_t* status_word, void* cuda_stream);
 
-/* Test support for the time-out path: enqueue a one-thread kernel that arms a barrier for bytes
- * that never arrive (no copy is issued), polls it `polls` times (1 .. 2^20) and then sets
- * OCTO_STATUS_COPY_TIMEOUT, exactly as the bulk-copy waits of the letterbox and crop kernels do
- * when they give up.  Afterwards octo_stage_status returns OCTO_E_DEVICE_TIMEOUT until the status
+/* Test support for the time-out path: enqueue a kernel whose first warp waits for a barrier that is complete
+ * and whose other warps wait for bytes that never arrive (no copy is issued): they poll 2 * `polls` times
+ * (1 .. 2^20) and then set OCTO_STATUS_COPY_TIMEOUT, exactly as the bulk-copy waits of the letterbox, decode
+ * and crop kernels do when they give up.  Afterwards octo_stage_status returns OCTO_E_DEVICE_TIMEOUT until the status
  * word is cleared; the context stays usable. */
 OCTO_API int octo_stage_selftest_wait(octo_stage_t* st, int32_t polls, void* cuda_stream);
 

@@ -333,6 +333,14 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
+// A wait for copies: a second round of polls before giving up (the copies in flight get one more chance to
+// land).  Threads wait each for themselves, so every thread whose wait ran out reports it.
+__device__ __forceinline__ bool mbar_wait_or_report(uint64_t* bar, uint32_t parity, unsigned int* status,
+                                                    int limit = 1 << 20) {
+    if (mbar_wait_bounded(bar, parity, limit) || mbar_wait_bounded(bar, parity, limit)) return true;
+    atomicOr(status, 0x4u);
+    return false;
+}
 // The same for a warp that expects to wait long (a producer waiting for its consumers): plain
 // phase tests with a sleep in between, so that the waiting warp takes almost no issue slots
 // from the working warps of its scheduler.

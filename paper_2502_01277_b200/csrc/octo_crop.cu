@@ -496,7 +496,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             if (k >= kCropStages) {
                 const uint32_t par = (ephase >> b) & 1u;
                 if (!mbar_wait_sleeping(&empty[b], par, kCropProducerSleepNs) && !mbar_wait_sleeping(&empty[b], par, kCropProducerSleepNs)) {
-                    if (lane == 0) atomicOr(status, 0x4u);
+                    atomicOr(status, 0x4u);
                     break;
                 }
                 ephase ^= 1u << b;
@@ -559,10 +559,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
         for (int k = 0;; ++k) {
             const int b = k % kCropStages;
             const uint32_t par = (fphase >> b) & 1u;
-            if (!mbar_wait_bounded(&full[b], par) && !mbar_wait_bounded(&full[b], par)) {
-                if (lane == 0) atomicOr(status, 0x4u);
-                break;
-            }
+            if (!mbar_wait_or_report(&full[b], par, status)) break;
             fphase ^= 1u << b;
             const CropPass cur = s_pass[b];
             if (!cur.valid) break;

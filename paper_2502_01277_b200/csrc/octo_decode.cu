@@ -382,10 +382,7 @@ decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, floa
     }
     if (t < values - bulk) s[bulk + t] = __ldg(src + bulk + t);
     __syncthreads();
-    if (!mbar_wait_bounded(&bar, 0) && !mbar_wait_bounded(&bar, 0)) {
-        if (t == 0) atomicOr(status, 0x4u);
-        return;
-    }
+    if (!mbar_wait_or_report(&bar, 0, status)) return;
     if (t >= rows) return;
     // lanes whose rows start in the same bank (32 / gcd(row_len, 32) lanes apart) start at different values
     const int banks = row_len & -row_len;  // gcd with a power of two

@@ -108,12 +108,7 @@ letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict
         s_xtab[dx] = e;
     }
     __syncthreads();  // barrier armed, table and row weights visible
-    bool copy_ok = mbar_wait_bounded(&bar, 0);
-    if (!copy_ok) {
-        // Give the copies in flight one more bounded chance to land before leaving.
-        copy_ok = mbar_wait_bounded(&bar, 0);
-        if (!copy_ok && threadIdx.x == 0) atomicOr(status, 0x4u);
-    }
+    const bool copy_ok = mbar_wait_or_report(&bar, 0, status);
 
     // one warp per output row of the band
     const int pairs = S >> 1;

@@ -349,18 +349,22 @@ static cudaError_t launch_adopt(const octo_stage* up, const octo_item_t* d_items
                          d_out);
 }
 
-// Test support: a wait that nothing ends.  One thread arms an mbarrier for `bytes` bytes that no
-// copy will ever deliver, polls it `polls` times, reports the timeout in the status word and
-// returns.  No copy is in flight at any point and the shared memory dies with the CTA.
+// Test support: a wait that nothing ends.  One mbarrier is armed for bytes that no copy will ever deliver,
+// another is complete.  The first warp finds the complete one; the other warps poll theirs 2 * `polls` times,
+// report the timeout in the status word and return.  No copy is in flight at any point and the shared memory
+// dies with the CTA.
 __global__ void wait_selftest_kernel(unsigned int* __restrict__ status, int polls) {
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bars[2];
     pdl_wait();
     if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
+        mbar_init(&bars[0], 1);
+        mbar_init(&bars[1], 1);
         mbar_fence_init();
-        mbar_expect_tx(&bar, 64u);
-        if (!mbar_wait_bounded(&bar, 0, polls)) atomicOr(status, 0x4u);
+        mbar_arrive(&bars[0]);
+        mbar_expect_tx(&bars[1], 64u);
     }
+    __syncthreads();
+    mbar_wait_or_report(&bars[threadIdx.x < 32 ? 0 : 1], 0, status, polls);
 }
 }  // namespace octo
 
@@ -396,7 +400,7 @@ extern "C" int octo_adopt_items_device(octo_stage_t* st, const octo_stage_t* ups
 extern "C" int octo_stage_selftest_wait(octo_stage_t* st, int32_t polls, void* cuda_stream) {
     if (!st || polls < 1 || polls > (1 << 20)) return OCTO_E_INVALID_ARG;
     OCTO_CUDA(cudaSetDevice(st->cfg.device));
-    OCTO_CUDA(launch_kernel(wait_selftest_kernel, dim3(1), dim3(32), 0, static_cast<cudaStream_t>(cuda_stream),
+    OCTO_CUDA(launch_kernel(wait_selftest_kernel, dim3(1), dim3(128), 0, static_cast<cudaStream_t>(cuda_stream),
                             &st->d_ctr->status, (int)polls));
     st->launches += 1;
     return OCTO_OK;

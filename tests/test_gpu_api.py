@@ -208,8 +208,9 @@ def test_two_host_threads_drive_two_stages():
 
 def test_a_wait_that_runs_out_is_reported_and_cleared(stage):
     """The time-out path of the bounded device waits, made to run out without any copy in flight:
-    the self-test kernel arms a barrier for bytes nobody sends and gives up after a few hundred
-    polls.  The status word carries the bit, octo_stage_status reports OCTO_E_DEVICE_TIMEOUT, the
+    in the self-test kernel the first warp's wait ends, while the other warps wait for bytes nobody
+    sends and give up after a few hundred polls (a report by the first thread alone would be lost).
+    The status word carries the bit, octo_stage_status reports OCTO_E_DEVICE_TIMEOUT, the
     context stays usable, and clearing the word brings the stage back to OCTO_OK."""
     lib = octo.load_library()
     import ctypes
