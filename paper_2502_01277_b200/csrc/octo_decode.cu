@@ -351,10 +351,13 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
 // one contiguous piece of memory: one bulk copy stages them (five CTAs of 85-value rows keep 218 KB per
 // SM in flight), then a thread reduces a row out of shared memory.  A row of an odd number of values is
 // read without bank conflicts as it stands (lane stride = row length); for the others the lanes start
-// at rotated positions.  us per launch on [n, 25200, 5 + C] against the row groups of decode_kernel:
-// C = 80, n = 1 10.8 (18.7), n = 4 18.8 (23.0), n = 32 70.1 (95.7: 274 MB at 3.9 instead of 2.9 TB/s);
-// C = 7, n = 8 10.7 (31.3); C = 20, n = 64 44.1 (108.0).  64 rows per CTA measure the same, 256 worse
-// (n = 32 82.7).
+// at rotated positions.  The scan of a row was the bound while it kept an index and tested every value's
+// exponent (12 instructions a value); now a value costs a load, a multiply-add that turns NaN once a value is
+// not finite, and a maximum, and the few rows that pass look for the class that holds the maximum.
+// us per launch on [n, 25200, 5 + C], row groups of decode_kernel / that scan / this one: C = 80, n = 1 18.5 / 12.3 /
+// 10.3, n = 4 22.6 / 18.5 / 14.3, n = 32 96 / 70.7 / 57.4; C = 27, n = 64 111 / 52.2 / 46; C = 128, n = 256 776 / 915 /
+// 479 (7.2 TB/s).  Multi-label heads [32, 6300, 128]: 77.8 / 127 / 47.1 (every row had walked its classes a
+// second time, rows of one bank one after the other).  64 rows per CTA measure the same.
 constexpr int kDenseRows = 128;
 
 __global__ void __launch_bounds__(kDenseRows)
@@ -384,24 +387,39 @@ decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, floa
     __syncthreads();
     if (!mbar_wait_or_report(&bar, 0, status)) return;
     if (t >= rows) return;
-    // lanes whose rows start in the same bank (32 / gcd(row_len, 32) lanes apart) start at different values
-    const int banks = row_len & -row_len;  // gcd with a power of two
-    int e = banks >= 32 ? (t & 31) : (t & 31) / (32 / banks);
     const float* const row = s + t * row_len;
-    bool fin = true;
+    const float* const cls = row + 5;
+    float zero = 0.0f;  // sum of 0 * value: a NaN once a value was not finite
     float best = -INFINITY;
-    int best_k = 0x7fffffff;
-#pragma unroll 4
-    for (int i = 0; i < row_len; ++i) {
-        const float v = row[e];
-        fin &= finite_f(v);
-        const int k = e - 5;
-        if (k >= 0 && (v > best || (v == best && k < best_k))) { best = v; best_k = k; }  // first maximum
-        e = e + 1 == row_len ? 0 : e + 1;
+    if (row_len & 1) {
+#pragma unroll
+        for (int e = 0; e < 5; ++e) zero = __fmaf_rn(row[e], 0.0f, zero);
+#pragma unroll 8
+        for (int k = 0; k < C; ++k) {
+            const float v = cls[k];
+            zero = __fmaf_rn(v, 0.0f, zero);
+            best = fmaxf(best, v);
+        }
+    } else {
+        // lanes whose rows start in the same bank (32 / gcd(row_len, 32) lanes apart) start at different values
+        const int banks = row_len & -row_len;  // gcd with a power of two
+        int e = banks >= 32 ? (t & 31) : (t & 31) / (32 / banks);
+#pragma unroll 8
+        for (int i = 0; i < row_len; ++i) {
+            const float v = row[e];
+            zero = __fmaf_rn(v, 0.0f, zero);
+            if (e >= 5) best = fmaxf(best, v);
+            e = e + 1 == row_len ? 0 : e + 1;
+        }
     }
-    if (!fin) atomicOr(status, 0x1u);
-    const float ob = row[4];
-    if (!fin || !(row[2] > 0.0f) || !(row[3] > 0.0f)) return;
+    if (!(zero == 0.0f)) {
+        atomicOr(status, 0x1u);
+        return;
+    }
+    // (no class of a row scores above its best, unless both factors are negative)
+    const float ob = row[4], top = __fmul_rn(ob, best);
+    if (!(top > conf) && !(multi && ob < 0.0f)) return;
+    if (!(row[2] > 0.0f) || !(row[3] > 0.0f)) return;
     auto emit = [&](int cls, float score) {
         const int slot = atomicAdd(cand_count + img, 1);
         if (slot < key_stride) {
@@ -412,11 +430,12 @@ decode_dense_kernel(const float* __restrict__ head, int A, int C, int mode, floa
         }
     };
     if (!multi) {
-        const float score = __fmul_rn(ob, best);
-        if (score > conf) emit(agnostic ? 0 : best_k, score);
+        int k = 0;  // the first maximum
+        while (!agnostic && k < C - 1 && cls[k] != best) ++k;
+        emit(k, top);
     } else {
         for (int k = 0; k < C; ++k) {
-            const float score = __fmul_rn(ob, row[5 + k]);
+            const float score = __fmul_rn(ob, cls[k]);
             if (score > conf) emit(k, score);
         }
     }

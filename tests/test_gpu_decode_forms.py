@@ -56,6 +56,25 @@ def test_probability_rows(anchors, classes, variant):
     assert res.status & ~0x2 == (0x1 if anchors > 4 else 0)
 
 
+@pytest.mark.parametrize("classes", [1, 11, 58, 59, 123])
+@pytest.mark.parametrize("variant", ["single", "multi", "agnostic"])
+def test_probability_rows_of_any_sign(classes, variant):
+    """Factors of both signs (two negative ones make a score), zeros of both signs and equal maxima at the ends of
+    rows of 6 to 128 values, a value that is not finite at every position of a row."""
+    anchors, rng = 300, np.random.default_rng(classes)
+    head = np.zeros((2, anchors, 5 + classes), dtype=np.float32)
+    head[..., :4] = _boxes(rng, (2, anchors))
+    head[..., 4] = rng.choice([-1.0, -0.5, -0.0, 0.0, 0.25, 0.5, 1.0, 1.5], (2, anchors))
+    head[..., 5:] = -0.01
+    for k in (0, classes - 1, int(rng.integers(classes))):
+        head[..., 5 + k] = rng.choice([-0.75, -0.5, 0.0, 0.5, 0.75, 1.0], (2, anchors))
+    for e in range(5 + classes):
+        head[1, 2 * e + 1, e] = (np.nan, np.inf, -np.inf)[e % 3]
+    res, _ = _run(head, False, anchors, classes, head_is_logits=False, multi_label=variant == "multi",
+                  class_agnostic=variant == "agnostic")
+    assert res.status & 0x1
+
+
 @pytest.mark.parametrize("anchors", [3, 4, 127, 128, 516, 1028])
 @pytest.mark.parametrize("classes,logits", [(1, False), (39, True), (41, False), (128, True)])
 @pytest.mark.parametrize("multi", [False, True])
