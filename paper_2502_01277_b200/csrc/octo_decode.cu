@@ -188,28 +188,30 @@ decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf
 // consecutive addresses of one plane, so a CTA fetches long contiguous runs (DRAM pages are used
 // better the longer the run).  CW = 8 / AW groups of warps split the C class planes between them
 // (group g takes classes g, g + CW, ...) and leave their running first maxima in shared memory, where
-// one thread per anchor merges them.  Every thread keeps kPlaneBatch planes in flight.
-// Bound by HBM for large batches and by the number of planes a warp walks one after another for small
-// ones, so the split follows the size of the grid: 4 x 2 warps where that still gives every SM six CTAs,
-// else 1 x 8 (measured us per launch, heads of [n, 84, 8400], 1 x 8 / 4 x 2 / 8 x 1: n = 1 8.7 / 12.3 /
-// 17.1, n = 8 14.8 / 20.9 / 33.3, n = 32 31.2 / 31.2 / 41.4, n = 64 47.7 / 45.4 / 50.0, n = 200 110.7 /
-// 105.9 / 121.7; 25.2, 53.8, 61.4, - and 129.4 with 8 x 1 warps and no explicit batch of loads, which
-// the compiler had not kept in flight together).
+// one thread per anchor merges them.  Every thread keeps kBatch planes in flight.
+// Bound by HBM for large batches of the vector form, by issue for large batches of the scalar form (a value
+// costs a load, the multiply-add that turns NaN once a value is not finite, a comparison and two selects; with
+// clamped plane numbers and a test of every exponent heads of odd A were slower than before the loads were
+// batched), and by the number of planes a warp walks one after another for small ones.  So the split follows
+// the size of the grid: side by side (four warps, or eight in the scalar form) where that gives every SM two
+// CTAs (one), else one warp's width and eight groups.  us per decode + NMS pass without batches of loads / with
+// batches of clamped plane numbers / now, [n, 84, A]: A = 8401, n = 8 12.3 / 13.6 / 10.1, n = 32 24.2 / 28.2 / 17.4, n = 256 116 /
+// 156 / 109; A = 8400, n = 8 27.1 / 11.2 / 10.4, n = 32 31.1 / 21.9 / 16.4, n = 256 130 / 112 / 109; multi-label, n = 32 76.5 /
+// 27.9 / 21.4; seven classes, A = 8401, n = 13 9.9 / 13.2 / 8.8.
 // For multi-label heads in logit form a value is only run through the fixed logistic sequence when it
 // lies above `pre`, a bound placed safely below the threshold's logit, so that the common case costs
 // one comparison per value.
-constexpr int kPlaneBatch = 5;
-constexpr int kPlaneWideCtas = 888;  // six CTAs for each of 148 SMs
-constexpr int kPlaneRepeat = 5;      // class planes a lane reads at a time the second time (multi-label)
+constexpr int kPlaneRepeat = 5;  // class planes a lane reads at a time the second time (multi-label)
 
 template <int VEC, int AW, bool MULTI>
-__global__ void __launch_bounds__(kDecThreads)
+__global__ void __launch_bounds__(kDecThreads, 5)
 decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, float conf, float pre, int key_stride,
                      unsigned long long* __restrict__ keys, float4* __restrict__ boxes, int* __restrict__ cand_count,
                      unsigned int* __restrict__ status) {
     pdl_wait();
     constexpr int CW = kDecThreads / 32 / AW;
     constexpr int kCtaAnchors = AW * 32 * VEC;
+    constexpr int kBatch = VEC == 4 ? 5 : 8;
     __shared__ float s_best[CW][kCtaAnchors];
     __shared__ unsigned char s_k[CW][kCtaAnchors];
     __shared__ unsigned char s_flags[CW][AW * 32];  // bits 0..3: non-finite, 4..7: above `pre`
@@ -225,37 +227,50 @@ decode_planes_kernel(const float* __restrict__ head, int A, int C, int mode, flo
     const int col = aw * 32 + lane;  // this thread's group of VEC anchors inside the CTA
     const int a0 = blockIdx.x * kCtaAnchors + col * VEC;
 
-    float best[VEC];
+    float best[VEC], zero[VEC];  // zero: sum of 0 * value, a NaN once a value was not finite
     int best_k[VEC];
     unsigned flags = 0u;
 #pragma unroll
-    for (int u = 0; u < VEC; ++u) { best[u] = -INFINITY; best_k[u] = 255; }
+    for (int u = 0; u < VEC; ++u) { best[u] = -INFINITY; zero[u] = 0.0f; best_k[u] = 255; }
     if (a0 < A) {
-        const float* __restrict__ cls0 = hbase + (size_t)4 * A + a0;
-        for (int k0 = cw; k0 < C; k0 += CW * kPlaneBatch) {
-            float v[kPlaneBatch][VEC];
-#pragma unroll
-            for (int j = 0; j < kPlaneBatch; ++j) {
-                const int k = min(k0 + j * CW, C - 1);  // past the end: the last plane again (no new maximum)
-                if (VEC == 4) {
-                    const float4 q = __ldg(reinterpret_cast<const float4*>(cls0 + (size_t)k * A));
-                    v[j][0] = q.x; v[j][1 % VEC] = q.y; v[j][2 % VEC] = q.z; v[j][3 % VEC] = q.w;
-                } else {
-                    v[j][0] = __ldg(cls0 + (size_t)k * A);
-                }
+        auto load = [&](const float* __restrict__ p, float (&v)[VEC]) {
+            if (VEC == 4) {
+                const float4 q = __ldg(reinterpret_cast<const float4*>(p));
+                v[0] = q.x; v[1 % VEC] = q.y; v[2 % VEC] = q.z; v[3 % VEC] = q.w;
+            } else {
+                v[0] = __ldg(p);
             }
+        };
+        auto take = [&](const float (&v)[VEC], int k) {
 #pragma unroll
-            for (int j = 0; j < kPlaneBatch; ++j) {
-                const int k = k0 + j * CW;
-#pragma unroll
-                for (int u = 0; u < VEC; ++u) {
-                    const float x = v[j][u];
-                    if (!finite_f(x)) flags |= 1u << u;
-                    if (x > best[u] && k < C) { best[u] = x; best_k[u] = k; }
-                    if (MULTI && x > pre) flags |= 16u << u;
-                }
+            for (int u = 0; u < VEC; ++u) {
+                zero[u] = __fmaf_rn(v[u], 0.0f, zero[u]);
+                if (v[u] > best[u]) { best[u] = v[u]; best_k[u] = k; }
+                if (MULTI && v[u] > pre) flags |= 16u << u;
             }
+        };
+        const size_t step = (size_t)CW * (size_t)A;
+        const float* __restrict__ p = hbase + (size_t)(4 + cw) * (size_t)A + a0;
+        int k = cw;
+        for (; k + (kBatch - 1) * CW < C; k += kBatch * CW) {
+            float v[kBatch][VEC];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) { load(p, v[j]); p += step; }
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) take(v[j], k + j * CW);
         }
+        float v[kBatch - 1][VEC];  // what is left: fewer than a batch
+#pragma unroll
+        for (int j = 0; j < kBatch - 1; ++j) {
+            if (k + j * CW < C) load(p, v[j]);
+            p += step;
+        }
+#pragma unroll
+        for (int j = 0; j < kBatch - 1; ++j)
+            if (k + j * CW < C) take(v[j], k + j * CW);
+#pragma unroll
+        for (int u = 0; u < VEC; ++u)
+            if (!(zero[u] == 0.0f)) flags |= 1u << u;
     }
 #pragma unroll
     for (int u = 0; u < VEC; ++u) {
@@ -457,9 +472,10 @@ static cudaError_t launch_planes_split(const DecodeArgs& a, int mode, float pre,
 // Warps side by side along the anchors, by the number of CTAs that gives (see decode_planes_kernel).
 template <int VEC>
 static cudaError_t launch_planes(const DecodeArgs& a, int mode, float pre, cudaStream_t stream) {
-    const long long ctas = (long long)a.n * ((a.A + 128 * VEC - 1) / (128 * VEC));
-    return ctas >= kPlaneWideCtas ? launch_planes_split<VEC, 4>(a, mode, pre, stream)
-                                  : launch_planes_split<VEC, 1>(a, mode, pre, stream);
+    constexpr int kWide = VEC == 4 ? 4 : 8;
+    const long long ctas = (long long)a.n * ((a.A + 32 * VEC * kWide - 1) / (32 * VEC * kWide));
+    return ctas >= (VEC == 4 ? 2 : 1) * (long long)a.sm_count ? launch_planes_split<VEC, kWide>(a, mode, pre, stream)
+                                                              : launch_planes_split<VEC, 1>(a, mode, pre, stream);
 }
 
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
@@ -489,7 +505,7 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream) {
                              a.d_status);
     }
     const int per_cta4 = kDecThreads * 4;
-    if ((long long)a.n * ((a.A + per_cta4 - 1) / per_cta4) >= 296) {
+    if ((long long)a.n * ((a.A + per_cta4 - 1) / per_cta4) >= 2ll * a.sm_count) {
         dim3 grid((a.A + per_cta4 - 1) / per_cta4, a.n);
         return launch_kernel(decode_kernel<4>, grid, dim3(kDecThreads), 0, stream, a.d_head, a.A, a.C, mode,
                              a.conf, a.key_stride, a.d_keys, a.d_boxes, a.d_cand_count, a.d_status);

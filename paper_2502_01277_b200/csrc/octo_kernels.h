@@ -28,6 +28,7 @@ struct DecodeArgs {
     float4* d_boxes;  // box of every candidate, at its key's slot
     int* d_cand_count;
     unsigned int* d_status;
+    int sm_count;
 };
 
 struct NmsArgs {

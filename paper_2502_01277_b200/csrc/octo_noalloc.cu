@@ -42,6 +42,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
 std::mutex g_mu;
 unsigned char* g_dev_ptr[kMaxDevices];  // device address of g_static_scratch, per device
+int g_sm_count[kMaxDevices];
 bool g_ready[kMaxDevices];
 
 // First use on a device: resolve the device address of the array and opt the kernels
@@ -55,6 +56,7 @@ cudaError_t setup_device(int device, unsigned char** out) {
         if (p == nullptr) return cudaErrorInvalidSymbol;
         e = prepare_nms(nullptr);
         if (e == cudaSuccess) e = prepare_decode();
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sm_count[device], cudaDevAttrMultiProcessorCount, device);
         if (e != cudaSuccess) return e;
         g_dev_ptr[device] = p;
         g_ready[device] = true;
@@ -145,6 +147,7 @@ extern "C" int octo_postprocess_frame_static(int32_t device, const float* d_head
     da.conf = conf_thresh;
     da.key_stride = key_stride;
     da.d_keys = d_keys; da.d_boxes = d_boxes; da.d_cand_count = d_cand; da.d_status = &d_ctr->status;
+    da.sm_count = g_sm_count[device];
     e = launch_decode(da, stream);
     if (e != cudaSuccess) return report_cuda_error(e, "decode_kernel");
 

@@ -428,6 +428,7 @@ extern "C" int octo_postprocess_batch(octo_stage_t* st, const float* d_head, int
         da.conf = c.conf_thresh;
         da.key_stride = st->key_stride;
         da.d_keys = st->d_keys; da.d_boxes = st->d_boxes; da.d_cand_count = st->d_cand_count; da.d_status = &st->d_ctr->status;
+        da.sm_count = st->sm_count;
         OCTO_CUDA(launch_decode(da, stream));
     }
     st->launches += 1;

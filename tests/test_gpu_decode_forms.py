@@ -79,18 +79,27 @@ def test_probability_rows_of_any_sign(classes, variant):
 @pytest.mark.parametrize("classes,logits", [(1, False), (39, True), (41, False), (128, True)])
 @pytest.mark.parametrize("multi", [False, True])
 def test_planes(anchors, classes, logits, multi):
-    """Class counts around the planes a warp looks at together (8 warps x 5 planes), anchor counts around
+    """Class counts around the planes eight groups of warps look at together, anchor counts around
     a CTA's share (128 or 32), in the vector and the scalar form (anchors not a multiple of four)."""
     _planes(2, anchors, classes, logits, multi)
 
 
 @pytest.mark.parametrize("anchors,n", [(128 * 5, 512), (128 * 2 - 1, 512)])
 def test_planes_wide_split(anchors, n):
-    """Enough CTAs (888) for four warps side by side along the anchors: vector and scalar form."""
+    """Enough CTAs for four (eight) warps side by side along the anchors: vector and scalar form."""
     _planes(n, anchors, 9, True, True)
 
 
-def _planes(n, anchors, classes, logits, multi):
+@pytest.mark.parametrize("classes", [2, 7, 8, 9, 10, 11, 40, 63, 64, 65])
+@pytest.mark.parametrize("n,anchors", [(2, 516), (2, 517), (300, 64), (300, 66)])
+@pytest.mark.parametrize("multi", [False, True])
+def test_planes_around_a_batch_of_loads(classes, n, anchors, multi):
+    """Class counts around the planes a thread has in flight (5 or 8, of one, two or eight groups of warps), in
+    both splits of both forms, with values that are not finite in the first and the last plane."""
+    _planes(n, anchors, classes, classes % 2 == 0, multi, bad=True)
+
+
+def _planes(n, anchors, classes, logits, multi, bad=False):
     rng = np.random.default_rng(anchors * 17 + classes)
     head = np.full((n, 4 + classes, anchors), -6.0, dtype=np.float32)
     head[:, :4] = np.moveaxis(_boxes(rng, (n, anchors)), -1, 1)
@@ -100,4 +109,8 @@ def _planes(n, anchors, classes, logits, multi):
     head[1, 4 + classes - 1, anchors - 1] = 3.0  # the last value of the head
     if not logits:
         head[:, 4:] = 1.0 / (1.0 + np.exp(-head[:, 4:]))
-    _run(head.astype(np.float32), True, anchors, classes, head_is_logits=logits, multi_label=multi and classes > 1)
+    if bad:
+        head[0, 4 + classes - 1, 1] = np.nan
+        head[1, 4, 2], head[1, 4 + classes - 1, 5] = np.inf, -np.inf
+    res, _ = _run(head.astype(np.float32), True, anchors, classes, head_is_logits=logits, multi_label=multi and classes > 1)
+    assert (res.status & 0x1 != 0) == bad
