@@ -10,7 +10,8 @@
 // word by word of those bits (resolve_words), in a time that follows the length of the chains of overlapping
 // boxes, not the number of candidates of a class.  Up to kSmallMax candidates (the usual case in serving) are
 // one batch; more are bucketed by class first (histogram, scan, scatter) and cut into about as many
-// batches as the image has CTAs; on one CTA many small classes are taken by a warp each instead (kWarpClasses).  Survivors are re-keyed to (inverted score | anchor | class) and put in order
+// batches as the image has CTAs; on one CTA many small classes are taken by a warp each instead (kWarpShare).
+// Survivors are re-keyed to (inverted score | anchor | class) and put in order
 // by counting or by score buckets.
 // us per launch (CUDA events), against one thread per class that walked its candidates (and one warp per
 // class above 256): 200 candidates of one class, 8 images, 16.8 (67.4), of 7 classes 13.9 (28.3), of 80 classes
@@ -57,12 +58,17 @@ constexpr int kCountMax = 96;       // so many survivors are put in order by cou
 constexpr int kSubs = 16;           // score buckets of a class of a crowded image
 constexpr float kSubScale = 20.0f;  // ... of 1 / 20 each; scores below 1/4 share the last
 constexpr int kCountedMax = 128;    // a batch without larger classes orders its candidates by counting
-// An image on one CTA whose largest class is at most 1 / kWarpClasses of its candidates (above kSmallMax) has its
-// classes worked on by one warp each, side by side, instead of in batches one after the other: a warp tests
-// against survivors only.  us per launch, warps (batches): 5000 candidates of 80 classes, one image 61.5 (118),
-// 80 images 80.6 (128); 2000, 200 images 69 (95); 600, 80 images 28.1 (30.2); 3000 of 20 classes, 80 images 92
-// (114).  With fewer, larger classes the batches are better: 1000 of 7 classes, 80 images 62 (53).
-constexpr int kWarpClasses = 5;
+// An image on one CTA whose largest class is at most kWarpShare of its candidates (above kSmallMax) and at most
+// kWarpClassMax candidates has its classes worked on by one warp each, side by side, instead of in batches one
+// after the other: a warp tests against survivors only, but has a class to itself.  Which is better depends on how
+// many boxes survive, which is not known here.  Time of the batches over that of the warps (80 images): boxes in
+// clusters of twenty, 5000 of 80 classes 1.26, 2000 of 10 1.34, 5000 of 7 0.99, 8000 of 10 1.02, of 6 (1340 a class) 0.58; boxes
+// that hardly overlap, 5000 of 80 1.00, 2000 of 10 0.67.  The share lies above a fifth because five classes are rarely
+// even (850 of 5, one image: 41 us in batches, 34 by warps).
+constexpr float kWarpShare = 0.235f;
+constexpr int kWarpClassMax = 1280;
+constexpr int kWarpRankMax = 512;  // up to here a warp orders a class by counting, above by a network (80 images,
+                                   // 8000 candidates of 10 clustered classes: 554 us by counting, 362 so)
 constexpr int kCrowdedMin = 1024;  // an image with more candidates than this wants full-sized CTAs
 
 constexpr size_t kNmsSmemBytes = (size_t)kNmsSmemCap * (sizeof(float4) + sizeof(unsigned long long));
@@ -107,15 +113,19 @@ __device__ __forceinline__ void cmp_swap(unsigned long long* __restrict__ k, int
     if (a > b) { k[i] = b; k[j] = a; }
 }
 
-// Ascending bitonic sort of k[0, m) for any m by the whole CTA.  Every comparator puts the smaller key
-// at the lower index (the first stage of each merge pairs mirrored positions), so positions >= m can
-// stand for +infinity and are simply skipped.
-__device__ __forceinline__ void bitonic_cta(unsigned long long* __restrict__ k, int m, int tid, int nthreads) {
+// Ascending bitonic sort of k[0, m) for any m by the whole CTA or (CTA = false) by one warp.  Every comparator puts
+// the smaller key at the lower index (the first stage of each merge pairs mirrored positions), so positions >= m
+// can stand for +infinity and are simply skipped.
+template <bool CTA>
+__device__ __forceinline__ void bitonic_range(unsigned long long* __restrict__ k, int m, int tid, int nthreads) {
+    auto barrier = []() {
+        if (CTA) __syncthreads(); else __syncwarp();
+    };
     int np2 = 2;
     while (np2 < m) np2 <<= 1;
     const int half = np2 >> 1;
     for (int size = 2; size <= np2; size <<= 1) {
-        __syncthreads();
+        barrier();
         const int h = size >> 1;
         for (int t = tid; t < half; t += nthreads) {
             const int off = t & (h - 1);
@@ -124,7 +134,7 @@ __device__ __forceinline__ void bitonic_cta(unsigned long long* __restrict__ k, 
             if (j < m) cmp_swap(k, i, j);
         }
         for (int stride = size >> 2; stride > 0; stride >>= 1) {
-            __syncthreads();
+            barrier();
             for (int t = tid; t < half; t += nthreads) {
                 const int i = 2 * t - (t & (stride - 1));
                 const int j = i + stride;
@@ -132,7 +142,7 @@ __device__ __forceinline__ void bitonic_cta(unsigned long long* __restrict__ k, 
             }
         }
     }
-    __syncthreads();
+    barrier();
 }
 
 // Box of one anchor; es = distance between consecutive values of an anchor (1 in the rows
@@ -478,6 +488,99 @@ __device__ __forceinline__ int kept_before(const uint2* fate, int words, int lan
     return warp == 0 ? 0 : before;
 }
 
+// One class, the candidates [s, s + m), by one warp: keys ordered, boxes gathered from the head, each candidate tested
+// against the survivors before it.  Survivors (at most max_det) are left at the start, re-keyed; returns their number.
+__device__ __forceinline__ int warp_class(unsigned long long* keys, float4* boxes, int s, int m, int max_det,
+                                          const float* __restrict__ hbase, size_t as, size_t es, const IouTest& test,
+                                          int lane, unsigned int* status) {
+    (void)status;
+    const int e = s + m;
+    if (m > kWarpRankMax) {
+        bitonic_range<false>(keys + s, m, lane, 32);
+    } else if (m > 1) {
+        // every key counts the keys below it and moves to that position, staged in the (not yet used) box slots
+        unsigned long long* const tmp = reinterpret_cast<unsigned long long*>(boxes + s);
+        for (int i0 = lane; i0 < m; i0 += 128) {
+            // up to four keys per lane share one pass over the segment
+            const unsigned long long k0 = keys[s + i0];
+            const unsigned long long k1 = i0 + 32 < m ? keys[s + i0 + 32] : kKeySentinel;
+            const unsigned long long k2 = i0 + 64 < m ? keys[s + i0 + 64] : kKeySentinel;
+            const unsigned long long k3 = i0 + 96 < m ? keys[s + i0 + 96] : kKeySentinel;
+            int r0 = 0, r1 = 0, r2 = 0, r3 = 0;
+            for (int j = 0; j < m; ++j) {
+                const unsigned long long kj = keys[s + j];
+                r0 += kj < k0; r1 += kj < k1; r2 += kj < k2; r3 += kj < k3;
+            }
+            if (OCTO_IN_RANGE(r0 < m, status)) tmp[r0] = k0;
+            if (i0 + 32 < m && OCTO_IN_RANGE(r1 < m, status)) tmp[r1] = k1;
+            if (i0 + 64 < m && OCTO_IN_RANGE(r2 < m, status)) tmp[r2] = k2;
+            if (i0 + 96 < m && OCTO_IN_RANGE(r3 < m, status)) tmp[r3] = k3;
+        }
+        __syncwarp();
+        for (int p = lane; p < m; p += 32) keys[s + p] = tmp[p];
+        __syncwarp();
+    }
+    // four boxes per lane in flight (a lone warp pays the full round trip for every load it waits on)
+    for (int p0 = s + lane; p0 < e; p0 += 128) {
+        float4 b4[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int p = p0 + 32 * u;
+            if (p < e) b4[u] = gather_box(hbase + (size_t)(int)(keys[p] & ((1ull << kKeyAnchorBits) - 1)) * as, es);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int p = p0 + 32 * u;
+            if (p < e) boxes[p] = b4[u];
+        }
+    }
+    __syncwarp();
+    int nk = 0;
+    for (int c0 = s; c0 < e && nk < max_det; c0 += 32) {
+        const int p = c0 + lane;
+        const bool valid = p < e;
+        float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
+        unsigned long long k = kKeySentinel;
+        if (valid) { b = boxes[p]; k = keys[p]; }
+        bool alive = valid;
+        // four survivors per round: the tests of a round are independent of one another, so
+        // their latencies overlap (a lone warp is bound by the dependent chain, not by issue)
+        for (int t = 0; t < nk; t += 4) {
+            if (!__any_sync(0xffffffffu, alive)) break;
+            const float4 k0 = boxes[s + t];
+            const float4 k1 = boxes[s + min(t + 1, nk - 1)];
+            const float4 k2 = boxes[s + min(t + 2, nk - 1)];
+            const float4 k3 = boxes[s + min(t + 3, nk - 1)];
+            bool close = false;
+            bool hit = iou_quick(k0, b, test, close) | iou_quick(k1, b, test, close) | iou_quick(k2, b, test, close) |
+                       iou_quick(k3, b, test, close);
+            if (close) hit = iou_above(k0, b, test) | iou_above(k1, b, test) | iou_above(k2, b, test) | iou_above(k3, b, test);
+            if (hit) alive = false;
+        }
+        unsigned rem = __ballot_sync(0xffffffffu, alive);
+        unsigned keptmask = 0;
+        while (rem) {
+            const int l = __ffs(rem) - 1;
+            keptmask |= 1u << l;
+            const float4 lb = boxes[c0 + l];
+            if (alive && lane > l && iou_above(lb, b, test)) alive = false;
+            rem = __ballot_sync(0xffffffffu, alive) & ~((2u << l) - 1u);
+        }
+        __syncwarp();
+        const int allowed = min(__popc(keptmask), max_det - nk);
+        if ((keptmask >> lane) & 1u) {
+            const int r = __popc(keptmask & ((1u << lane) - 1u));
+            if (r < allowed && OCTO_IN_RANGE(s + nk + r < e, status)) {
+                boxes[s + nk + r] = b;
+                keys[s + nk + r] = global_key(k);
+            }
+        }
+        __syncwarp();
+        nk += allowed;
+    }
+    return nk;
+}
+
 // NMS of image `img` by a CTA of NT threads (SMEM_CAP candidates on chip), or by the cluster the CTA
 // belongs to when CLUSTER.  The image's candidate count, keys and (for the short path) boxes are in
 // global memory.
@@ -646,7 +749,7 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
             {
                 const int4 v = *reinterpret_cast<const int4*>(&seg_cnt[4 * lane]);
                 const int largest = __reduce_max_sync(0xffffffffu, max(max(v.x, v.y), max(v.z, v.w)));
-                const bool by_warps = team_ctas == 1u && kWarpClasses * largest <= cnt;
+                const bool by_warps = team_ctas == 1u && largest <= kWarpClassMax && (float)largest <= kWarpShare * (float)cnt;
                 if (lane == 0) s_by_warps = by_warps;
                 if (by_warps) {  // every class with candidates is listed, none is in a batch
                     scan_classes(lane, seg_cnt, seg_start);
@@ -773,172 +876,92 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
             }
         };
 
-        // ---- classes of at most kTeamMin, a batch of them at a time: one candidate per thread.  (Before the large
-        // classes, whose boxes take the memory of the slots.) ----
-        const int nbatch = s_nbatch;
-        const bool bucketed = on_chip || s_most <= kCountedMax;
-        for (int q = (int)crank; q < nbatch; q += (int)team_ctas) {
-            const int lo = s_lo[q], m = s_hi[q] - lo;
-            if (m <= 0) continue;
-            const BatchMem<NT> mem(smem_raw);
-            unsigned long long key = kKeySentinel;
-            float4 box = make_float4(0.f, 0.f, 0.f, 0.f);
-            int slot = 0;
-            if (tid < m && OCTO_IN_RANGE(m <= NT && lo >= 0 && lo + m <= cnt, status)) {
-                key = keys[lo + tid];
-                if (on_chip) {
-                    slot = slots[lo + tid];
-                    box = __ldcg(gb + slot);
-                } else {
-                    box = gather_box(hbase + (size_t)(key & ((1ull << kKeyAnchorBits) - 1)) * as, es);
-                }
-                mem.skey[tid] = key;
-                mem.rank[tid] = 0;
-            }
-            if (tid == 0) mem.skey[m] = kKeySentinel;  // (m = NT: the first word of the boxes, not read)
-            __syncthreads();
-            nms_batch<NT>(mem, key, box, m, bucketed, P.iou_test, s_fate, status,
-                          [&](int cls) { return seg_start[cls] - lo; },
-                          [&](unsigned long long k, int& from, int& to) {
-                              const int cls = (int)(k >> 57), start = seg_start[cls] - lo, all = seg_cnt[cls];
-                              if (on_chip) {
-                                  const int b = score_bucket(k, kSubs, kSubScale), at = cls * kSubs + b;
-                                  from = start + s_sub[at];
-                                  to = b + 1 < kSubs ? start + s_sub[at + 1] : start + all;
-                              } else {
-                                  from = start;
-                                  to = start + all;
-                              }
-                          });
-            const int words = (m + 31) >> 5;
-            int all = 0;
-            const int before = kept_before(s_fate, words, lane, warp, all);
-            // survivors and their slots: thread c still knows candidate c's slot, and its rank says where it went
-            unsigned short* const sslot = reinterpret_cast<unsigned short*>(mem.sup);
-            if (tid < m) sslot[mem.rank[tid]] = (unsigned short)slot;
-            __syncthreads();
-            const unsigned kept = warp < words ? s_fate[warp].x : 0u;
-            if ((kept >> lane) & 1u) {
-                const int at = lo + before + __popc(kept & ((1u << lane) - 1u)), cand = batch_cand(tid);
-                keys0[at] = global_key(mem.skey[cand]);
-                // (a large class's boxes may take the first CTA's slots)
-                if (on_chip && s_nlarge == 0) slots0[at] = sslot[cand];
-            }
-            if (tid == 0) {
-                kept0[q] = all;
-                atomicAdd(total0, all);
-            }
-            __syncthreads();
-        }
-
         // ---- many small classes on one CTA: one warp each, handed out by a counter ----
         if (s_by_warps) {
-            const int nclasses = s_nlarge;
-            for (;;) {
-                int q = 0;
-                if (lane == 0) q = atomicAdd(&s_next, 1);
-                q = __shfl_sync(0xffffffffu, q, 0);
-                if (q >= nclasses) break;
-                const int cls = s_large[q], m = seg_cnt[cls];
-                const int s = seg_start[cls], e = s + m;
-                if (m > 1) {
-                    // every key counts the keys below it and moves to that position, staged in the (not yet
-                    // used) box slots of the segment
-                    unsigned long long* const tmp = reinterpret_cast<unsigned long long*>(boxes + s);
-                    for (int i0 = lane; i0 < m; i0 += 128) {
-                        // up to four keys per lane share one pass over the segment
-                        const unsigned long long k0 = keys[s + i0];
-                        const unsigned long long k1 = i0 + 32 < m ? keys[s + i0 + 32] : kKeySentinel;
-                        const unsigned long long k2 = i0 + 64 < m ? keys[s + i0 + 64] : kKeySentinel;
-                        const unsigned long long k3 = i0 + 96 < m ? keys[s + i0 + 96] : kKeySentinel;
-                        int r0 = 0, r1 = 0, r2 = 0, r3 = 0;
-                        for (int j = 0; j < m; ++j) {
-                            const unsigned long long kj = keys[s + j];
-                            r0 += kj < k0; r1 += kj < k1; r2 += kj < k2; r3 += kj < k3;
-                        }
-                        tmp[r0] = k0;
-                        if (i0 + 32 < m) tmp[r1] = k1;
-                        if (i0 + 64 < m) tmp[r2] = k2;
-                        if (i0 + 96 < m) tmp[r3] = k3;
-                    }
-                    __syncwarp();
-                    for (int p = lane; p < m; p += 32) keys[s + p] = tmp[p];
-                    __syncwarp();
+            auto by_warps = [&](unsigned long long* k, float4* b) {
+                const int nclasses = s_nlarge;
+                for (;;) {
+                    int q = 0;
+                    if (lane == 0) q = atomicAdd(&s_next, 1);
+                    q = __shfl_sync(0xffffffffu, q, 0);
+                    if (q >= nclasses) break;
+                    const int cls = s_large[q];
+                    const int nk = warp_class(k, b, seg_start[cls], seg_cnt[cls], max_det, hbase, as, es, P.iou_test, lane, status);
+                    finish_class(cls, seg_start[cls], nk, lane, 32);
                 }
-                // boxes of the class from the head, four per lane in flight (a lone warp pays the full
-                // round trip for every load it waits on)
-                for (int p0 = s + lane; p0 < e; p0 += 128) {
-                    float4 b4[4];
-    #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int p = p0 + 32 * u;
-                        if (p < e) {
-                            const int anchor = (int)(keys[p] & ((1ull << kKeyAnchorBits) - 1));
-                            b4[u] = gather_box(hbase + (size_t)anchor * as, es);
-                        }
-                    }
-    #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int p = p0 + 32 * u;
-                        if (p < e) boxes[p] = b4[u];
-                    }
-                }
-                __syncwarp();
-                int nk = 0;  // survivors of this class, compacted at [s, s + nk)
-                for (int c0 = s; c0 < e && nk < max_det; c0 += 32) {
-                    const int p = c0 + lane;
-                    const bool valid = p < e;
-                    float4 b = make_float4(0.f, 0.f, 0.f, 0.f);
-                    unsigned long long k = kKeySentinel;
-                    if (valid) { b = boxes[p]; k = keys[p]; }
-                    bool alive = valid;
-                    // four survivors per round: the tests of a round are independent of one another, so
-                    // their latencies overlap (a lone warp is bound by the dependent chain, not by issue)
-                    for (int t = 0; t < nk; t += 4) {
-                        if (!__any_sync(0xffffffffu, alive)) break;
-                        const float4 k0 = boxes[s + t];
-                        const float4 k1 = boxes[s + min(t + 1, nk - 1)];
-                        const float4 k2 = boxes[s + min(t + 2, nk - 1)];
-                        const float4 k3 = boxes[s + min(t + 3, nk - 1)];
-                        bool close = false;
-                        bool hit = iou_quick(k0, b, P.iou_test, close) | iou_quick(k1, b, P.iou_test, close) |
-                                   iou_quick(k2, b, P.iou_test, close) | iou_quick(k3, b, P.iou_test, close);
-                        if (close)
-                            hit = iou_above(k0, b, P.iou_test) | iou_above(k1, b, P.iou_test) |
-                                  iou_above(k2, b, P.iou_test) | iou_above(k3, b, P.iou_test);
-                        if (hit) alive = false;
-                    }
-                    unsigned rem = __ballot_sync(0xffffffffu, alive);
-                    unsigned keptmask = 0;
-                    while (rem) {
-                        const int l = __ffs(rem) - 1;
-                        keptmask |= 1u << l;
-                        const float4 lb = boxes[c0 + l];
-                        if (alive && lane > l && iou_above(lb, b, P.iou_test)) alive = false;
-                        rem = __ballot_sync(0xffffffffu, alive) & ~((2u << l) - 1u);
-                    }
-                    __syncwarp();
-                    const int allowed = min(__popc(keptmask), max_det - nk);
-                    if ((keptmask >> lane) & 1u) {
-                        const int r = __popc(keptmask & ((1u << lane) - 1u));
-                        if (r < allowed && OCTO_IN_RANGE(s + nk + r < e, status)) {
-                            boxes[s + nk + r] = b;
-                            keys[s + nk + r] = global_key(k);
-                        }
-                    }
-                    __syncwarp();
-                    nk += allowed;
-                }
-                finish_class(cls, s, nk, lane, 32);
-            }
+            };
+            // (in the half-sized form the code for pointers of shared memory alone is 5 to 10 % faster than the code for
+            // both, in the full-sized form 10 % slower)
+            if (NT == kNmsThreadsFull) by_warps(keys, boxes);
+            else if (on_chip) by_warps(reinterpret_cast<unsigned long long*>(smem_raw + (size_t)SMEM_CAP * sizeof(float4)),
+                                      reinterpret_cast<float4*>(smem_raw));
+            else by_warps(gk, P.gboxes + (size_t)img * P.key_stride);
         } else {
+            // ---- classes of at most kTeamMin, a batch of them at a time: one candidate per thread.  (Before the large
+            // classes, whose boxes take the memory of the slots.) ----
+            const int nbatch = s_nbatch;
+            const bool bucketed = on_chip || s_most <= kCountedMax;
+            for (int q = (int)crank; q < nbatch; q += (int)team_ctas) {
+                const int lo = s_lo[q], m = s_hi[q] - lo;
+                if (m <= 0) continue;
+                const BatchMem<NT> mem(smem_raw);
+                unsigned long long key = kKeySentinel;
+                float4 box = make_float4(0.f, 0.f, 0.f, 0.f);
+                int slot = 0;
+                if (tid < m && OCTO_IN_RANGE(m <= NT && lo >= 0 && lo + m <= cnt, status)) {
+                    key = keys[lo + tid];
+                    if (on_chip) {
+                        slot = slots[lo + tid];
+                        box = __ldcg(gb + slot);
+                    } else {
+                        box = gather_box(hbase + (size_t)(key & ((1ull << kKeyAnchorBits) - 1)) * as, es);
+                    }
+                    mem.skey[tid] = key;
+                    mem.rank[tid] = 0;
+                }
+                if (tid == 0) mem.skey[m] = kKeySentinel;  // (m = NT: the first word of the boxes, not read)
+                __syncthreads();
+                nms_batch<NT>(mem, key, box, m, bucketed, P.iou_test, s_fate, status,
+                              [&](int cls) { return seg_start[cls] - lo; },
+                              [&](unsigned long long k, int& from, int& to) {
+                                  const int cls = (int)(k >> 57), start = seg_start[cls] - lo, all = seg_cnt[cls];
+                                  if (on_chip) {
+                                      const int b = score_bucket(k, kSubs, kSubScale), at = cls * kSubs + b;
+                                      from = start + s_sub[at];
+                                      to = b + 1 < kSubs ? start + s_sub[at + 1] : start + all;
+                                  } else {
+                                      from = start;
+                                      to = start + all;
+                                  }
+                              });
+                const int words = (m + 31) >> 5;
+                int all = 0;
+                const int before = kept_before(s_fate, words, lane, warp, all);
+                // survivors and their slots: thread c still knows candidate c's slot, and its rank says where it went
+                unsigned short* const sslot = reinterpret_cast<unsigned short*>(mem.sup);
+                if (tid < m) sslot[mem.rank[tid]] = (unsigned short)slot;
+                __syncthreads();
+                const unsigned kept = warp < words ? s_fate[warp].x : 0u;
+                if ((kept >> lane) & 1u) {
+                    const int at = lo + before + __popc(kept & ((1u << lane) - 1u)), cand = batch_cand(tid);
+                    keys0[at] = global_key(mem.skey[cand]);
+                    // (a large class's boxes may take the first CTA's slots)
+                    if (on_chip && s_nlarge == 0) slots0[at] = sslot[cand];
+                }
+                if (tid == 0) {
+                    kept0[q] = all;
+                    atomicAdd(total0, all);
+                }
+                __syncthreads();
+            }
+
             // ---- large classes, by all warps of a CTA ----
             __shared__ unsigned t_sup[kTeamBlock * kTeamWords];
             const int nlarge = s_nlarge;
             for (int q = (int)crank; q < nlarge; q += (int)team_ctas) {
                 const int cls = s_large[q], m = seg_cnt[cls];
                 const int s = seg_start[cls], e = s + m;
-                bitonic_cta(keys + s, m, tid, NT);
+                bitonic_range<true>(keys + s, m, tid, NT);
                 for (int p = s + tid; p < e; p += NT)
                     boxes[p] = gather_box(hbase + (size_t)(keys[p] & ((1ull << kKeyAnchorBits) - 1)) * as, es);
                 int nk = 0;
@@ -1040,7 +1063,7 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
             if (have_slots) boxes_at = gb;
         } else {
             ordered = packed;
-            bitonic_cta(ordered, total, tid, NT);
+            bitonic_range<true>(ordered, total, tid, NT);
         }
     }
     if (P.class_agnostic) {

@@ -82,14 +82,23 @@ def test_large_classes(m, share, cluster):
 
 
 @pytest.mark.parametrize("m,share,kind,max_det", [(513, 0.0, "grid", 300), (513, 0.19, "grid", 1000), (2000, 0.21, "grid", 1000),
+                                                  (2000, 0.25, "grid", 1000),
                                                   (1500, 0.0, "chain", 2), (1900, 0.0, "apart", 2000),
                                                   (900, 0.0, "same", 300), (8192, 0.1, "grid", 1000),
                                                   (8300, 0.0, "grid", 1000)])
 def test_many_classes_on_one_cta(m, share, kind, max_det):
-    """Classes of at most a fifth of the image: one warp per class (one of more: batches); full-sized CTAs and,
+    """Classes of less than a quarter of the image: one warp per class (one of more: batches); full-sized CTAs and,
     with more images than SMs, half-sized ones."""
     for batch in (1, 160) if m <= 2000 else (1,):
         _check(m, kind, share, cluster=1, max_det=max_det, classes=40, batch=batch)
+
+
+@pytest.mark.parametrize("m,classes,share", [(2600, 5, 0.0), (4200, 8, 0.0), (2600, 20, 0.16), (8192, 7, 0.0),
+                                             (8192, 6, 0.0), (9000, 8, 0.0), (9000, 6, 0.1)])
+@pytest.mark.parametrize("kind", ["grid", "powers"])
+def test_a_warp_orders_a_class_by_a_network(m, classes, share, kind):
+    """Classes of 512 to 1280 candidates on one CTA, on chip and off; the largest classes go to the whole CTA."""
+    _check(m, kind, share, cluster=1, max_det=1000, classes=classes)
 
 
 @pytest.mark.parametrize("m,max_det", [(120, 5), (256, 300), (600, 5), (600, 1), (1100, 70)])
