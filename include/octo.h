@@ -385,10 +385,10 @@ OCTO_API int octo_stage_kernel_times(octo_stage_t* st, octo_kernel_times_t* time
 /* CTAs per image of the NMS launches (paper Section III-C: a stage is scheduled by its latency,
  * and a crowded scene served at a small batch leaves most of the GPU idle with one CTA per image).
  * cluster = 0 (the default): automatic.  The stage gives every image a thread-block cluster of 2,
- * 4 or 8 CTAs while the batch has at most a half, a quarter or an eighth as many images as the GPU
- * has SMs and an image with more than 512 candidates was reported lately: for 64 launches from
- * the call that finds the report (the kernel reports through mapped host memory; nothing is copied or
- * synchronised, so the report of a launch may arrive a few calls late).  cluster =
+ * 4 or 8 CTAs, the largest size of which the GPU holds one for each image of the batch at once, while an
+ * image with more than 512 candidates was reported lately: for 64 launches from the call that finds the
+ * report (the kernel reports through mapped host memory; nothing is copied or synchronised, so the report
+ * of a launch may arrive a few calls late).  cluster =
  * 1, 2, 4, 8: that size for every launch (clamped to what the device can co-schedule).  Results do
  * not depend on the size.  OCTO_E_INVALID_ARG for any other value. */
 OCTO_API int octo_stage_set_nms_cluster(octo_stage_t* st, int32_t cluster);

@@ -100,9 +100,9 @@ int report_cuda_error(cudaError_t e, const char* what);
 // Opt the kernels of every table capacity into the shared memory they need (current device).
 cudaError_t prepare_letterbox();
 cudaError_t prepare_decode();
-// max_cluster (optional): the largest cluster of the NMS kernel (8, 4, 2 or 1) that the current
-// device can co-schedule.
-cudaError_t prepare_nms(int* max_cluster = nullptr);
+// clusters (optional): how many clusters of 2, 4 and 8 CTAs of the NMS kernel the current device holds at once.
+constexpr int kNmsClusterSizes = 3;
+cudaError_t prepare_nms(int* clusters = nullptr);
 cudaError_t prepare_crop();
 
 cudaError_t launch_letterbox(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,

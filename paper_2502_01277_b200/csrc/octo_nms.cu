@@ -52,7 +52,7 @@ static NmsParams nms_params(const NmsArgs& a) {
     return p;
 }
 
-cudaError_t prepare_nms(int* max_cluster) {
+cudaError_t prepare_nms(int* clusters) {
     cudaError_t e;
     e = cudaFuncSetAttribute(nms_kernel<8, kNmsThreadsFull>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNmsSmemBytes);
     if (e != cudaSuccess) return e;
@@ -62,11 +62,10 @@ cudaError_t prepare_nms(int* max_cluster) {
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(nms_kernel<512, kNmsThreadsHalf>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNmsSmemBytesHalf);
     if (e != cudaSuccess) return e;
-    if (max_cluster) {
-        // the largest cluster (one CTA per SM: the kernel takes nearly all shared memory of an SM)
-        // of which the device can hold at least one
-        *max_cluster = 1;
-        for (int c = 8; c > 1; c >>= 1) {
+    if (clusters) {
+        // (one CTA per SM: the kernel takes nearly all shared memory of an SM)
+        for (int k = 0; k < kNmsClusterSizes; ++k) {
+            const int c = 2 << k;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)c);
             cfg.blockDim = dim3(kNmsThreadsFull);
@@ -78,12 +77,11 @@ cudaError_t prepare_nms(int* max_cluster) {
             attr[0].val.clusterDim.z = 1;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            int active = 0;
-            if (cudaOccupancyMaxActiveClusters(&active, nms_kernel<8, kNmsThreadsFull>, &cfg) == cudaSuccess && active > 0) {
-                *max_cluster = c;
-                break;
+            clusters[k] = 0;
+            if (cudaOccupancyMaxActiveClusters(&clusters[k], nms_kernel<8, kNmsThreadsFull>, &cfg) != cudaSuccess) {
+                clusters[k] = 0;
+                (void)cudaGetLastError();
             }
-            (void)cudaGetLastError();
         }
     }
     return cudaSuccess;

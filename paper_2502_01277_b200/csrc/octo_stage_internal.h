@@ -36,7 +36,7 @@ struct octo_stage {
     // ([0]) and with more than the short path takes, 512 ([1]).  For kNmsClusterWindow launches from the one
     // that finds a report, launches with few images give every image a cluster of CTAs ([1]) and launches
     // with many keep to full-sized CTAs ([0]).
-    int nms_max_cluster;
+    int nms_clusters[octo::kNmsClusterSizes];  // how many clusters of 2, 4, 8 CTAs the device holds at once
     int nms_cluster_mode;  // 0 automatic, else the caller's size
     int nms_cluster_last;  // size of the latest launch
     bool nms_half_last;    // the latest launch ran two half-sized CTAs per SM

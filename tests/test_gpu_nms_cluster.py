@@ -62,6 +62,23 @@ def test_more_candidates_than_fit_on_chip_under_a_cluster():
         st.close()
 
 
+@pytest.mark.parametrize("n,most", [(15, 8), (18, 4), (37, 2), (75, 1)])
+def test_automatic_size_is_one_wave_of_clusters(n, most):
+    """n clusters of the size chosen for n crowded images run at once.  A B200 holds 15 clusters of 8 and 33 of
+    4, fewer than its 148 SMs would make."""
+    from test_gpu_parity import _check_dets
+    b = _batch(700, 60, n)
+    st = make_stage(b.workload, b.n)
+    try:
+        ref = _oracle_dets(b)
+        for i in range(2):
+            res = run_stage_gpu(st, b.frames, b.sizes, b.head, max_items=[8])  # synchronises
+            _check_dets(res, ref)
+        assert 1 <= st.last_nms_cluster() <= most and (n > 37 or st.last_nms_cluster() > 1)
+    finally:
+        st.close()
+
+
 def test_automatic_choice_follows_the_candidate_counts():
     from test_gpu_parity import _check_dets
     dense = _batch(5000, 250, 2, max_det=1000)
