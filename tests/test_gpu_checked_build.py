@@ -158,3 +158,14 @@ def test_half_sized_nms_ctas_under_the_checked_build(checked):
     NMS module; it asserts the launch forms and parity, the status word is checked there too)."""
     from test_gpu_nms_cluster import test_more_images_than_sms_run_two_half_sized_ctas_per_sm as case
     case()
+
+
+@pytest.mark.parametrize("sizes_of,batch", [((6500, *[100] * 25), 1), ((6500, 500, 450, 400, 350, 300, 100, 400), 1),
+                                            ((3500, 250, 256, 200, 257, 190, 150, 200), 160), ((1024, 512, 256, 129, 3), 160),
+                                            ([900] * 8, 1), ([1125] * 8, 1)])
+def test_nms_ways_under_the_checked_build(checked, sizes_of, batch):
+    """Batches and whole-CTA classes of images beyond the chip, half-sized CTAs, classes a warp orders by a network.
+    (The comparison requires a status word without any other bit.)"""
+    from test_gpu_nms_forms import _check
+    _check(sum(sizes_of), "grid", 0.0, classes=len(sizes_of), sizes_of=sizes_of, max_det=1000, batch=batch, crowded=2,
+           half=batch > 1)
