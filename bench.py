@@ -43,17 +43,17 @@ NCU_TRAFFIC = {
     # kernel: (source files, sha256[:16] of their code (comments and layout stripped) at capture time, bytes per unit, unit)
     # captured on the sweep workload at B = 64; decode_planes on the anchor_free workload at B = 64
     "crop": (("paper_2502_01277_b200/csrc/octo_crop.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-             "cb3b58cf225f647f", 487791.2, "crop"),
+             "614ff9e83b927477", 491013.2, "crop"),
     "letterbox": (("paper_2502_01277_b200/csrc/octo_letterbox.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-                  "82ba43ca31895b9a", 3706404.0, "frame"),
+                  "382ad8f271898953", 3693716.0, "frame"),
     "decode": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-               "5ec9cd6b248b8101", 1740516.0, "frame"),
+               "5b5bd9b48466c54a", 1740264.0, "frame"),
     "decode_planes": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-                      "5ec9cd6b248b8101", 2810668.0, "frame"),
+                      "5b5bd9b48466c54a", 2817000.0, "frame"),
 }
 # Warp instructions the crop kernel executes per crop (ncu smsp__inst_executed.sum of the same capture):
-# the kernel is bound by instruction issue, so its issue rate is reported beside the byte rates.
-NCU_CROP_WARP_INST = 84255.7
+# its issue rate is reported beside the byte rates (two thirds of the issue slots are used).
+NCU_CROP_WARP_INST = 83008.2
 
 
 def parse_args():
@@ -572,14 +572,15 @@ def run_octo(args):
         "frac_dram": (traffic / (dom_ms * 1e-3) / 1e9 / hbm_peak) if traffic else None,
     }
     if dominant == "crop":
-        # What limits the kernel in practice: instruction issue (ncu: issue slots about 70 % busy, no
-        # memory pipe above 60 %).  Issue rate = executed warp instructions / time against one
+        # What limits the kernel in practice is latency inside a unit of work at the 24 warps an SM holds (ncu: 1.5
+        # warps of a scheduler eligible, issue slots 65 % and shared-memory wavefronts 76 % busy, DRAM 52 %).
+        # Issue rate = executed warp instructions / time against one
         # instruction per scheduler and clock (4 schedulers per SM) at the clock seen during the run.
         sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
         mhz = clocks.get("sm_mhz") or peaks.get("sm_max_mhz") or 1965.0
         inst = NCU_CROP_WARP_INST * units if traffic else None
         roofline["issue"] = {
-            "limits_the_kernel": True, "warp_inst_per_launch": inst,
+            "limits_the_kernel": False, "warp_inst_per_launch": inst,
             "achieved_ginst_s": inst / (dom_ms * 1e-3) / 1e9 if inst else None,
             "peak_ginst_s": sm_count * 4 * mhz * 1e6 / 1e9,
             "frac": (inst / (dom_ms * 1e-3)) / (sm_count * 4 * mhz * 1e6) if inst else None,

@@ -3,7 +3,8 @@
 // HBM-bound scan.  For logit heads sigma <= 1 makes sigma(obj) > conf a necessary condition
 // for score = fl(sigma(obj) * sigma(cls)) > conf, so the scan reads only the obj value of
 // each 340-byte row (one DRAM sector) and fetches the whole row, 32 bytes at a time by a group
-// of eight lanes (four passing rows per warp in flight together), for the few anchors that pass.  Probability heads are read densely (decode_dense_kernel, where a 16-byte boundary allows it).  A passing row is
+// of eight lanes (four passing rows per warp in flight together), for the few anchors that pass.
+// Probability heads are read densely (decode_dense_kernel, where a 16-byte boundary allows it).  A passing row is
 // reduced by eight lanes (finite check, first-maximum class), scored in the fixed binary32
 // sequence and appended to the image's key list with one atomic; the key carries class,
 // inverted score bits and anchor, so later steps need nothing else from this kernel and the
@@ -153,7 +154,8 @@ decode_kernel(const float* __restrict__ head, int A, int C, int mode, float conf
                 // one candidate per class whose own score passes; the keys of a row go out in
                 // groups of up to eight with one counter update per group
                 const float so = logits ? sigmoid_fixed(ob) : ob;
-                const float4 box = box_corners(__shfl_sync(0xffffffffu, e0, gbase), __shfl_sync(0xffffffffu, e0, gbase + 1), bw, bh);
+                const float4 box = box_corners(__shfl_sync(0xffffffffu, e0, gbase), __shfl_sync(0xffffffffu, e0, gbase + 1),
+                                               bw, bh);
                 for (int e0i = 0; e0i < row_len; e0i += 8) {  // the same trip count in every group
                     const int e = e0i + gl;
                     float score = 0.0f;

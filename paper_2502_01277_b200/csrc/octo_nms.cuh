@@ -6,13 +6,15 @@
 //
 // Candidates are worked on in batches of whole classes, one thread (or up to four) per candidate
 // (nms_batch): put in order (by counting inside a class, or inside its score bucket; where one is large, words
-// of 32 by counting, then every candidate's place in every word by binary search); each tested against the earlier candidates of its class (one bit each); which survive is settled
-// word by word of those bits (resolve_words), in a time that follows the length of the chains of overlapping
+// of 32 by counting, then every candidate's place in every word by binary search); each tested against the
+// earlier candidates of its class (one bit each); which survive is settled word by word of those bits
+// (resolve_words), in a time that follows the length of the chains of overlapping
 // boxes, not the number of candidates of a class.  Up to kSmallMax candidates (the usual case in serving) are
 // one batch; more are bucketed by class first (histogram, scan, scatter) and cut into about as many
 // batches as the image has CTAs; on one CTA many small classes are taken by a warp each instead (kWarpShare).
-// Survivors are re-keyed to (inverted score | anchor | class) and put in order
-// by counting or by score buckets.
+// Survivors are re-keyed to (inverted score | anchor | class) and put in order by counting, by score buckets or
+// (more than threads) by a network.  Boxes: as the decode step left them beside the keys for the short path, for
+// batches on chip and for records while no class went to a warp or to the whole CTA; from the head otherwise.
 // us per launch (CUDA events), against one thread per class that walked its candidates (and one warp per
 // class above 256): 200 candidates of one class, 8 images, 16.8 (67.4), of 7 classes 13.9 (28.3), of 80 classes
 // 12.7 (12.6); 90 candidates under class-agnostic NMS 12.7 (35.7); 5000 candidates of 80 classes, one image
@@ -264,10 +266,9 @@ struct RegionMap {
 };
 
 // Finds the place of the m (<= NT) survivors in list / lpos in the output order: emit(place, key, pos), one
-// thread per survivor.  Few by counting; more
-// are dealt to 256 buckets by score first and counted inside their bucket (766 survivors of a crowded image:
-// 8 K cycles; 28 K with a network over all of them).  list has room for a pad; tmp: NT + 2 keys, rank: NT integers.  All threads of the CTA; ends with
-// a barrier.
+// thread per survivor.  Few by counting; more are dealt to 256 buckets by score first and counted inside their
+// bucket (766 survivors of a crowded image: 8 K cycles; 28 K with a network over all of them).  list has room for
+// a pad; tmp: NT + 2 keys, rank: NT integers.  All threads of the CTA; ends with a barrier.
 template <int NT, typename Emit>
 __device__ __forceinline__ void order_survivors(unsigned long long* list, const unsigned short* lpos, int m,
                                                 unsigned long long* tmp, int* rank, int tid, Emit emit) {
@@ -1103,7 +1104,8 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
                 corner = reinterpret_cast<const float*>(boxes_at + opos[r])[k];
             } else {
                 const float* __restrict__ row = hbase + (size_t)((g >> 7) & ((1ull << kKeyAnchorBits) - 1)) * as;
-                const float centre = __ldg(row + (size_t)(k & 1) * es), half = __fmul_rn(0.5f, __ldg(row + (size_t)(2 + (k & 1)) * es));
+                const float centre = __ldg(row + (size_t)(k & 1) * es);
+                const float half = __fmul_rn(0.5f, __ldg(row + (size_t)(2 + (k & 1)) * es));
                 corner = k < 2 ? __fsub_rn(centre, half) : __fadd_rn(centre, half);  // as box_corners
             }
         }

@@ -386,9 +386,11 @@ extern "C" int octo_adopt_items_device(octo_stage_t* st, const octo_stage_t* ups
     st->have_dets = false;
     cudaError_t e;
     const int un = upstream->tab_on_device ? 1 : upstream->n_frames;
-    if (un <= 8) e = launch_adopt<8>(upstream, upstream->d_items[branch], upstream->d_last_n_items[branch], first, n, st->cfg.net_size, st->d_tab, stream);
-    else if (un <= 64) e = launch_adopt<64>(upstream, upstream->d_items[branch], upstream->d_last_n_items[branch], first, n, st->cfg.net_size, st->d_tab, stream);
-    else e = launch_adopt<512>(upstream, upstream->d_items[branch], upstream->d_last_n_items[branch], first, n, st->cfg.net_size, st->d_tab, stream);
+    const octo_item_t* const items = upstream->d_items[branch];
+    const int32_t* const n_items = upstream->d_last_n_items[branch];
+    if (un <= 8) e = launch_adopt<8>(upstream, items, n_items, first, n, st->cfg.net_size, st->d_tab, stream);
+    else if (un <= 64) e = launch_adopt<64>(upstream, items, n_items, first, n, st->cfg.net_size, st->d_tab, stream);
+    else e = launch_adopt<512>(upstream, items, n_items, first, n, st->cfg.net_size, st->d_tab, stream);
     if (e != cudaSuccess) return cuda_fail(e, "adopt_items_kernel");
     st->launches += 1;
     st->tab_on_device = true;
