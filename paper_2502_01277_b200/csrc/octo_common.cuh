@@ -373,9 +373,12 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst_smem, const void* src_gmem
 __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {
     bulk_g2s(smem_u32(dst_smem), src_gmem, bytes, smem_u32(bar));
 }
-// A value that is the same in every lane of a converged warp (or zero in the others), in a register that
-// the warp shares.
-__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __reduce_or_sync(0xffffffffu, v); }
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t one;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(one));
+    return one != 0;
+}
 
 // ---------------------------------------------------------------------------------------
 // Fixed binary32 arithmetic shared by decode and NMS.  Every operation is an explicitly

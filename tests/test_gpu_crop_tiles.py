@@ -54,3 +54,9 @@ def test_row_bands(count):
 def test_tall_and_wide_crops(count, batch):
     """At 900 x 3 crops every crop is one tile, except the last ones."""
     _check(count, ((16, 97), (264, 8), (40, 64)), batch)
+
+
+@pytest.mark.parametrize("first", [1, 5, 9, 13])
+def test_rows_of_a_pass_four_at_a_time(first):
+    """Passes of few rows: the source rows are requested four at a time, the last one to three by themselves."""
+    _check(9, tuple((8, first + i) for i in range(4)))
