@@ -252,7 +252,8 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
     return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// One output row (or column tile of it) by one warp: lane l owns the pixel pairs l, l + 32, ...
+// One output row (or column tile of it) by one or more warps: lane l of warp `part` of `parts` owns the pixel
+// pairs l + 32 part, l + 32 (part + parts), ...
 // so neighbouring lanes read neighbouring table entries and row words (no bank conflicts)
 // and the warp writes 128 contiguous bytes per plane and step.  row0 / xt are shared-space
 // addresses of the first staged row and of the tile's first table entry; o0 / o1 / o2 point
@@ -261,10 +262,10 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b) {
 // (fill_h2 holds it in both halves).
 template <bool LERP_Y, bool FILL>
 __device__ __forceinline__ void sample_row(uint32_t row0, uint32_t row_step, float wx, float wy, uint32_t xt,
-                                           int pairs, int lane, __half* __restrict__ o0, __half* __restrict__ o1,
-                                           __half* __restrict__ o2, uint32_t fill_h2) {
+                                           int pairs, int lane, int part, int parts, __half* __restrict__ o0,
+                                           __half* __restrict__ o1, __half* __restrict__ o2, uint32_t fill_h2) {
     const float nwx = -kF32IntValue * wx;
-    for (int pair = lane; pair < pairs; pair += 32) {
+    for (int pair = lane + 32 * part; pair < pairs; pair += 32 * parts) {
         const uint4 ee = lds128(xt + 16u * (uint32_t)pair);  // two XEntry: {off, wts} x 2
         unsigned long long p0, p1, p2;
         sample_pair<LERP_Y>(row0, row_step, ee.x, ee.y, ee.z, ee.w, wx, nwx, wy, p0, p1, p2);

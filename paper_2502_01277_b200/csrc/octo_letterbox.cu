@@ -1,6 +1,6 @@
 // Letterbox kernel: n BGR uint8 frames -> fp16 NCHW [n, 3, S, S] detector batch.
 //
-// HBM-bound gather.  One CTA produces kRows output rows of one frame.  The source rows
+// HBM-bound gather.  One CTA produces up to kLbRows output rows of one frame.  The source rows
 // those output rows tap (one row where the vertical weight is zero, e.g. the 3:1 reduction
 // of 1080p, else two) are fetched whole into shared memory by the bulk-copy (TMA) engine
 // with 16-byte coalesced transactions and an mbarrier; rows that carry no weight are never
@@ -16,26 +16,27 @@ namespace octo {
 
 constexpr int kLbThreads = 256;
 constexpr int kLbRows = 8;  // most output rows a CTA produces; fewer for very wide frames
+static_assert(kLbRows <= kLbThreads / 32, "a warp for every row of a CTA");
 
+// A warp stages its own output row, behind a barrier of its own, and waits for nothing else but the table of taps;
+// where a CTA has fewer rows than warps (small batches), several warps share a row.  What needs no memory (barriers,
+// which rows are tapped) comes before the wait for the previous kernel.  Large batches are bound by HBM, small
+// ones by this chain: against one thread that walked the rows twice and issued every copy, and one barrier for all
+// of them, a pass over one small frame went from 18.1 to 17.1 us, one camera 24.2 / 23.5, eight 55.7 / 53.6, thirteen
+// 1277x717 frames 36.6 / 34.9, 32 frames 220 / 219, 256 frames unchanged.
 template <int CAP>
 __global__ void __launch_bounds__(kLbThreads)
 letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict__ out, int S, int band_rows,
-                 int slot_bytes, int nslots, uint32_t fill_h2, int swap_rb, unsigned int* __restrict__ status) {
+                 int slot_bytes, int row_slots, int share, uint32_t fill_h2, int swap_rb, unsigned int* __restrict__ status) {
     extern __shared__ __align__(128) unsigned char smem[];
-    pdl_wait();
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ __align__(16) RowInfo s_row[kLbRows];  // per-row data; step < 0 marks a canvas (pad) row
+    __shared__ __align__(8) uint64_t bar[kLbRows];
 
     const FrameDesc& fd = tab.f[blockIdx.y];
     const int dy0 = blockIdx.x * band_rows;
     const int w = fd.w, h = fd.h, nw = fd.nw, nh = fd.nh, pad_l = fd.pad_l, pad_t = fd.pad_t;
-    const float inv_dx = 1.0f / (float)(2 * nw), inv_dy = 1.0f / (float)(2 * nh);
-    // every scale factor folded into the vertical weights: 1 / (255 * den_x * den_y)
-    const float inv_all = 1.0f / (255.0f * (float)(2 * nw) * (float)(2 * nh));
     const int chunks = S >> 3;
     const size_t plane = (size_t)S * (size_t)S;
     __half* const out_img = out + (size_t)blockIdx.y * 3 * plane;
-    const uint4 fill4 = make_uint4(fill_h2, fill_h2, fill_h2, fill_h2);
     const int nrows = min(band_rows, S - dy0);
     // the staged rows start after the table of horizontal taps
     XEntry* const s_xtab = reinterpret_cast<XEntry*>(smem);
@@ -44,6 +45,8 @@ letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict
     // Does this band touch the image at all?
     const bool any_image = max(dy0, pad_t) < min(dy0 + nrows, pad_t + nh);
     if (!any_image) {
+        pdl_wait();
+        const uint4 fill4 = make_uint4(fill_h2, fill_h2, fill_h2, fill_h2);
         for (int t = threadIdx.x; t < nrows * chunks; t += kLbThreads) {
             const int r = t / chunks;
             __half* const o0 = out_img + (size_t)(dy0 + r) * S + ((t - r * chunks) << 3);
@@ -54,52 +57,40 @@ letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict
         return;
     }
 
-    if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
+    if (threadIdx.x < kLbRows) mbar_init(&bar[threadIdx.x], 1);
+    // this warp's row, and its share of it
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int parts = 1 << share, r = warp >> share, part = warp & (parts - 1);
+    const int iy = dy0 + r - pad_t;
+    const bool image = r < nrows && iy >= 0 && iy < nh;  // else a canvas row, or none
+    int y0 = 0, ry = 0;
+    if (image) src_coord(iy, h, nh, 1.0f / (float)(2 * nh), y0, ry);
+    if (threadIdx.x < kLbRows) {
         mbar_fence_init();
         fence_proxy_async();
+    }
+    __syncthreads();  // barriers ready
+    pdl_wait();
+    const uint32_t rows_s = smem_u32(s_rows) + (uint32_t)(r * row_slots * slot_bytes);
+    if (image && part == 0 && elect_one()) {
         const uint32_t row_bytes = (uint32_t)((3 * w + 15) & ~15);
-        uint32_t total = 0;
-        int slot = 0;
-        for (int r = 0; r < nrows; ++r) {
-            const int iy = dy0 + r - pad_t;
-            RowInfo ri;
-            ri.row0 = 0; ri.step = -1; ri.wx = 0.0f; ri.wy = 0.0f;
-            if (iy < 0 || iy >= nh) { s_row[r] = ri; continue; }
-            int y0, ry;
-            src_coord(iy, h, nh, inv_dy, y0, ry);
-            ri.row0 = slot * slot_bytes;
-            ri.step = slot_bytes;
-            ri.wx = (float)(2 * nh - ry) * inv_all;
-            ri.wy = (float)ry * inv_all;
-            s_row[r] = ri;
-            slot += ry != 0 ? 2 : 1;
-            total += row_bytes * (ry != 0 ? 2u : 1u);
-        }
-        mbar_expect_tx(&bar, total);
-        slot = 0;
-        for (int r = 0; r < nrows; ++r) {
-            const int iy = dy0 + r - pad_t;
-            if (iy < 0 || iy >= nh) continue;
-            int y0, ry;
-            src_coord(iy, h, nh, inv_dy, y0, ry);
-            const uint8_t* src = fd.data + (size_t)y0 * (size_t)fd.pitch;
+        const uint8_t* const src = fd.data + (size_t)y0 * (size_t)fd.pitch;
+        mbar_expect_tx(&bar[r], ry != 0 ? 2u * row_bytes : row_bytes);
+        bool ok = true;
 #ifdef OCTO_BOUNDS_CHECK
-            if (!OCTO_IN_RANGE(slot + (ry != 0 ? 2 : 1) <= nslots && (int)row_bytes + 16 <= slot_bytes &&
-                               y0 + (ry != 0 ? 1 : 0) < h && (int)row_bytes <= fd.pitch, status)) {
-                // keep the barrier's byte count right without touching memory
-                asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bar)),
-                             "r"(row_bytes * (ry != 0 ? 2u : 1u)) : "memory");
-                slot += ry != 0 ? 2 : 1;
-                continue;
-            }
+        ok = OCTO_IN_RANGE((ry != 0 ? 2 : 1) <= row_slots && (int)row_bytes + 16 <= slot_bytes && y0 + (ry != 0 ? 1 : 0) < h &&
+                           (int)row_bytes <= fd.pitch, status);
+        if (!ok)  // keep the barrier's byte count right without touching memory
+            asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&bar[r])),
+                         "r"(row_bytes * (ry != 0 ? 2u : 1u)) : "memory");
 #endif
-            bulk_g2s(s_rows + (size_t)slot * slot_bytes, src, row_bytes, &bar);
-            if (ry != 0) bulk_g2s(s_rows + (size_t)(slot + 1) * slot_bytes, src + fd.pitch, row_bytes, &bar);
-            slot += ry != 0 ? 2 : 1;
+        if (ok) {
+            bulk_g2s(rows_s, src, row_bytes, smem_u32(&bar[r]));
+            if (ry != 0) bulk_g2s(rows_s + (uint32_t)slot_bytes, src + fd.pitch, row_bytes, smem_u32(&bar[r]));
         }
     }
     // table of horizontal taps, built while the copies are in flight
+    const float inv_dx = 1.0f / (float)(2 * nw);
     for (int dx = threadIdx.x; dx < S; dx += kLbThreads) {
         const int ix = dx - pad_l;
         XEntry e;
@@ -107,33 +98,28 @@ letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict
         else e = make_xentry<false>(ix, w, nw, inv_dx, 0);
         s_xtab[dx] = e;
     }
-    __syncthreads();  // barrier armed, table and row weights visible
-    const bool copy_ok = mbar_wait_or_report(&bar, 0, status);
+    __syncthreads();  // table visible
+    if (r >= nrows) return;
 
-    // one warp per output row of the band
     const int pairs = S >> 1;
-    const int lane = threadIdx.x & 31;
-    const uint32_t rows_s = smem_u32(s_rows), xtab_s = smem_u32(s_xtab);
-    __half* const out0 = out_img + (swap_rb ? 2 : 0) * plane;  // plane of input channel 0
-    __half* const out1 = out_img + plane;
-    __half* const out2 = out_img + (swap_rb ? 0 : 2) * plane;  // plane of input channel 2
-    for (int r = threadIdx.x >> 5; r < nrows; r += kLbThreads / 32) {
-        const RowInfo ri = s_row[r];
-        const size_t o = (size_t)(dy0 + r) * S;
-        if (ri.step < 0 || !copy_ok) {
-            for (int pair = lane; pair < pairs; pair += 32) {
-                *reinterpret_cast<uint32_t*>(out0 + o + 2 * pair) = fill_h2;
-                *reinterpret_cast<uint32_t*>(out1 + o + 2 * pair) = fill_h2;
-                *reinterpret_cast<uint32_t*>(out2 + o + 2 * pair) = fill_h2;
-            }
-        } else if (ri.wy != 0.0f) {
-            sample_row<true, true>(rows_s + (uint32_t)ri.row0, (uint32_t)ri.step, ri.wx, ri.wy, xtab_s, pairs, lane,
-                                   out0 + o, out1 + o, out2 + o, fill_h2);
-        } else {
-            sample_row<false, true>(rows_s + (uint32_t)ri.row0, (uint32_t)ri.step, ri.wx, ri.wy, xtab_s, pairs, lane,
-                                    out0 + o, out1 + o, out2 + o, fill_h2);
+    const size_t o = (size_t)(dy0 + r) * S;
+    __half* const o0 = out_img + (swap_rb ? 2 : 0) * plane + o;  // plane of input channel 0
+    __half* const o1 = out_img + plane + o;
+    __half* const o2 = out_img + (swap_rb ? 0 : 2) * plane + o;  // plane of input channel 2
+    if (!image || !mbar_wait_or_report(&bar[r], 0, status)) {
+        for (int pair = lane + 32 * part; pair < pairs; pair += 32 * parts) {
+            *reinterpret_cast<uint32_t*>(o0 + 2 * pair) = fill_h2;
+            *reinterpret_cast<uint32_t*>(o1 + 2 * pair) = fill_h2;
+            *reinterpret_cast<uint32_t*>(o2 + 2 * pair) = fill_h2;
         }
+        return;
     }
+    // every scale factor folded into the vertical weights: 1 / (255 * den_x * den_y)
+    const float inv_all = 1.0f / (255.0f * (float)(2 * nw) * (float)(2 * nh));
+    const float wx = (float)(2 * nh - ry) * inv_all, wy = (float)ry * inv_all;
+    const uint32_t xtab_s = smem_u32(s_xtab);
+    if (ry != 0) sample_row<true, true>(rows_s, (uint32_t)slot_bytes, wx, wy, xtab_s, pairs, lane, part, parts, o0, o1, o2, fill_h2);
+    else sample_row<false, true>(rows_s, (uint32_t)slot_bytes, wx, wy, xtab_s, pairs, lane, part, parts, o0, o1, o2, fill_h2);
 }
 
 // Staging slots an output row needs: one when every row of every frame taps a single source
@@ -165,6 +151,8 @@ static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S
     band_rows = band_rows < 1 ? 1 : (band_rows > kLbRows ? kLbRows : band_rows);
     // small batches: fewer rows per CTA so that the grid still covers the SMs about twice
     while (band_rows > 2 && (long long)n * ((S + band_rows - 1) / band_rows) < 296) band_rows >>= 1;
+    int share = 0;  // 2^share warps to a row
+    while ((band_rows << (share + 1)) <= kLbThreads / 32) ++share;
     const size_t smem = lb_smem_bytes(S, band_rows * slots_per_row(frames, n), slot_bytes);
     const __half hf = __double2half((double)pad_value / 255.0);  // one rounding, nearest even
     const uint32_t fb = *reinterpret_cast<const unsigned short*>(&hf);
@@ -172,7 +160,7 @@ static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S
     dim3 grid((S + band_rows - 1) / band_rows, n);
     return launch_kernel(letterbox_kernel<CAP>, grid, dim3(kLbThreads), smem, stream, tab,
                          reinterpret_cast<__half*>(d_out), S, band_rows, slot_bytes,
-                         band_rows * slots_per_row(frames, n), fill_h2, swap_rb, d_status);
+                         slots_per_row(frames, n), share, fill_h2, swap_rb, d_status);
 }
 
 // largest dynamic shared memory a launch may ask for (see kLetterboxMaxWidth)
