@@ -149,8 +149,10 @@ static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S
     const long long room = 56 * 1024 - (long long)lb_smem_bytes(S, 0, slot_bytes);
     int band_rows = (int)(room / per_row);
     band_rows = band_rows < 1 ? 1 : (band_rows > kLbRows ? kLbRows : band_rows);
-    // small batches: fewer rows per CTA so that the grid still covers the SMs about twice
-    while (band_rows > 2 && (long long)n * ((S + band_rows - 1) / band_rows) < 296) band_rows >>= 1;
+    // small batches: fewer rows per CTA, whose warps share them, until there are four (of eight rows: eight) CTAs per
+    // SM.  Four 720p frames 46.3 -> 45.5 us a pass against two CTAs per SM (two rows each 47.5), eight 1080p 53.7 ->
+    // 53.1, thirteen 1277x717 34.7 -> 33.7; single rows are no faster (one camera) or slower (two, 32.8 -> 33.5)
+    while (band_rows > 2 && (long long)n * ((S + band_rows - 1) / band_rows) < (band_rows > 4 ? 1184 : 592)) band_rows >>= 1;
     int share = 0;  // 2^share warps to a row
     while ((band_rows << (share + 1)) <= kLbThreads / 32) ++share;
     const size_t smem = lb_smem_bytes(S, band_rows * slots_per_row(frames, n), slot_bytes);
