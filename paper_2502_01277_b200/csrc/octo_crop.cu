@@ -344,12 +344,16 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
         // The first kCropTilesAhead tiles of a CTA are fixed (block index + j * grid size) and
         // resolved up front, lane j resolving tile j, so that their round trips overlap: with few
         // tiles per CTA (small batches) the chain is paid once, not once per tile.
-        const Tile ahead = resolve(lane < kCropTilesAhead ? (int)blockIdx.x + lane * (int)gridDim.x : all_tiles);
+        // (Three where that is all of them: a CTA then need not ask the counter to learn that nothing is left; one
+        // camera 24.2 -> 24.0 us a pass, thirteen 1277x717 frames with crops of 96x33 33.3 -> 32.8.)
+        const int fixed = all_tiles <= (kCropTilesAhead + 1) * (int)gridDim.x ? kCropTilesAhead + 1 : kCropTilesAhead;
+        const bool drawing = all_tiles > fixed * (int)gridDim.x;
+        const Tile ahead = resolve(lane < fixed ? (int)blockIdx.x + lane * (int)gridDim.x : all_tiles);
         // first pass of the next tile, if there is one
         auto open_tile = [&]() {
             Tile t;
-            if (w_tiles < kCropTilesAhead) {
-                const int src = w_tiles;
+            if (w_tiles < fixed || !drawing) {
+                const int src = w_tiles;  // (lane `fixed` holds no tile)
                 t.ok = __shfl_sync(0xffffffffu, ahead.ok, src);
                 t.slot = __shfl_sync(0xffffffffu, ahead.slot, src);
                 t.band = __shfl_sync(0xffffffffu, ahead.band, src);
