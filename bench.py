@@ -43,17 +43,17 @@ NCU_TRAFFIC = {
     # kernel: (source files, sha256[:16] of their code (comments and layout stripped) at capture time, bytes per unit, unit)
     # captured on the sweep workload at B = 64; decode_planes on the anchor_free workload at B = 64
     "crop": (("paper_2502_01277_b200/csrc/octo_crop.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-             "614ff9e83b927477", 491013.2, "crop"),
+             "e7cf1d68ed38ac44", 490656.1, "crop"),
     "letterbox": (("paper_2502_01277_b200/csrc/octo_letterbox.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-                  "382ad8f271898953", 3693716.0, "frame"),
+                  "e01b273567d36b8b", 3686080.0, "frame"),
     "decode": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-               "5b5bd9b48466c54a", 1740264.0, "frame"),
+               "ad62776268f5859a", 1740604.0, "frame"),
     "decode_planes": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-                      "5b5bd9b48466c54a", 2817000.0, "frame"),
+                      "ad62776268f5859a", 2810520.0, "frame"),
 }
 # Warp instructions the crop kernel executes per crop (ncu smsp__inst_executed.sum of the same capture):
 # its issue rate is reported beside the byte rates (two thirds of the issue slots are used).
-NCU_CROP_WARP_INST = 83008.2
+NCU_CROP_WARP_INST = 84129.8
 
 
 def parse_args():
