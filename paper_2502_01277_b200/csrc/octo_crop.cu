@@ -155,7 +155,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
     __shared__ __align__(8) uint64_t full[kCropStages], empty[kCropStages];
     __shared__ CropPass s_pass[kCropStages];
     __shared__ __align__(16) RowInfo s_row[kCropStages][kCropMaxPassRows];  // per-row data of the staged passes
-    __shared__ __align__(16) uint32_t s_src[2 * kCropMaxPassRows + 4];  // where the rows of a pass lie in their frame, four read ahead
+    __shared__ __align__(16) uint32_t s_src[2 * kCropMaxPassRows + 4];  // the source rows of a pass, four read ahead
     __shared__ int s_off[CAP + 1];                                // exclusive scan of the frame counts
     __shared__ int4 s_first;  // of the first tile: left edge (-1: no tile), width, fitted width, left offset
 
@@ -518,8 +518,8 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             __syncwarp();  // table, pass record and row data are written before the barrier is armed
             if (lane == 0) mbar_expect_tx(&full[b], (uint32_t)(staged * w_seg));
             __syncwarp();
-            // One bulk copy per row, issued by one elected lane from a list of where the rows lie, four at a time
-            // and without a condition among the four; the next four offsets are read while these go out.  (Copies
+            // One bulk copy per row, issued by one elected lane from a list of row numbers, four at a time and
+            // without a condition among the four; the next four numbers are read while these go out.  (Copies
             // that every lane issues for itself go out one lane after the other, 97 cycles each beside the
             // consumers; so they take 66, and 32 crowds, whose small crops wait for the producer, 1173 us a pass
             // instead of 1228.  With a condition on every copy of the loop 115 cycles, 1299 us; a loop of the whole warp with
@@ -530,7 +530,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                 // the new rows are the last `newrows` of {y0, y0 + 1}
                 const int first_new = need2 + 1 - newrows;  // 0: y0 is new, 1: only y0 + 1
                 const int slot_new = slot_top + first_new;
-                const uint32_t at = (uint32_t)(w_ry0 + y0 + first_new) * (uint32_t)w_pitch;
+                const uint32_t y_new = (uint32_t)(w_ry0 + y0 + first_new);
 #ifdef OCTO_BOUNDS_CHECK
                 bad = !OCTO_IN_RANGE(slot_new >= 0 && slot_new + newrows <= w_cap_slots &&
                                      slot_new + newrows <= 2 * kCropMaxPassRows &&
@@ -539,8 +539,8 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                                      w_seg_lo + w_seg <= w_pitch && (w_seg & 15) == 0, status);
 #endif
                 if (!bad) {
-                    s_src[slot_new] = at;
-                    if (newrows == 2) s_src[slot_new + 1] = at + (uint32_t)w_pitch;
+                    s_src[slot_new] = y_new;
+                    if (newrows == 2) s_src[slot_new + 1] = y_new + 1u;
                 }
             }
             __syncwarp();
@@ -557,20 +557,21 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                 const uint8_t* const base = w_data + w_seg_lo;
                 const uint32_t bar = smem_u32(&full[b]), seg = (uint32_t)w_seg, stride = (uint32_t)w_stride;
                 uint32_t list = smem_u32(s_src), dst = smem_u32(s_rows0) + (uint32_t)(b * kCropRowBudget);
+                auto row = [&](uint32_t y) { return base + (uint64_t)y * (uint32_t)w_pitch; };  // (a frame may span more than 4 GiB)
                 uint4 at = lds128(list);
                 int left = staged;
                 for (; left >= 4; left -= 4, dst += 4u * stride) {
                     list += 16u;
                     const uint4 next = lds128(list);
-                    bulk_g2s(dst, base + at.x, seg, bar);
-                    bulk_g2s(dst + stride, base + at.y, seg, bar);
-                    bulk_g2s(dst + 2u * stride, base + at.z, seg, bar);
-                    bulk_g2s(dst + 3u * stride, base + at.w, seg, bar);
+                    bulk_g2s(dst, row(at.x), seg, bar);
+                    bulk_g2s(dst + stride, row(at.y), seg, bar);
+                    bulk_g2s(dst + 2u * stride, row(at.z), seg, bar);
+                    bulk_g2s(dst + 3u * stride, row(at.w), seg, bar);
                     at = next;
                 }
-                if (left > 0) bulk_g2s(dst, base + at.x, seg, bar);
-                if (left > 1) bulk_g2s(dst + stride, base + at.y, seg, bar);
-                if (left > 2) bulk_g2s(dst + 2u * stride, base + at.z, seg, bar);
+                if (left > 0) bulk_g2s(dst, row(at.x), seg, bar);
+                if (left > 1) bulk_g2s(dst + stride, row(at.y), seg, bar);
+                if (left > 2) bulk_g2s(dst + 2u * stride, row(at.z), seg, bar);
             }
             __syncwarp();
             advance(nr);
