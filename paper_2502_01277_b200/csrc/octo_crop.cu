@@ -37,15 +37,15 @@
 
 namespace octo {
 
-// Shared memory for staged source rows.  A row segment longer than kCropMaxStride - 16 bytes
+// Shared memory for staged source rows.  A row segment longer than half a ring buffer less 16 bytes
 // (a rectangle wider than about 5300 pixels) is split into column tiles, so two rows always
 // fit.  Two buffers form a ring between the producer warp and the consumer warps.
 constexpr int kCropStages = 2;         // ring depth (row buffers)
 constexpr int kCropTables = kCropStages + 1;  // tap tables, one more than ring slots
-constexpr int kCropRowBudget = 32768;  // bytes per ring buffer
-constexpr int kCropMaxStride = kCropRowBudget / 2;
+constexpr int kCropRowBudget = 32768;  // bytes per ring buffer (see crop_layout)
 constexpr int kCropTilePx = 5300;
 constexpr int kCropMaxPassRows = 32;   // one producer lane per output row of a pass
+constexpr int kCropListBytes = 4 * 2 * kCropMaxPassRows;  // a pass's source rows
 constexpr int kCropCtasPerSm = 3;
 constexpr int kCropConsumerWarps = 7;   // with the producer warp 8 warps: 80 registers a thread at 3 CTAs per SM
 constexpr int kCropConsumers = 32 * kCropConsumerWarps;
@@ -66,6 +66,49 @@ struct __align__(16) CropPass {
     int32_t units;     // ... and (run, two column pairs) units are dealt to the consumer threads
     int32_t _pad[2];
 };
+
+// Static shared memory of a CTA; n <= CAP frames.
+template <int CAP>
+struct CropShared {
+    uint64_t full[kCropStages], empty[kCropStages];
+    int4 first;  // of the first tile: left edge (-1: no tile), width, fitted width, left offset
+    CropPass pass[kCropStages];
+    RowInfo row[kCropStages][kCropMaxPassRows];  // per-row data of the staged passes
+    int off[CAP + 1];  // exclusive scan of the frame counts
+};
+
+// Dynamic shared memory: the ring buffers, at kCropStages * kCropRowBudget the tap tables, and the list
+// of a pass's source rows behind them, or between the two where the ring buffers make room for it.
+struct CropLayout {
+    int row_budget, list_at, bytes;
+};
+constexpr bool crop_ctas_fit(int bytes) {  // three CTAs of so much shared memory and the 1024 bytes the system takes
+    return kCropCtasPerSm * ((bytes + 1024 + 127) & ~127) <= 228 * 1024;
+}
+// The grid is sized for three CTAs per SM, which the shared memory allows up to a certain crop width.  At the last of
+// these widths the list would cost the third CTA (and with it a second wave: 29 crops of 416x416 16.9 -> 23.4 us, 184 of
+// them 42 -> 54), so there the ring buffers make room for it; elsewhere they keep their 32 KB, since a staged row less
+// in a pass of six costs 11 % (rectangles 1800 pixels wide).  (Static memory counts in steps of 128 bytes here: with the
+// exact size a third CTA would fit at 408 columns and 9 to 64 frames too, 23 % slower for small rectangles, 20 % faster
+// for others.)
+template <int CAP>
+constexpr CropLayout crop_layout(int out_w) {
+    const int fixed = (int)sizeof(CropShared<CAP>);
+    const int tables_end = kCropStages * kCropRowBudget + kCropTables * (int)sizeof(XEntry) * out_w;
+    const int tight = kCropRowBudget - kCropListBytes / kCropStages;
+    if (crop_ctas_fit(((fixed + 127) & ~127) + tables_end) && !crop_ctas_fit(fixed + tables_end + kCropListBytes))
+        return {tight, kCropStages * tight, tables_end};
+    return {kCropRowBudget, tables_end, tables_end + kCropListBytes};
+}
+template <int CAP>
+constexpr bool crop_shortened(int out_w) { return crop_layout<CAP>(out_w).row_budget != kCropRowBudget; }
+template <int CAP>
+constexpr bool crop_three(int out_w) { return crop_ctas_fit((int)sizeof(CropShared<CAP>) + crop_layout<CAP>(out_w).bytes); }
+static_assert(crop_three<1>(416) && crop_three<8>(416) && crop_three<64>(400) && crop_three<512>(328),
+              "widest crops of which an SM holds three CTAs");
+static_assert(!crop_three<1>(424) && !crop_three<8>(424) && !crop_three<64>(408) && !crop_three<512>(336), "and the next");
+static_assert(!crop_shortened<1>(408) && !crop_shortened<8>(408) && !crop_shortened<64>(392) && !crop_shortened<512>(320) &&
+              crop_shortened<8>(416) && !crop_shortened<8>(424), "only the last width shortens the ring buffers");
 
 // Per output row of a staged pass (RowInfo): row0 = byte offset of the staged copy of the top
 // tap row, relative to the ring buffer and to the tap table's offsets; step = kRowStep bits:
@@ -150,17 +193,18 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             int* __restrict__ offsets, int* __restrict__ n_items, octo_item_t* __restrict__ items,
             __half* __restrict__ out, int ow, int oh, int swap_rb, StageCounters* __restrict__ ctr,
             const QRecord* __restrict__ qrec, const int* __restrict__ qpacked, unsigned int* __restrict__ qstatus,
-            int* __restrict__ sched, const CropOpts opts) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ __align__(8) uint64_t full[kCropStages], empty[kCropStages];
-    __shared__ CropPass s_pass[kCropStages];
-    __shared__ __align__(16) RowInfo s_row[kCropStages][kCropMaxPassRows];  // per-row data of the staged passes
-    __shared__ __align__(16) uint32_t s_src[2 * kCropMaxPassRows + 4];  // the source rows of a pass, four read ahead
-    __shared__ int s_off[CAP + 1];                                // exclusive scan of the frame counts
-    __shared__ int4 s_first;  // of the first tile: left edge (-1: no tile), width, fitted width, left offset
+            int* __restrict__ sched, const CropOpts opts, int row_budget, int list_at) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ __align__(16) CropShared<CAP> sh;
+    auto &full = sh.full, &empty = sh.empty;
+    auto& s_pass = sh.pass;
+    auto& s_row = sh.row;
+    auto& s_off = sh.off;
+    auto& s_first = sh.first;
 
     unsigned char* const s_rows0 = smem;
     XEntry* const s_xtab0 = reinterpret_cast<XEntry*>(smem + kCropStages * kCropRowBudget);  // kCropTables tables of ow entries
+    uint32_t* const s_src = reinterpret_cast<uint32_t*>(smem + list_at);
     unsigned int* const status = QUEUE ? qstatus : &ctr->status;
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -285,7 +329,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             w_seg_lo = lo;
             w_seg = hi - lo;
             w_stride = w_seg + 16;
-            w_cap_slots = div_small(kCropRowBudget, w_stride);  // >= 2
+            w_cap_slots = div_small(row_budget, w_stride);  // >= 2
             // Work units of a pass: (run of consecutive rows, two column pairs half a tile apart).
             // A pass is cut into as many runs as fit the consumer threads side by side (224
             // columns: 4 runs x 56 units = the 224 consumer threads).
@@ -409,7 +453,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             }
             const int full_seg = ((3 * rx1 + 15) & ~15) - ((3 * rx0) & ~15);
             w_tile_cols =
-                (full_seg + 16 > kCropMaxStride) ? max(4, (int)((long long)kCropTilePx * w_nw / w_cw) & ~3) : ow;
+                (full_seg + 16 > row_budget >> 1) ? max(4, (int)((long long)kCropTilePx * w_nw / w_cw) & ~3) : ow;
             w_c0 = 0;
             set_tile();
             w_row_lo = w_band * w_band_rows;
@@ -534,7 +578,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
 #ifdef OCTO_BOUNDS_CHECK
                 bad = !OCTO_IN_RANGE(slot_new >= 0 && slot_new + newrows <= w_cap_slots &&
                                      slot_new + newrows <= 2 * kCropMaxPassRows &&
-                                     (slot_new + newrows) * w_stride <= kCropRowBudget &&
+                                     (slot_new + newrows) * w_stride <= row_budget &&
                                      w_ry0 + y0 + first_new + newrows <= w_fh && w_seg_lo >= 0 &&
                                      w_seg_lo + w_seg <= w_pitch && (w_seg & 15) == 0, status);
 #endif
@@ -556,12 +600,13 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             if (elect_one()) {
                 const uint8_t* const base = w_data + w_seg_lo;
                 const uint32_t bar = smem_u32(&full[b]), seg = (uint32_t)w_seg, stride = (uint32_t)w_stride;
-                uint32_t list = smem_u32(s_src), dst = smem_u32(s_rows0) + (uint32_t)(b * kCropRowBudget);
+                uint32_t list = smem_u32(s_src), dst = smem_u32(s_rows0) + (uint32_t)(b * row_budget);
+                const uint32_t list_end = list + (uint32_t)kCropListBytes - 16u;
                 auto row = [&](uint32_t y) { return base + (uint64_t)y * (uint32_t)w_pitch; };  // (a frame may span more than 4 GiB)
                 uint4 at = lds128(list);
                 int left = staged;
                 for (; left >= 4; left -= 4, dst += 4u * stride) {
-                    list += 16u;
+                    list = min(list + 16u, list_end);  // (read ahead, but not past the end)
                     const uint4 next = lds128(list);
                     bulk_g2s(dst, row(at.x), seg, bar);
                     bulk_g2s(dst + stride, row(at.y), seg, bar);
@@ -599,7 +644,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             const CropPass cur = s_pass[b];
             if (!cur.valid) break;
             const uint32_t xt = smem_u32(s_xtab0) + (uint32_t)(cur.table * ow + cur.c0) * (uint32_t)sizeof(XEntry);
-            const uint32_t rows = smem_u32(s_rows0) + (uint32_t)b * kCropRowBudget;
+            const uint32_t rows = smem_u32(s_rows0) + (uint32_t)(b * row_budget);
             const uint32_t rinfo = smem_u32(&s_row[b][0]);
             const size_t tile_off = (size_t)cur.slot * 3 * plane + (size_t)cur.r0 * ow + cur.c0;
             __half* const t0 = out0 + tile_off;
@@ -655,7 +700,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                         const uint32_t omax = max(max(ea.x & ~3u, ea.z & ~3u), max(eb.x & ~3u, eb.z & ~3u));
                         const long long lo = (long long)(int)rw.x + (long long)omin;
                         const long long hi = (long long)(int)rw.x + (long long)omax + step + 12;
-                        if (!OCTO_IN_RANGE(lo >= 0 && hi <= kCropRowBudget && r < kCropMaxPassRows &&
+                        if (!OCTO_IN_RANGE(lo >= 0 && hi <= row_budget && r < kCropMaxPassRows &&
                                            cur.slot >= 0 && cur.slot < max_items && cur.r0 + r < oh &&
                                            cur.c0 + 2 * (quad + quads) + 1 < ow, status))
                             continue;
@@ -726,10 +771,6 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
     }
 }
 
-static size_t crop_smem_bytes(int out_w) {
-    return (size_t)kCropStages * kCropRowBudget + (size_t)kCropTables * sizeof(XEntry) * (size_t)out_w;
-}
-
 static int crop_grid(int sm_count, int slots, int out_h) {
     // The kernel cuts crops into row bands itself once it knows how many items there are; the
     // grid only has to be large enough for the finest cut.
@@ -745,16 +786,17 @@ static cudaError_t launch_crop_cap(const CropArgs& a, cudaStream_t stream) {
     if (!a.d_tab)
         for (int i = 0; i < a.n; ++i) tab.f[i] = a.frames[i];
     const int grid = crop_grid(a.sm_count, a.max_items, a.out_h);
-    const size_t smem = crop_smem_bytes(a.out_w);
+    const CropLayout layout = crop_layout<CAP>(a.out_w);
     auto kernel = a.general ? crop_kernel<CAP, false, true> : crop_kernel<CAP, false, false>;
-    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, tab, a.d_tab, a.n,
+    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), (size_t)layout.bytes, stream, tab, a.d_tab, a.n,
                          a.max_det, a.first_item, a.max_items, a.d_bcount, a.d_bidx, a.d_dets, a.d_offsets, a.d_n_items,
                          a.d_items, reinterpret_cast<__half*>(a.d_out), a.out_w, a.out_h, a.swap_rb, a.d_ctr,
-                         (const QRecord*)nullptr, (const int*)nullptr, (unsigned int*)nullptr, a.d_ctr->sched, a.opts);
+                         (const QRecord*)nullptr, (const int*)nullptr, (unsigned int*)nullptr, a.d_ctr->sched, a.opts,
+                         layout.row_budget, layout.list_at);
 }
 
 cudaError_t prepare_crop() {
-    const int smem = (int)crop_smem_bytes(2048);
+    const int smem = crop_layout<512>(2048).bytes;
     cudaError_t e;
     const void* kernels[] = {
         (const void*)crop_kernel<8, false, false>,   (const void*)crop_kernel<8, false, true>,
@@ -785,16 +827,16 @@ cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int
     FrameTable<1> tab;  // unused in queue mode
     memset(&tab, 0, sizeof(tab));
     const int grid = crop_grid(sm_count, bz, out_h);
-    const size_t smem = crop_smem_bytes(out_w);
+    const CropLayout layout = crop_layout<1>(out_w);
     CropOpts opts;
     memset(&opts, 0, sizeof(opts));
     if (general) opts = *general;
     auto kernel = general ? crop_kernel<1, true, true> : crop_kernel<1, true, false>;
-    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), smem, stream, tab,
+    return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), (size_t)layout.bytes, stream, tab,
                          (const FrameDesc*)nullptr, 0, 0, 0, bz, (const int*)nullptr, (const int*)nullptr,
                          (const octo_det_t*)nullptr, (int*)nullptr, (int*)nullptr, (octo_item_t*)nullptr,
                          reinterpret_cast<__half*>(d_out), out_w, out_h, swap_rb, (StageCounters*)nullptr, d_staged,
-                         d_qpacked, d_status, d_sched, opts);
+                         d_qpacked, d_status, d_sched, opts, layout.row_budget, layout.list_at);
 }
 
 }  // namespace octo

@@ -169,3 +169,9 @@ def test_nms_ways_under_the_checked_build(checked, sizes_of, batch):
     from test_gpu_nms_forms import _check
     _check(sum(sizes_of), "grid", 0.0, classes=len(sizes_of), sizes_of=sizes_of, max_det=1000, batch=batch, crowded=2,
            half=batch > 1)
+
+
+@pytest.mark.parametrize("batch,widths", [(1, (408, 416)), (9, (392, 400)), (65, (320, 328))])
+def test_widest_crops_of_three_ctas(checked, batch, widths):
+    from test_gpu_crop_tiles import test_widest_crops_of_three_ctas as run
+    run(batch, widths)

@@ -4,6 +4,7 @@ widths below and above what one pass of the threads covers.  Every crop is compa
 the distance of one binary16 step (values below 1); slots past the last crop stay untouched."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2502_01277_b200 as octo
@@ -60,3 +61,57 @@ def test_tall_and_wide_crops(count, batch):
 def test_rows_of_a_pass_four_at_a_time(first):
     """Passes of few rows: the source rows are requested four at a time, the last one to three by themselves."""
     _check(9, tuple((8, first + i) for i in range(4)))
+
+
+@pytest.mark.parametrize("batch,widths", [(1, (400, 408, 416, 424)), (9, (384, 392, 400, 408)), (65, (312, 320, 328, 336))])
+def test_widest_crops_of_three_ctas(batch, widths):
+    """Widths around the last of which an SM holds three CTAs, where the ring buffers are shorter: rectangles of which a
+    pass stages from two rows to all it needs."""
+    w, h, net = 2400, 160, 640
+    scale, top = w / net, (net - 43) / 2
+    rects = [(0, 2400), (100, 2170), (310, 1800), (500, 1790), (800, 1330), (900, 500), (30, 330), (1700, 90), (2300, 40)]
+    rng = np.random.default_rng(batch)
+    frames = [rng.integers(0, 256, (h, 3 * w), dtype=np.uint8) for _ in range(batch)]
+    head = np.zeros((batch, len(rects), 6), dtype=np.float32)
+    for i, (x, width) in enumerate(rects):
+        head[:, i] = (x + width / 2) / scale, top + 20, width / scale, 36 if i % 2 else 8, 1.0, 0.9 - 0.02 * i
+    crops = tuple((width, 24) for width in widths)
+    st = octo.Stage(net_size=net, max_batch=batch, num_anchors=len(rects), num_classes=1, head_is_logits=False,
+                    iou_thresh=1.0, branches=crops)
+    try:
+        ref = oracle.run_stage(frames, [(w, h)] * batch, head, net, crops, logits=False, iou_thr=1.0, do_letterbox=False,
+                               threads=8)
+        total = len(rects) * batch
+        res = run_stage_gpu(st, frames, [(w, h)] * batch, head, max_items=[total] * len(crops))
+        _check_dets(res, ref)
+        assert res.status == 0
+        for k in range(len(crops)):
+            assert res.n_items[k] == (total, total)
+            assert half_absdiff(res.crops[k], ref.crops[k]) <= PIX_TOL
+    finally:
+        st.close()
+
+
+@pytest.mark.parametrize("width", [408, 416, 424])
+def test_widest_queued_crops_of_three_ctas(width):
+    w, h, net, rects = 2400, 160, 640, [(0, 2400), (310, 1800), (500, 1790), (30, 330)]
+    frame = np.random.default_rng(width).integers(0, 256, (h, 3 * w), dtype=np.uint8)
+    head = np.zeros((1, len(rects), 6), dtype=np.float32)
+    for i, (x, side) in enumerate(rects):
+        head[0, i] = (x + side / 2) * net / w, net / 2, side * net / w, 36 if i % 2 else 8, 1.0, 0.9 - 0.02 * i
+    st = octo.Stage(net_size=net, max_batch=1, num_anchors=len(rects), num_classes=1, head_is_logits=False, iou_thresh=1.0,
+                    branches=((8, 8),))
+    q = octo.Queue(64, width, 24, max_bz=8)
+    try:
+        st.preprocess([torch.from_numpy(frame).cuda()], [(w, h)])
+        dets, counts = st.postprocess(torch.from_numpy(head).cuda())
+        q.push(st, 0)
+        out, _, info = q.pop(8)
+        d, c = octo.dets_to_numpy(dets, counts)
+        assert c[0] == len(rects) and int(info[0]) == len(rects)
+        got = out.view(torch.int16).cpu().numpy().view(np.uint16)
+        for i in range(len(rects)):
+            assert half_absdiff(got[i], oracle.crop(frame, w, h, d[0, i:i + 1], width, 24)) <= PIX_TOL
+    finally:
+        q.close()
+        st.close()
