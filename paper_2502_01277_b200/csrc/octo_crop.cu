@@ -482,7 +482,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
         int tb = kCropTables - 1;
         for (int k = 0;; ++k) {
             const int b = k % kCropStages;
-            // ---- prepare the pass in registers; nothing of ring slot b is touched yet ----
+            // ---- prepare the pass in registers and its list; nothing of ring slot b is touched yet ----
             if (w_valid && w_new) {
                 // taps of every output column: byte offset inside a frame row + integer weights.
                 // Tables rotate with the tiles.  There is one more table than ring slots: the
@@ -541,34 +541,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             p.run_rows = w_runs > 1 ? (int)__umulhi((uint32_t)(nr + w_runs - 1), w_run_magic) : nr;
             p.units = (w_ncols >> 2) * w_runs;
             p._pad[0] = 0; p._pad[1] = 0;
-            // ---- ring slot b: wait until the consumers have finished the pass that used it ----
-            if (k >= kCropStages) {
-                const uint32_t par = (ephase >> b) & 1u;
-                if (!mbar_wait_sleeping(&empty[b], par, kCropProducerSleepNs) &&
-                    !mbar_wait_sleeping(&empty[b], par, kCropProducerSleepNs)) {
-                    atomicOr(status, 0x4u);
-                    break;
-                }
-                ephase ^= 1u << b;
-            }
-            if (lane == 0) s_pass[b] = p;
-            if (!w_valid) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&full[b]);  // the end-of-work record
-                break;
-            }
-            if (in_pass) s_row[b][lane] = ri;
-            fence_proxy_async();
-            __syncwarp();  // table, pass record and row data are written before the barrier is armed
-            if (lane == 0) mbar_expect_tx(&full[b], (uint32_t)(staged * w_seg));
-            __syncwarp();
-            // One bulk copy per row, issued by one elected lane from a list of row numbers, four at a time and
-            // without a condition among the four; the next four numbers are read while these go out.  (Copies
-            // that every lane issues for itself go out one lane after the other, 97 cycles each beside the
-            // consumers; so they take 66, and 32 crowds, whose small crops wait for the producer, 1173 us a pass
-            // instead of 1228.  With a condition on every copy of the loop 115 cycles, 1299 us; a loop of the whole warp with
-            // one lane issuing 145, 1476; sixteen-byte list entries with address and destination 68, 1191; eight at a
-            // time 64, 1173.)
+            // the list of the rows to stage (the pass before has read its own)
             bool bad = false;
             if (in_pass && newrows > 0) {
                 // the new rows are the last `newrows` of {y0, y0 + 1}
@@ -587,12 +560,40 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                     if (newrows == 2) s_src[slot_new + 1] = y_new + 1u;
                 }
             }
-            __syncwarp();
+            // ---- ring slot b: wait until the consumers have finished the pass that used it ----
+            if (k >= kCropStages) {
+                const uint32_t par = (ephase >> b) & 1u;
+                if (!mbar_wait_sleeping(&empty[b], par, kCropProducerSleepNs) &&
+                    !mbar_wait_sleeping(&empty[b], par, kCropProducerSleepNs)) {
+                    atomicOr(status, 0x4u);
+                    break;
+                }
+                ephase ^= 1u << b;
+            }
+            if (lane == 0) s_pass[b] = p;
+            if (!w_valid) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[b]);  // the end-of-work record
+                break;
+            }
+            if (in_pass) s_row[b][lane] = ri;
+            fence_proxy_async();
+            __syncwarp();  // list, table, pass record and row data are written before the barrier is armed
+            // One bulk copy per row, issued by one elected lane from the list, four at a time and without a condition
+            // among the four; the next four numbers are read while these go out.  (Copies that every lane issues for
+            // itself go out one lane after the other, 97 cycles each beside the consumers; so they take 66.  With a condition on
+            // every copy of the loop 115 cycles; a loop of the whole warp with one lane issuing 145.  Launches of 24 640
+            // crops of 128x128 from 150 to 250 pixels: 899 us lane by lane, 857 so; of 1600 from rectangles 1360 wide, whose
+            // passes have seven rows, 232 lane by lane, 237 with the list written after the wait and a condition on
+            // each of the last copies, 234 so.  Passes of at most 16 rows lane by lane: up to 5 % slower.)
 #ifdef OCTO_BOUNDS_CHECK
             if (__any_sync(0xffffffffu, bad)) {  // keep the barrier's byte count right without touching memory
-                if (lane == 0)
+                if (lane == 0) {
+                    mbar_expect_tx(&full[b], (uint32_t)(staged * w_seg));
                     asm volatile("mbarrier.complete_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full[b])),
                                  "r"((uint32_t)(staged * w_seg)) : "memory");
+                }
+                __syncwarp();
                 advance(nr);
                 continue;
             }
@@ -604,6 +605,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                 const uint32_t list_end = list + (uint32_t)kCropListBytes - 16u;
                 auto row = [&](uint32_t y) { return base + (uint64_t)y * (uint32_t)w_pitch; };  // (a frame may span more than 4 GiB)
                 uint4 at = lds128(list);
+                mbar_expect_tx(&full[b], (uint32_t)staged * seg);
                 int left = staged;
                 for (; left >= 4; left -= 4, dst += 4u * stride) {
                     list = min(list + 16u, list_end);  // (read ahead, but not past the end)
@@ -614,9 +616,16 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
                     bulk_g2s(dst + 3u * stride, row(at.w), seg, bar);
                     at = next;
                 }
-                if (left > 0) bulk_g2s(dst, row(at.x), seg, bar);
-                if (left > 1) bulk_g2s(dst + stride, row(at.y), seg, bar);
-                if (left > 2) bulk_g2s(dst + 2u * stride, row(at.z), seg, bar);
+                if (left == 3) {
+                    bulk_g2s(dst, row(at.x), seg, bar);
+                    bulk_g2s(dst + stride, row(at.y), seg, bar);
+                    bulk_g2s(dst + 2u * stride, row(at.z), seg, bar);
+                } else if (left == 2) {
+                    bulk_g2s(dst, row(at.x), seg, bar);
+                    bulk_g2s(dst + stride, row(at.y), seg, bar);
+                } else if (left == 1) {
+                    bulk_g2s(dst, row(at.x), seg, bar);
+                }
             }
             __syncwarp();
             advance(nr);
