@@ -57,6 +57,13 @@ def test_tall_and_wide_crops(count, batch):
     _check(count, ((16, 97), (264, 8), (40, 64)), batch)
 
 
+@pytest.mark.parametrize("count", [55, 56, 58, 59, 83, 84])
+def test_third_tiles(count):
+    """Sixteen tiles a crop for 444 CTAs (148 SMs): third tiles for none of them, for a few (drawn from the counter), for
+    an eighth and more (fixed), for nearly all; fourth tiles."""
+    _check(count, ((8, 128), (40, 127)))
+
+
 @pytest.mark.parametrize("first", [1, 5, 9, 13])
 def test_rows_of_a_pass_four_at_a_time(first):
     """Passes of few rows: the source rows are requested four at a time, the last one to three by themselves."""
