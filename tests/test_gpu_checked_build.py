@@ -175,3 +175,8 @@ def test_nms_ways_under_the_checked_build(checked, sizes_of, batch):
 def test_widest_crops_of_three_ctas(checked, batch, widths):
     from test_gpu_crop_tiles import test_widest_crops_of_three_ctas as run
     run(batch, widths)
+
+
+def test_passes_of_64_rows(checked):
+    from test_gpu_crop_tiles import test_passes_of_64_rows as run
+    run()

@@ -70,6 +70,33 @@ def test_rows_of_a_pass_four_at_a_time(first):
     _check(9, tuple((8, first + i) for i in range(4)))
 
 
+def test_passes_of_64_rows():
+    """Narrow rectangles reduced more than twofold, so many that most crops are one tile: passes of 32 output rows that
+    stage two source rows for each, and of one row less."""
+    w, h, net, count, batch = 512, 512, 256, 900, 2
+    rng = np.random.default_rng(8)
+    frames = [rng.integers(0, 256, (h, 3 * w), dtype=np.uint8) for _ in range(batch)]
+    head = np.zeros((batch, count, 6), dtype=np.float32)
+    i = np.arange(count)
+    for b in range(batch):
+        head[b, :, 0], head[b, :, 1] = 4 + 0.27 * i, 128 + (i % 7)
+        head[b, :, 2], head[b, :, 3] = 2 + i % 5, 100 + i % 156
+        head[b, :, 4], head[b, :, 5] = 1.0, 0.99 - 0.0005 * i
+    crops = ((8, 64), (16, 40), (8, 33))
+    st = octo.Stage(net_size=net, max_batch=batch, num_anchors=count, num_classes=1, head_is_logits=False, iou_thresh=1.0,
+                    max_det=count, branches=crops)
+    try:
+        ref = oracle.run_stage(frames, [(w, h)] * batch, head, net, crops, logits=False, iou_thr=1.0, max_det=count,
+                               do_letterbox=False, threads=8)
+        res = run_stage_gpu(st, frames, [(w, h)] * batch, head, max_items=[count * batch] * len(crops))
+        _check_dets(res, ref)
+        assert res.status == 0 and res.n_items[0] == (count * batch, count * batch)
+        for k in range(len(crops)):
+            assert half_absdiff(res.crops[k], ref.crops[k]) <= PIX_TOL
+    finally:
+        st.close()
+
+
 @pytest.mark.parametrize("batch,widths", [(1, (400, 408, 416, 424)), (9, (384, 392, 400, 408)), (65, (312, 320, 328, 336))])
 def test_widest_crops_of_three_ctas(batch, widths):
     """Widths around the last of which an SM holds three CTAs, where the ring buffers are shorter: rectangles of which a
