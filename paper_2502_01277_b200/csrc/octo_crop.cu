@@ -39,7 +39,7 @@ namespace octo {
 
 // Shared memory for staged source rows.  A row segment longer than half a ring buffer less 16 bytes
 // (a rectangle wider than about 5300 pixels) is split into column tiles, so two rows always
-// fit.  Two buffers form a ring between the producer warp and the consumer warps.
+// fit (see crop_longest_row).  Two buffers form a ring between the producer warp and the consumer warps.
 constexpr int kCropStages = 2;         // ring depth (row buffers)
 constexpr int kCropTables = kCropStages + 1;  // tap tables, one more than ring slots
 constexpr int kCropRowBudget = 32768;  // bytes per ring buffer (see crop_layout)
@@ -104,6 +104,34 @@ template <int CAP>
 constexpr bool crop_shortened(int out_w) { return crop_layout<CAP>(out_w).row_budget != kCropRowBudget; }
 template <int CAP>
 constexpr bool crop_three(int out_w) { return crop_ctas_fit((int)sizeof(CropShared<CAP>) + crop_layout<CAP>(out_w).bytes); }
+// Longest row segment (with its 16 bytes of slack) of a column tile of four columns, the narrowest there is, for
+// rectangles in frames of up to w x h.  The columns reach over three steps of w / out_w or, where the resized rectangle is
+// narrower than the slot, of at most 5 / 4 h / out_h (its width, a rounded number, is two or more), and over 3 / 4 of
+// the rectangle.
+constexpr int crop_longest_row(int out_w, int out_h, bool keep_aspect, int w, int h) {
+    long long span = 3ll * w / out_w;
+    if (keep_aspect) {
+        const long long fitted = 15ll * h / (4ll * out_h), most = 3ll * w / 4;
+        const long long s = fitted < most ? fitted : most;
+        if (s > span) span = s;
+    }
+    return (int)((3 * (span + 3) + 45) & ~15ll) + 16;  // (both taps at either end, both ends on 16 bytes)
+}
+// Launches that may meet a longer row than half a ring buffer holds take a form of the kernel with longer buffers: crops
+// of 8 columns from frames of more than about 14 000 pixels, crops of up to 11 rows that keep the aspect of rectangles
+// in frames of more than 8192 pixels and of 1400 for every row.  (Frames of that size reach a stage as regions only.)
+constexpr int kCropMaxSide = 16384;  // of a frame
+constexpr int kCropWideBudget = 2 * crop_longest_row(8, 1, true, kCropMaxSide, kCropMaxSide);
+constexpr bool crop_wide(int out_w, int out_h, bool keep_aspect, int w, int h) {
+    return 2 * crop_longest_row(out_w, out_h, keep_aspect, w, h) > kCropRowBudget - kCropListBytes / kCropStages;
+}
+constexpr CropLayout crop_layout_wide(int out_w) {
+    const int tables_end = kCropStages * kCropWideBudget + kCropTables * (int)sizeof(XEntry) * out_w;
+    return {kCropWideBudget, tables_end, tables_end + kCropListBytes};
+}
+static_assert(!crop_wide(8, 1, false, 8192, kCropMaxSide) && !crop_wide(16, 12, true, kCropMaxSide, kCropMaxSide) &&
+              crop_wide(8, 300, false, kCropMaxSide, kCropMaxSide), "few launches take the longer buffers");
+static_assert(crop_layout_wide(2048).bytes + (int)sizeof(CropShared<512>) + 1024 <= 227 * 1024, "which fit");
 static_assert(crop_three<1>(416) && crop_three<8>(416) && crop_three<64>(400) && crop_three<512>(328),
               "widest crops of which an SM holds three CTAs");
 static_assert(!crop_three<1>(424) && !crop_three<8>(424) && !crop_three<64>(408) && !crop_three<512>(336), "and the next");
@@ -185,7 +213,9 @@ __device__ __forceinline__ int div_small(int a, int b) {
 // The frame table comes either by value in kernel parameter space (`tab`, first-level stages:
 // no table copy on the critical path) or from device memory (`gtab`, chained stages whose
 // table an upstream stage's items define on the device).
-template <int CAP, bool QUEUE, bool GENERAL>
+//
+// WIDE = true: ring buffers for the longest rows there are (crop_wide).
+template <int CAP, bool QUEUE, bool GENERAL, bool WIDE = false>
 __global__ void __launch_bounds__(kCropKernelThreads, kCropCtasPerSm)
 crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __restrict__ gtab, int n, int max_det,
             int first_item, int max_items,
@@ -203,7 +233,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
     auto& s_first = sh.first;
 
     unsigned char* const s_rows0 = smem;
-    XEntry* const s_xtab0 = reinterpret_cast<XEntry*>(smem + kCropStages * kCropRowBudget);  // kCropTables tables of ow entries
+    XEntry* const s_xtab0 = reinterpret_cast<XEntry*>(smem + kCropStages * (WIDE ? kCropWideBudget : kCropRowBudget));  // kCropTables tables of ow entries
     uint32_t* const s_src = reinterpret_cast<uint32_t*>(smem + list_at);
     unsigned int* const status = QUEUE ? qstatus : &ctr->status;
 
@@ -329,7 +359,7 @@ crop_kernel(const __grid_constant__ FrameTable<CAP> tab, const FrameDesc* __rest
             w_seg_lo = lo;
             w_seg = hi - lo;
             w_stride = w_seg + 16;
-            w_cap_slots = div_small(row_budget, w_stride);  // >= 2
+            w_cap_slots = div_small(row_budget, w_stride);  // >= 2 (crop_longest_row)
             // Work units of a pass: (run of consecutive rows, two column pairs half a tile apart).
             // A pass is cut into as many runs as fit the consumer threads side by side (224
             // columns: 4 runs x 56 units = the 224 consumer threads).
@@ -792,14 +822,17 @@ static int crop_grid(int sm_count, int slots, int out_h) {
     return grid < 1 ? 1 : grid;  // a zero-slot window still gets its offsets and totals
 }
 
-template <int CAP>
+template <int CAP, bool WIDE = false>
 static cudaError_t launch_crop_cap(const CropArgs& a, cudaStream_t stream) {
     FrameTable<CAP> tab;  // built per call (copied into kernel parameter space by the launch)
     if (!a.d_tab)
         for (int i = 0; i < a.n; ++i) tab.f[i] = a.frames[i];
     const int grid = crop_grid(a.sm_count, a.max_items, a.out_h);
-    const CropLayout layout = crop_layout<CAP>(a.out_w);
-    auto kernel = a.general ? crop_kernel<CAP, false, true> : crop_kernel<CAP, false, false>;
+    const CropLayout layout = WIDE ? crop_layout_wide(a.out_w) : crop_layout<CAP>(a.out_w);
+    auto kernel = crop_kernel<CAP, false, true, WIDE>;
+    if constexpr (!WIDE) {
+        if (!a.general) kernel = crop_kernel<CAP, false, false>;
+    }
     return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), (size_t)layout.bytes, stream, tab, a.d_tab, a.n,
                          a.max_det, a.first_item, a.max_items, a.d_bcount, a.d_bidx, a.d_dets, a.d_offsets, a.d_n_items,
                          a.d_items, reinterpret_cast<__half*>(a.d_out), a.out_w, a.out_h, a.swap_rb, a.d_ctr,
@@ -808,7 +841,6 @@ static cudaError_t launch_crop_cap(const CropArgs& a, cudaStream_t stream) {
 }
 
 cudaError_t prepare_crop() {
-    const int smem = crop_layout<512>(2048).bytes;
     cudaError_t e;
     const void* kernels[] = {
         (const void*)crop_kernel<8, false, false>,   (const void*)crop_kernel<8, false, true>,
@@ -817,7 +849,11 @@ cudaError_t prepare_crop() {
         (const void*)crop_kernel<1, true, false>,    (const void*)crop_kernel<1, true, true>,
     };
     for (const void* k : kernels) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, crop_layout<512>(2048).bytes);
+        if (e != cudaSuccess) return e;
+    }
+    for (const void* k : {(const void*)crop_kernel<512, false, true, true>, (const void*)crop_kernel<1, true, true, true>}) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, crop_layout_wide(2048).bytes);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -827,6 +863,7 @@ cudaError_t prepare_crop() {
 // the shared-memory scan of the per-frame counts, so it follows n even when the frame table is
 // read from device memory.
 cudaError_t launch_crop(const CropArgs& a, cudaStream_t stream) {
+    if (crop_wide(a.out_w, a.out_h, a.opts.keep_aspect != 0, a.max_w, a.max_h)) return launch_crop_cap<512, true>(a, stream);
     if (a.n <= 8) return launch_crop_cap<8>(a, stream);
     if (a.n <= 64) return launch_crop_cap<64>(a, stream);
     return launch_crop_cap<512>(a, stream);
@@ -835,15 +872,22 @@ cudaError_t launch_crop(const CropArgs& a, cudaStream_t stream) {
 // Crop the records staged by a queue pop (at most bz of them) into the downstream batch.
 cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int bz, void* d_out, int out_w,
                               int out_h, int swap_rb, int sm_count, unsigned int* d_status, int* d_sched,
-                              const CropOpts* general, cudaStream_t stream) {
+                              const CropOpts* general, int max_w, int max_h, cudaStream_t stream) {
     FrameTable<1> tab;  // unused in queue mode
     memset(&tab, 0, sizeof(tab));
     const int grid = crop_grid(sm_count, bz, out_h);
-    const CropLayout layout = crop_layout<1>(out_w);
     CropOpts opts;
     memset(&opts, 0, sizeof(opts));
     if (general) opts = *general;
-    auto kernel = general ? crop_kernel<1, true, true> : crop_kernel<1, true, false>;
+    else opts.sc[0] = opts.sc[1] = opts.sc[2] = 1.0f;
+    const bool keep_aspect = opts.keep_aspect != 0;
+    bool wide = crop_wide(out_w, out_h, keep_aspect, kCropMaxSide, kCropMaxSide);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    // (a captured pop may meet the frames of later pushes)
+    if (wide && cudaStreamIsCapturing(stream, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone)
+        wide = crop_wide(out_w, out_h, keep_aspect, max_w, max_h);
+    const CropLayout layout = wide ? crop_layout_wide(out_w) : crop_layout<1>(out_w);
+    auto kernel = wide ? crop_kernel<1, true, true, true> : general ? crop_kernel<1, true, true> : crop_kernel<1, true, false>;
     return launch_kernel(kernel, dim3(grid), dim3(kCropKernelThreads), (size_t)layout.bytes, stream, tab,
                          (const FrameDesc*)nullptr, 0, 0, 0, bz, (const int*)nullptr, (const int*)nullptr,
                          (const octo_det_t*)nullptr, (int*)nullptr, (int*)nullptr, (octo_item_t*)nullptr,

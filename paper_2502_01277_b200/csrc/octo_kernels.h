@@ -76,6 +76,7 @@ struct CropArgs {
     const FrameDesc* frames;  // host
     const FrameDesc* d_tab;   // device-resident frame table of a chained stage, or null
     int n;
+    int max_w, max_h;  // largest frame
     int max_det, first_item, max_items;
     const int* d_bcount;  // this branch's [max_batch]
     const int* d_bidx;    // this branch's [max_batch][max_det], or null: item j of a frame is its detection j
@@ -112,7 +113,7 @@ cudaError_t launch_nms(const NmsArgs& a, cudaStream_t stream);
 cudaError_t launch_crop(const CropArgs& a, cudaStream_t stream);  // batch assembler + crop-resize
 cudaError_t launch_crop_queue(const QRecord* d_staged, const int* d_qpacked, int bz, void* d_out, int out_w,
                               int out_h, int swap_rb, int sm_count, unsigned int* d_status, int* d_sched,
-                              const CropOpts* general, cudaStream_t stream);
+                              const CropOpts* general, int max_w, int max_h, cudaStream_t stream);
 
 constexpr int kLetterboxMaxWidth = 8192;  // widest frame the row staging supports
 

@@ -144,6 +144,7 @@ struct octo_queue {
     int* d_qpacked;
     bool general;   // crop options set (octo_queue_set_options)
     CropOpts opts;
+    int max_w, max_h;  // largest frame of any push
 };
 
 static void queue_free(octo_queue* q) {
@@ -209,6 +210,8 @@ extern "C" int octo_queue_push(octo_queue_t* q, octo_stage_t* st, int32_t branch
     if (!st->have_dets) return OCTO_E_NO_POSTPROCESS;
     if (cudaSetDevice(q->device) != cudaSuccess) return OCTO_E_CUDA;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+    if (st->max_w > q->max_w) q->max_w = st->max_w;
+    if (st->max_h > q->max_h) q->max_h = st->max_h;
     cudaError_t e;
     if (st->n_frames <= 8) e = push_cap<8>(st, branch, q->d_ring, q->capacity, q->d_state, stream);
     else if (st->n_frames <= 64) e = push_cap<64>(st, branch, q->d_ring, q->capacity, q->d_state, stream);
@@ -233,7 +236,8 @@ extern "C" int octo_queue_pop_due(octo_queue_t* q, int32_t bz, int32_t max_wait,
     cudaError_t e = launch_kernel(queue_pop_kernel, dim3(1), dim3(256), 0, stream, q->d_ring, q->capacity, q->d_state,
                                   bz, max_wait, q->d_staged, reinterpret_cast<QRecord*>(d_items_out), d_info, q->d_qpacked);
     if (e != cudaSuccess) return OCTO_E_CUDA;
-    e = launch_crop_queue(q->d_staged, q->d_qpacked, bz, d_out_f16, q->out_w, q->out_h, q->swap_rb,
-                                      q->sm_count, &q->d_state->status, q->d_state->sched, q->general ? &q->opts : nullptr, stream);
+    e = launch_crop_queue(q->d_staged, q->d_qpacked, bz, d_out_f16, q->out_w, q->out_h, q->swap_rb, q->sm_count,
+                          &q->d_state->status, q->d_state->sched, q->general ? &q->opts : nullptr,
+                          q->max_w, q->max_h, stream);
     return e == cudaSuccess ? OCTO_OK : OCTO_E_CUDA;
 }

@@ -233,7 +233,7 @@ extern "C" int octo_preprocess_batch(octo_stage_t* st, const octo_frame_t* frame
     if (!st || !frames || !d_out_f16_nchw || n < 1) return OCTO_E_INVALID_ARG;
     if (n > st->cfg.max_batch) return OCTO_E_CAPACITY;
     if (reinterpret_cast<uintptr_t>(d_out_f16_nchw) & 15) return OCTO_E_ALIGNMENT;
-    int max_w = 0;
+    int max_w = 0, max_h = 0;
     for (int i = 0; i < n; ++i) {
         const octo_frame_t& f = frames[i];
         if (!f.d_data || f.width < 1 || f.height < 1) return OCTO_E_INVALID_ARG;
@@ -242,6 +242,7 @@ extern "C" int octo_preprocess_batch(octo_stage_t* st, const octo_frame_t* frame
         if ((long long)f.pitch_bytes < 3LL * f.width) return OCTO_E_INVALID_ARG;
         if ((reinterpret_cast<uintptr_t>(f.d_data) & 15) || (f.pitch_bytes & 15)) return OCTO_E_ALIGNMENT;
         if (f.width > max_w) max_w = f.width;
+        if (f.height > max_h) max_h = f.height;
     }
     st->n_frames = 0;
     st->have_dets = false;
@@ -255,6 +256,7 @@ extern "C" int octo_preprocess_batch(octo_stage_t* st, const octo_frame_t* frame
         letterbox_geometry(fd.w, fd.h, st->cfg.net_size, &fd);
     }
     st->max_w = max_w;
+    st->max_h = max_h;
     OCTO_CUDA(cudaSetDevice(st->cfg.device));
     {
         ScopedKernelTimer t(st, OCTO_K_LETTERBOX, static_cast<cudaStream_t>(cuda_stream));
@@ -272,6 +274,7 @@ extern "C" int octo_adopt_regions(octo_stage_t* st, const octo_region_t* regions
     if (!st || !regions || n < 1) return OCTO_E_INVALID_ARG;
     if (n > st->cfg.max_batch) return OCTO_E_CAPACITY;
     const int S = st->cfg.net_size;
+    int max_w = 0, max_h = 0;
     for (int i = 0; i < n; ++i) {
         const octo_region_t& r = regions[i];
         if (!r.d_data || r.width < 1 || r.height < 1) return OCTO_E_INVALID_ARG;
@@ -280,6 +283,8 @@ extern "C" int octo_adopt_regions(octo_stage_t* st, const octo_region_t* regions
         if ((reinterpret_cast<uintptr_t>(r.d_data) & 15) || (r.pitch_bytes & 15)) return OCTO_E_ALIGNMENT;
         if (r.rx0 < 0 || r.ry0 < 0 || r.rx1 <= r.rx0 || r.ry1 <= r.ry0 || r.rx1 > r.width || r.ry1 > r.height)
             return OCTO_E_INVALID_ARG;
+        if (r.width > max_w) max_w = r.width;
+        if (r.height > max_h) max_h = r.height;
     }
     st->n_frames = 0;
     st->have_dets = false;
@@ -302,7 +307,8 @@ extern "C" int octo_adopt_regions(octo_stage_t* st, const octo_region_t* regions
         fd.gx = (float)(r.rx1 - r.rx0) / (float)S;
         fd.gy = (float)(r.ry1 - r.ry0) / (float)S;
     }
-    st->max_w = 0;
+    st->max_w = max_w;
+    st->max_h = max_h;
     st->n_frames = n;
     return OCTO_OK;
 }
@@ -394,7 +400,8 @@ extern "C" int octo_adopt_items_device(octo_stage_t* st, const octo_stage_t* ups
     if (e != cudaSuccess) return cuda_fail(e, "adopt_items_kernel");
     st->launches += 1;
     st->tab_on_device = true;
-    st->max_w = 0;
+    st->max_w = upstream->max_w;
+    st->max_h = upstream->max_h;
     st->n_frames = n;
     return OCTO_OK;
 }
@@ -523,6 +530,8 @@ extern "C" int octo_crop_batch(octo_stage_t* st, int32_t branch, int32_t first_i
     a.frames = st->frames;
     a.d_tab = st->tab_on_device ? st->d_tab : nullptr;
     a.n = st->n_frames;
+    a.max_w = st->max_w;
+    a.max_h = st->max_h;
     a.max_det = c.max_det;
     a.first_item = first_item;
     a.max_items = max_items;

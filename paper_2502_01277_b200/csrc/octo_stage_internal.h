@@ -26,7 +26,7 @@ struct octo_stage {
     octo::FrameDesc frames[OCTO_MAX_BATCH];
     int n_frames;
     bool tab_on_device;  // the current batch's table is d_tab (octo_adopt_items_device), not `frames`
-    int max_w;
+    int max_w, max_h;  // largest frame of the batch
     bool have_dets;
     const octo_det_t* d_dets;
     const int32_t* d_last_n_items[OCTO_MAX_BRANCHES];  // {packed, total} of the last crop call per branch (caller's buffer)

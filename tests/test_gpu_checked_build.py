@@ -180,3 +180,9 @@ def test_widest_crops_of_three_ctas(checked, batch, widths):
 def test_passes_of_64_rows(checked):
     from test_gpu_crop_tiles import test_passes_of_64_rows as run
     run()
+
+
+@pytest.mark.parametrize("keep_aspect,oh", [(False, 3), (True, 2)])
+def test_few_columns_of_a_16384_pixel_frame(checked, keep_aspect, oh):
+    from test_gpu_crop_tiles import test_few_columns_of_a_16384_pixel_frame as run
+    run(keep_aspect, oh)

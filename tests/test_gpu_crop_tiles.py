@@ -149,3 +149,39 @@ def test_widest_queued_crops_of_three_ctas(width):
     finally:
         q.close()
         st.close()
+
+
+@pytest.mark.parametrize("keep_aspect,oh", [(False, 3), (True, 2)])
+def test_few_columns_of_a_16384_pixel_frame(keep_aspect, oh):
+    """Four columns of a crop 8 pixels wide reach over 6144 pixels of such a frame, three of the seven that a rectangle of
+    16384x4681 keeps in 8x2 over 7022: two of their rows need longer ring buffers.  Crops of a stage whose regions the
+    host gives, and of a queue."""
+    w, h, net = 16384, 4681, 64
+    dev = torch.randint(0, 256, (h, 3 * w), dtype=torch.uint8, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5))
+    frame = dev.cpu().numpy()
+    rects = [(0, 16384), (0, 16000), (700, 16384), (4, 14600), (3000, 9000), (8000, 8100)]
+    head = np.zeros((1, len(rects), 6), dtype=np.float32)
+    for i, (lo, hi) in enumerate(rects):
+        head[0, i] = (lo + hi) / 2 * net / w, net / 2, (hi - lo) * net / w, net, 1.0, 0.9 - 0.02 * i
+    options = dict(keep_aspect=keep_aspect)
+    whole = np.zeros(1, dtype=octo.ITEM_DTYPE)
+    whole["rx1"], whole["ry1"] = w, h
+    st = octo.Stage(net_size=net, max_batch=1, num_anchors=len(rects), num_classes=1, head_is_logits=False, iou_thresh=1.0,
+                    branches=((8, oh), (16, oh)), crop_options=[options] * 2)
+    q = octo.Queue(64, 8, oh, max_bz=8)
+    try:
+        q.set_options(**options)
+        st.adopt_regions([dev], [(w, h)], whole)
+        dets, counts = st.postprocess(torch.from_numpy(head).cuda())
+        got = [st.crop(b, len(rects))[0] for b in range(2)]
+        q.push(st, 0)
+        got.append(q.pop(8)[0])
+        d, c = octo.dets_to_numpy(dets, counts)
+        assert c[0] == len(rects) and st.status() == 0
+        for buf, ow in zip(got, (8, 16, 8)):
+            crops = buf.view(torch.int16).cpu().numpy().view(np.uint16)
+            for i in range(len(rects)):
+                assert half_absdiff(crops[i], oracle.crop(frame, w, h, d[0, i:i + 1], ow, oh, **options)) <= PIX_TOL
+    finally:
+        q.close()
+        st.close()
