@@ -107,7 +107,7 @@ cudaError_t prepare_nms(int* clusters = nullptr);
 cudaError_t prepare_crop();
 
 cudaError_t launch_letterbox(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                             int swap_rb, unsigned int* d_status, cudaStream_t stream);
+                             int swap_rb, int sm_count, unsigned int* d_status, cudaStream_t stream);
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t stream);
 cudaError_t launch_nms(const NmsArgs& a, cudaStream_t stream);
 cudaError_t launch_crop(const CropArgs& a, cudaStream_t stream);  // batch assembler + crop-resize

@@ -21,9 +21,9 @@ static_assert(kLbRows <= kLbThreads / 32, "a warp for every row of a CTA");
 // A warp stages its own output row, behind a barrier of its own, and waits for nothing else but the table of taps;
 // where a CTA has fewer rows than warps (small batches), several warps share a row.  What needs no memory (barriers,
 // which rows are tapped) comes before the wait for the previous kernel.  Large batches are bound by HBM, small
-// ones by this chain: against one thread that walked the rows twice and issued every copy, and one barrier for all
-// of them, a pass over one small frame went from 18.1 to 17.1 us, one camera 24.2 / 23.5, eight 55.7 / 53.6, thirteen
-// 1277x717 frames 36.6 / 34.9, 32 frames 220 / 219, 256 frames unchanged.
+// ones by this chain.  One thread that walked the rows twice and issued every copy, and one barrier for all of them /
+// a barrier and copies per warp / rows shared by warps too (us a launch over 1080p frames from memory): one 4.3 / 4.1 / 3.5, two 5.3 /
+// 4.8 / 4.2, eight 11.5 / 9.4 / 9.2, 64 50.7 / - / 49.1.
 template <int CAP>
 __global__ void __launch_bounds__(kLbThreads)
 letterbox_kernel(const __grid_constant__ FrameTable<CAP> tab, __half* __restrict__ out, int S, int band_rows,
@@ -137,22 +137,42 @@ static size_t lb_smem_bytes(int S, int slots, int slot_bytes) {
     return (((size_t)S * sizeof(XEntry) + 127) & ~(size_t)127) + (size_t)slots * slot_bytes;
 }
 
+// Output rows of a CTA, when `fit` of them fit.  They are halved (7 and 6 to 3, 5 and 3 to 2) until there are eight
+// CTAs per SM of more than four rows, two and a half of four, four of three (which two of the eight warps have no row
+// of); single rows only where two do not fit.
+// us a launch over frames that come from memory / lie in L2, by the rows of a CTA (* taken):
+//   640x480    @ 640,  3 frames: 4 rows* 5.2 / 4.9, 2 rows 5.4 / 5.3
+//   1080x1920  @ 640,  3 frames: 4 rows* 5.2 / 4.7, 2 rows 5.8 / 5.5;  8 frames: 8 rows 9.2 / 9.3, 4 rows* 9.6 / 9.3
+//   1920x1080  @ 640,  1 frame:  4 rows 3.6 / 2.8, 2 rows* 3.4 / 2.9;  3 frames: 4 rows* 5.1 / 4.1, 2 rows 4.9 / 4.7
+//   1920x1080  @ 640, 12 frames: 8 rows 13.3 / 12.7, 4 rows* 12.0 / 11.9;  32 frames: 8 rows* 27.3 / 26.1
+//   1280x720   @ 640,  2 frames: 3 rows 4.8 / 4.0, 2 rows* 4.5 / 4.2, 1 row 5.1 / 5.2
+//   1280x720   @ 640,  4 frames: 6 rows 7.0 / 5.5, 4 rows 6.4 / 5.6, 3 rows* 6.1 / 5.6, 2 rows 5.9 / 6.0
+//   1280x720   @ 640,  8 frames: 6 rows 11.4 / 11.4, 4 rows 10.4 / 10.0, 3 rows* 9.6 / 9.6, 2 rows 10.4 / 10.2
+//   1277x717   @ 416,  4 frames: 7 rows 6.2 / 5.3, 3 rows 5.8 / 4.7, 2 rows* 4.8 / 4.3, 1 row 5.7 / 5.3
+//   2560x1440  @ 640,  2 frames: 3 rows 5.7 / 3.8, 2 rows* 5.2 / 4.5, 1 row 5.2 / 5.0
+constexpr int letterbox_rows(int fit, int n, int S, int sm_count) {
+    int rows = fit < kLbRows ? fit : kLbRows;
+    while (rows > 2 && 2ll * n * ((S + rows - 1) / rows) < (rows > 4 ? 16ll : rows == 4 ? 5ll : 8ll) * sm_count)
+        rows = rows > 4 ? rows / 2 : 2;
+    return rows;
+}
+static_assert(letterbox_rows(8, 1, 640, 148) == 2 && letterbox_rows(8, 3, 640, 148) == 4 && letterbox_rows(8, 15, 640, 148) == 8 &&
+              letterbox_rows(6, 2, 640, 148) == 2 && letterbox_rows(6, 3, 640, 148) == 3 && letterbox_rows(7, 4, 416, 148) == 2 &&
+              letterbox_rows(3, 1, 640, 148) == 2 && letterbox_rows(3, 3, 640, 148) == 3 && letterbox_rows(5, 1, 640, 148) == 2 &&
+              letterbox_rows(2, 1, 640, 148) == 2 && letterbox_rows(1, 9, 640, 148) == 1, "rows as stated");
+
 template <int CAP>
 static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                              int swap_rb, unsigned int* d_status, cudaStream_t stream) {
+                              int swap_rb, int sm_count, unsigned int* d_status, cudaStream_t stream) {
     FrameTable<CAP> tab;  // built per call (copied into kernel parameter space by the launch)
     for (int i = 0; i < n; ++i) tab.f[i] = frames[i];
     const int slot_bytes = ((3 * max_w + 15) & ~15) + 16;  // 16 bytes of slack: a tap reads 12 bytes from its word
-    // rows per CTA: as many as fit about 56 KB of shared memory (four CTAs per SM), at most
-    // kLbRows, at least one (a single row of the widest supported frame still fits)
+    // as many rows as fit about 56 KB of shared memory (four CTAs per SM), at least one (a single row of the widest
+    // supported frame still fits)
     const int per_row = slots_per_row(frames, n) * slot_bytes;
     const long long room = 56 * 1024 - (long long)lb_smem_bytes(S, 0, slot_bytes);
-    int band_rows = (int)(room / per_row);
-    band_rows = band_rows < 1 ? 1 : (band_rows > kLbRows ? kLbRows : band_rows);
-    // small batches: fewer rows per CTA, whose warps share them, until there are four (of eight rows: eight) CTAs per
-    // SM.  Four 720p frames 46.3 -> 45.5 us a pass against two CTAs per SM (two rows each 47.5), eight 1080p 53.7 ->
-    // 53.1, thirteen 1277x717 34.7 -> 33.7; single rows are no faster (one camera) or slower (two, 32.8 -> 33.5)
-    while (band_rows > 2 && (long long)n * ((S + band_rows - 1) / band_rows) < (band_rows > 4 ? 1184 : 592)) band_rows >>= 1;
+    const int fit = (int)(room / per_row);
+    const int band_rows = letterbox_rows(fit < 1 ? 1 : fit, n, S, sm_count);
     int share = 0;  // 2^share warps to a row
     while ((band_rows << (share + 1)) <= kLbThreads / 32) ++share;
     const size_t smem = lb_smem_bytes(S, band_rows * slots_per_row(frames, n), slot_bytes);
@@ -178,10 +198,10 @@ cudaError_t prepare_letterbox() {
 }
 
 cudaError_t launch_letterbox(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
-                             int swap_rb, unsigned int* d_status, cudaStream_t stream) {
-    if (n <= 8) return launch_cap<8>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, stream);
-    if (n <= 64) return launch_cap<64>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, stream);
-    return launch_cap<512>(frames, n, d_out, S, max_w, pad_value, swap_rb, d_status, stream);
+                             int swap_rb, int sm_count, unsigned int* d_status, cudaStream_t stream) {
+    if (n <= 8) return launch_cap<8>(frames, n, d_out, S, max_w, pad_value, swap_rb, sm_count, d_status, stream);
+    if (n <= 64) return launch_cap<64>(frames, n, d_out, S, max_w, pad_value, swap_rb, sm_count, d_status, stream);
+    return launch_cap<512>(frames, n, d_out, S, max_w, pad_value, swap_rb, sm_count, d_status, stream);
 }
 
 }  // namespace octo

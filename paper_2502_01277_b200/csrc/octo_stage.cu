@@ -261,7 +261,7 @@ extern "C" int octo_preprocess_batch(octo_stage_t* st, const octo_frame_t* frame
     {
         ScopedKernelTimer t(st, OCTO_K_LETTERBOX, static_cast<cudaStream_t>(cuda_stream));
         OCTO_CUDA(launch_letterbox(st->frames, n, d_out_f16_nchw, st->cfg.net_size, max_w, st->cfg.pad_value,
-                                   st->cfg.swap_rb, &st->d_ctr->status,
+                                   st->cfg.swap_rb, st->sm_count, &st->d_ctr->status,
                                    static_cast<cudaStream_t>(cuda_stream)));
     }
     st->launches += 1;
