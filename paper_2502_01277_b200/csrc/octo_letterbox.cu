@@ -138,9 +138,13 @@ static size_t lb_smem_bytes(int S, int slots, int slot_bytes) {
 }
 
 // Output rows of a CTA, when `fit` of them fit.  They are halved (7 and 6 to 3, 5 and 3 to 2) until there are eight
-// CTAs per SM of more than four rows, two and a half of four, four of three (which two of the eight warps have no row
-// of); single rows only where two do not fit.
+// CTAs per SM of more than four rows (five where the table of taps is longer than the source rows of an output row, so that
+// it wants to be shared), two and a half of four, four of three (which two of the eight warps have no row of); single
+// rows only where two do not fit.
 // us a launch over frames that come from memory / lie in L2, by the rows of a CTA (* taken):
+//   320x240    @ 640, 12 frames: 8 rows* 12.2 / 12.0, 4 rows 12.9 / 13.1
+//   640x480    @ 640, 12 frames: 8 rows* 10.6 / 10.2, 4 rows 11.5 / 11.4;  8 frames: 8 rows 8.0 / 8.1, 4 rows* 8.5 / 8.6
+//   800x600    @ 640, 12 frames: 8 rows* 13.6 / 13.7, 4 rows 13.8 / 13.6;  8 frames: 8 rows 10.6 / 10.6, 4 rows* 9.9 / 9.9
 //   640x480    @ 640,  3 frames: 4 rows* 5.2 / 4.9, 2 rows 5.4 / 5.3
 //   1080x1920  @ 640,  3 frames: 4 rows* 5.2 / 4.7, 2 rows 5.8 / 5.5;  8 frames: 8 rows 9.2 / 9.3, 4 rows* 9.6 / 9.3
 //   1920x1080  @ 640,  1 frame:  4 rows 3.6 / 2.8, 2 rows* 3.4 / 2.9;  3 frames: 4 rows* 5.1 / 4.1, 2 rows 4.9 / 4.7
@@ -150,16 +154,19 @@ static size_t lb_smem_bytes(int S, int slots, int slot_bytes) {
 //   1280x720   @ 640,  8 frames: 6 rows 11.4 / 11.4, 4 rows 10.4 / 10.0, 3 rows* 9.6 / 9.6, 2 rows 10.4 / 10.2
 //   1277x717   @ 416,  4 frames: 7 rows 6.2 / 5.3, 3 rows 5.8 / 4.7, 2 rows* 4.8 / 4.3, 1 row 5.7 / 5.3
 //   2560x1440  @ 640,  2 frames: 3 rows 5.7 / 3.8, 2 rows* 5.2 / 4.5, 1 row 5.2 / 5.0
-constexpr int letterbox_rows(int fit, int n, int S, int sm_count) {
+constexpr int letterbox_rows(int fit, int n, int S, bool long_table, int sm_count) {
     int rows = fit < kLbRows ? fit : kLbRows;
-    while (rows > 2 && 2ll * n * ((S + rows - 1) / rows) < (rows > 4 ? 16ll : rows == 4 ? 5ll : 8ll) * sm_count)
+    while (rows > 2 && 2ll * n * ((S + rows - 1) / rows) < (rows > 4 ? long_table ? 10ll : 16ll : rows == 4 ? 5ll : 8ll) * sm_count)
         rows = rows > 4 ? rows / 2 : 2;
     return rows;
 }
-static_assert(letterbox_rows(8, 1, 640, 148) == 2 && letterbox_rows(8, 3, 640, 148) == 4 && letterbox_rows(8, 15, 640, 148) == 8 &&
-              letterbox_rows(6, 2, 640, 148) == 2 && letterbox_rows(6, 3, 640, 148) == 3 && letterbox_rows(7, 4, 416, 148) == 2 &&
-              letterbox_rows(3, 1, 640, 148) == 2 && letterbox_rows(3, 3, 640, 148) == 3 && letterbox_rows(5, 1, 640, 148) == 2 &&
-              letterbox_rows(2, 1, 640, 148) == 2 && letterbox_rows(1, 9, 640, 148) == 1, "rows as stated");
+static_assert(letterbox_rows(8, 1, 640, false, 148) == 2 && letterbox_rows(8, 3, 640, false, 148) == 4 &&
+              letterbox_rows(8, 14, 640, false, 148) == 4 && letterbox_rows(8, 15, 640, false, 148) == 8 &&
+              letterbox_rows(8, 9, 640, true, 148) == 4 && letterbox_rows(8, 10, 640, true, 148) == 8 &&
+              letterbox_rows(6, 2, 640, false, 148) == 2 && letterbox_rows(6, 3, 640, false, 148) == 3 &&
+              letterbox_rows(7, 4, 416, false, 148) == 2 && letterbox_rows(5, 1, 640, false, 148) == 2 &&
+              letterbox_rows(3, 1, 640, false, 148) == 2 && letterbox_rows(3, 3, 640, false, 148) == 3 &&
+              letterbox_rows(2, 1, 640, false, 148) == 2 && letterbox_rows(1, 9, 640, false, 148) == 1, "rows as stated");
 
 template <int CAP>
 static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S, int max_w, int pad_value,
@@ -172,7 +179,7 @@ static cudaError_t launch_cap(const FrameDesc* frames, int n, void* d_out, int S
     const int per_row = slots_per_row(frames, n) * slot_bytes;
     const long long room = 56 * 1024 - (long long)lb_smem_bytes(S, 0, slot_bytes);
     const int fit = (int)(room / per_row);
-    const int band_rows = letterbox_rows(fit < 1 ? 1 : fit, n, S, sm_count);
+    const int band_rows = letterbox_rows(fit < 1 ? 1 : fit, n, S, S * (int)sizeof(XEntry) >= per_row, sm_count);
     int share = 0;  // 2^share warps to a row
     while ((band_rows << (share + 1)) <= kLbThreads / 32) ++share;
     const size_t smem = lb_smem_bytes(S, band_rows * slots_per_row(frames, n), slot_bytes);

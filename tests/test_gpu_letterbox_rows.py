@@ -14,15 +14,15 @@ pytestmark = pytest.mark.gpu
 S = 104
 
 # (width, height, rows that fit, batches on both sides of the steps of the rule on 148 SMs, rows of a CTA there)
-CASES = [(100, 37, 8, {1: 2, 14: 2, 15: 4, 91: 4, 92: 8}), (104, 104, 8, {1: 2, 15: 4, 92: 8}),
+CASES = [(100, 37, 8, {1: 2, 14: 2, 15: 4, 56: 4, 57: 8}), (400, 90, 8, {15: 4, 91: 4, 92: 8}), (104, 104, 8, {1: 2, 15: 4, 57: 8}),
          (1300, 77, 7, {1: 2, 16: 2, 17: 3, 78: 3, 79: 7}), (1500, 100, 6, {1: 2, 16: 2, 17: 3, 65: 3, 66: 6}),
          (1800, 64, 5, {56: 2, 57: 5}), (2200, 90, 4, {14: 2, 15: 4}), (3000, 40, 3, {1: 2, 16: 2, 17: 3}),
          (4600, 20, 2, {1: 2, 30: 2}), (8192, 24, 1, {1: 1, 30: 1})]
 
 
-def _rows(fit, n, sms=148):
+def _rows(fit, n, long_table, sms=148):
     rows = min(fit, 8)
-    while rows > 2 and 2 * n * -(-S // rows) < (16 if rows > 4 else 5 if rows == 4 else 8) * sms:
+    while rows > 2 and 2 * n * -(-S // rows) < ((10 if long_table else 16) if rows > 4 else 5 if rows == 4 else 8) * sms:
         rows = rows // 2 if rows > 4 else 2
     return rows
 
@@ -34,7 +34,7 @@ def test_cases_reach_every_number_of_rows():
         row = (3 * w + 15) // 16 * 16 + 16
         assert min(8, (56 * 1024 - 896) // (slots * row)) == fit
         for n, rows in batches.items():
-            assert _rows(fit, n) == rows
+            assert _rows(fit, n, 8 * S >= slots * row) == rows
             reached.add(rows)
     assert reached == set(range(1, 9))
 
