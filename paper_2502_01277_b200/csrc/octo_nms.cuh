@@ -348,7 +348,7 @@ struct BatchMem {
     static constexpr size_t kBytes = (size_t)B * (8 + 8 + 16 + 4 + 4 * kBatchRows + 4 + 2);
 };
 
-// Greedy NMS of m (<= NT) candidates of whole classes, none of more than 512: thread c < m brings candidate
+// Greedy NMS of m (<= B) candidates of whole classes, none of more than 512, by so many warps: thread c < m brings candidate
 // c (key, box); on return mem.skey / mem.sbox hold them ordered by class and score and fate[w].x says which
 // of them survive, as one bit each: bit l of word w is candidate batch_cand(32 w + l).  class_start: where a
 // class begins.  bucketed: thread c's candidate lies in a bucket of mem.skey (which has a pad), buckets in
@@ -356,8 +356,8 @@ struct BatchMem {
 // inside it; else from words of 32 and binary search.  All threads of the CTA, after a barrier.
 __device__ __forceinline__ int batch_cand(int tid) { return (tid & ~31) | ((tid & 7) << 2) | ((tid >> 3) & 3); }
 
-template <int NT, typename Start, typename Range>
-__device__ __forceinline__ void nms_batch(const BatchMem<NT>& mem, unsigned long long key, const float4 box, int m,
+template <int B, typename Start, typename Range>
+__device__ __forceinline__ void nms_batch(const BatchMem<B>& mem, int warps, unsigned long long key, const float4 box, int m,
                                           bool bucketed, const IouTest& test, uint2* fate, unsigned int* status,
                                           Start class_start, Range range) {
     (void)status;
@@ -366,7 +366,7 @@ __device__ __forceinline__ void nms_batch(const BatchMem<NT>& mem, unsigned long
     // the lanes of a warp read the same shared-memory words as they walk.  Part 0 of candidate c is thread
     // c, which holds its key and box in registers.
     const int words = (m + 31) >> 5;
-    const int parts = 4 * words <= NT / 32 ? 4 : 2 * words <= NT / 32 ? 2 : 1;
+    const int parts = 4 * words <= warps ? 4 : 2 * words <= warps ? 2 : 1;
     const int word = warp % max(words, 1), part = warp / max(words, 1);  // part >= parts: nothing to do
     const int c = word * 32 + lane;
     const bool busy = part < parts && c < m;
@@ -446,7 +446,7 @@ __device__ __forceinline__ void nms_batch(const BatchMem<NT>& mem, unsigned long
                         if (iou_above(mem.sbox[j], b, test)) bits |= 1u << ((j >> 2) - 8 * w0);
                 }
                 to[p] = (unsigned char)bits;
-                for (int w = 1; w <= rows && room; ++w) to[4 * NT * w + p] = (unsigned char)(bits >> (8 * w));
+                for (int w = 1; w <= rows && room; ++w) to[4 * B * w + p] = (unsigned char)(bits >> (8 * w));
             }
         } else if (room) {
             // a byte is tested whole (the lanes read the same boxes) and what is not an earlier candidate of
@@ -465,14 +465,14 @@ __device__ __forceinline__ void nms_batch(const BatchMem<NT>& mem, unsigned long
                         for (int t = lo; t < hi; ++t)
                             if (iou_above(mem.sbox[base + 4 * t], b, test)) bits |= 1u << t;
                     }
-                    to[4 * NT * (w - w0) + p] = (unsigned char)(bits & (0xffu << lo) & (0xffu >> (8 - hi)));
+                    to[4 * B * (w - w0) + p] = (unsigned char)(bits & (0xffu << lo) & (0xffu >> (8 - hi)));
                 }
             }
         }
     }
     __syncthreads();
     const int cand = batch_cand(tid);
-    if (warp < words) resolve_words<NT>(mem.sup, cand, m, cand < m ? mem.sstart[cand] >> 5 : 0, fate, tid, words);
+    if (warp < words) resolve_words<B>(mem.sup, cand, m, cand < m ? mem.sstart[cand] >> 5 : 0, fate, tid, words);
     __syncthreads();
 }
 
@@ -598,7 +598,8 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
     __shared__ __align__(16) int s_sub[128 * kSubs];  // crowded images: keys per class and score bucket, then where it begins
     static_assert(BatchMem<NT>::kBytes + 16 + 2 * SMEM_CAP <= (size_t)SMEM_CAP * sizeof(float4),
                   "a batch and the slots of all keys fit the memory of the boxes");
-    constexpr int kShortThreads = NT < kSmallMax ? NT : kSmallMax;
+    constexpr int kShort = kSmallMax;  // candidates of the short path, and threads of its smaller form
+    static_assert(NT == kShort || NT == 2 * kShort, "a thread for every candidate of the short path");
     unsigned int* const status = &P.ctr->status;
     (void)status;  // referenced by the range checks of the checked build only
 
@@ -649,16 +650,19 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
     const float4* boxes_at = nullptr;
     bool written = false;  // the records are
     int nout;
+    int nt = NT;  // threads that go on
     if (cnt <= kSmallMax) {
-        // The first CTA alone (no cluster barrier follows on this path), and of it as many threads as there may be
-        // candidates: the barriers of the short phases are between 16 warps instead of 32 (a pass over one small frame
-        // 17.05 -> 16.65 us, one camera 24.7 -> 24.2, two into a queue 32.3 -> 31.7, four 45.2 -> 44.8).
-        if (crank != 0 || tid >= kShortThreads) return;
-        const BatchMem<kShortThreads> mem(smem_raw);
+        // The first CTA alone (no cluster barrier follows on this path).  Up to 256 candidates 512 of its threads go on:
+        // the barriers of the short phases are between 16 warps instead of 32, and a candidate still has two threads.
+        // Decode and NMS of one image with 1024 threads / with 512, us: 40 candidates 8.4 / 7.3, 128 of 7 classes 9.1 / 8.0,
+        // 256 of one class 17.2 / 16.9, 300 of one class 18.6 / 20.0, class-agnostic 20.1 / 22.2.
+        if (NT > kShort && cnt <= kShort / 2) nt = kShort;
+        if (crank != 0 || tid >= nt) return;
+        const BatchMem<kShort> mem(smem_raw);
         int pos = 0;
         if (tid < cnt) pos = atomicAdd(&seg_cnt[(int)(first_key >> 57)], 1);
         if (tid < cnt) mem.rank[tid] = 0;
-        if (tid == 0) mem.skey[cnt] = kKeySentinel;  // (a key more than fits when cnt is that of the threads: never read then)
+        if (tid == 0) mem.skey[cnt] = kKeySentinel;  // (a key more than fits when cnt is kShort: never read then)
         __syncthreads();
         if (warp == 0) {  // where each class starts, and the largest
             scan_classes(lane, seg_cnt, seg_start);
@@ -683,7 +687,7 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
                 first_box = ubox[tid];
             }
         }
-        nms_batch<kShortThreads>(mem, first_key, first_box, cnt, bucketed, P.iou_test, s_fate, status,
+        nms_batch<kShort>(mem, nt / 32, first_key, first_box, cnt, bucketed, P.iou_test, s_fate, status,
                       [&](int cls) { return seg_start[cls]; },
                       [&](unsigned long long k, int& lo, int& hi) {
                           lo = seg_start[(int)(k >> 57)];
@@ -702,11 +706,11 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
             spos[q] = (unsigned short)cand;
         }
         nout = min(m, max_det);
-        opos = spos + kShortThreads;
-        unsigned long long* const tmp = reinterpret_cast<unsigned long long*>(spos + 2 * kShortThreads);
-        ordered = tmp + kShortThreads + 2;
+        opos = spos + kShort;
+        unsigned long long* const tmp = reinterpret_cast<unsigned long long*>(spos + 2 * kShort);
+        ordered = tmp + kShort + 2;
         __syncthreads();
-        order_survivors<kShortThreads>(surv, spos, m, tmp, mem.rank, tid, [&](int r, unsigned long long g, int at) {
+        order_survivors<kShort>(surv, spos, m, tmp, mem.rank, tid, [&](int r, unsigned long long g, int at) {
             if (r >= max_det || !OCTO_IN_RANGE(r >= 0 && r < m && at < cnt, status)) return;
             ordered[r] = g;
             if (P.class_agnostic) opos[r] = (unsigned short)at;
@@ -926,7 +930,7 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
                 }
                 if (tid == 0) mem.skey[m] = kKeySentinel;  // (m = NT: the first word of the boxes, not read)
                 __syncthreads();
-                nms_batch<NT>(mem, key, box, m, bucketed, P.iou_test, s_fate, status,
+                nms_batch<NT>(mem, NT / 32, key, box, m, bucketed, P.iou_test, s_fate, status,
                               [&](int cls) { return seg_start[cls] - lo; },
                               [&](unsigned long long k, int& from, int& to) {
                                   const int cls = (int)(k >> 57), start = seg_start[cls] - lo, all = seg_cnt[cls];
@@ -1071,7 +1075,6 @@ __device__ __forceinline__ void nms_image(const NmsParams& P, const FrameDesc& f
             bitonic_range<true>(ordered, total, tid, NT);
         }
     }
-    const int nt = cnt <= kSmallMax ? kShortThreads : NT;
     if (P.class_agnostic) {
         // NMS ran with every candidate in class 0: a warp recovers the real class (first maximum)
         for (int r = warp; r < nout; r += nt / 32) {
