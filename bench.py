@@ -43,9 +43,9 @@ NCU_TRAFFIC = {
     # kernel: (source files, sha256[:16] of their code (comments and layout stripped) at capture time, bytes per unit, unit)
     # captured on the sweep workload at B = 64; decode_planes on the anchor_free workload at B = 64
     "crop": (("paper_2502_01277_b200/csrc/octo_crop.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-             "e7cf1d68ed38ac44", 490656.1, "crop"),
+             "a71e426366ec7bc6", 490296.5, "crop"),
     "letterbox": (("paper_2502_01277_b200/csrc/octo_letterbox.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-                  "e01b273567d36b8b", 3686080.0, "frame"),
+                  "c41d846e0f6f2b57", 3689820.0, "frame"),
     "decode": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
                "ad62776268f5859a", 1740604.0, "frame"),
     "decode_planes": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
@@ -53,7 +53,7 @@ NCU_TRAFFIC = {
 }
 # Warp instructions the crop kernel executes per crop (ncu smsp__inst_executed.sum of the same capture):
 # its issue rate is reported beside the byte rates (two thirds of the issue slots are used).
-NCU_CROP_WARP_INST = 84129.8
+NCU_CROP_WARP_INST = 83416.1
 
 
 def parse_args():

@@ -8,7 +8,7 @@
 // table entry of a slot is written by the CTA that processes the slot's first row band.
 //
 // Crop-resize: bound by the latency inside a unit of work at the 24 warps an SM holds with 80 registers a
-// thread (1.5 warps of a scheduler are eligible; issue slots 65 % and shared-memory wavefronts 76 % busy,
+// thread (1.6 warps of a scheduler are eligible; issue slots 67 % and shared-memory wavefronts 79 % busy,
 // DRAM 52 %).  A persistent grid works through (slot, row band) tiles (whole crops where there are many; the
 // last crops of a launch are cut finer so that the grid ends together).  A CTA's first two tiles are fixed (three where
 // that is all), the others come from an atomic counter, so no host synchronisation sits between NMS and cropping.  Inside a CTA
