@@ -118,8 +118,8 @@ constexpr int crop_longest_row(int out_w, int out_h, bool keep_aspect, int w, in
     return (int)((3 * (span + 3) + 45) & ~15ll) + 16;  // (both taps at either end, both ends on 16 bytes)
 }
 // Launches that may meet a longer row than half a ring buffer holds take a form of the kernel with longer buffers: crops
-// of 8 columns from frames of more than about 14 000 pixels, crops of up to 11 rows that keep the aspect of rectangles
-// in frames of more than 8192 pixels and of 1400 for every row.  (Frames of that size reach a stage as regions only.)
+// of 8 columns from frames more than about 14 000 pixels wide (which reach a stage as regions only), crops of up to 11
+// rows that keep their aspect from frames more than 7200 pixels wide and 1440 high for every row of the crop.
 constexpr int kCropMaxSide = 16384;  // of a frame
 constexpr int kCropWideBudget = 2 * crop_longest_row(8, 1, true, kCropMaxSide, kCropMaxSide);
 constexpr bool crop_wide(int out_w, int out_h, bool keep_aspect, int w, int h) {
