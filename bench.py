@@ -43,7 +43,7 @@ NCU_TRAFFIC = {
     # kernel: (source files, sha256[:16] of their code (comments and layout stripped) at capture time, bytes per unit, unit)
     # captured on the sweep workload at B = 64; decode_planes on the anchor_free workload at B = 64
     "crop": (("paper_2502_01277_b200/csrc/octo_crop.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
-             "a71e426366ec7bc6", 490296.5, "crop"),
+             "9669e94a75454bef", 489539.1, "crop"),
     "letterbox": (("paper_2502_01277_b200/csrc/octo_letterbox.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
                   "c41d846e0f6f2b57", 3689820.0, "frame"),
     "decode": (("paper_2502_01277_b200/csrc/octo_decode.cu", "paper_2502_01277_b200/csrc/octo_common.cuh"),
@@ -53,7 +53,7 @@ NCU_TRAFFIC = {
 }
 # Warp instructions the crop kernel executes per crop (ncu smsp__inst_executed.sum of the same capture):
 # its issue rate is reported beside the byte rates (two thirds of the issue slots are used).
-NCU_CROP_WARP_INST = 83416.1
+NCU_CROP_WARP_INST = 83415.5
 
 
 def parse_args():
